@@ -128,7 +128,7 @@ __global__ void k_update_x(SlotDev* S) {
 // of this arithmetic has the same pair constants, passed as the launch parameter `pkc` (read from the
 // constant bank, no registers); otherwise each item takes its slot's constants.
 template <typename Policy, int R, int V, int U, bool kShared>
-__global__ void __launch_bounds__(kThreads, 2) k_pairs(SlotDev* S, const int2* __restrict__ items,
+__global__ void __launch_bounds__(kThreads, Policy::kMinBlocks) k_pairs(SlotDev* S, const int2* __restrict__ items,
                                                     const int* __restrict__ n_items, int* __restrict__ counter,
                                                     int half, int prec, int pol, const float2* __restrict__ exp_tab,
                                                     int* __restrict__ err, const PairConsts pkc,

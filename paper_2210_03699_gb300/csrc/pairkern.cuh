@@ -171,8 +171,27 @@ __device__ __forceinline__ void acc_add(F2& acc, F2 x) {
     acc.hi = s.hi;
     acc.lo = __fadd_rn(acc.lo, __fadd_rn(s.lo, x.lo));
 }
-// a0 b0 + a1 b1 + a2 b2
-__device__ __forceinline__ F2 dot3(F2 a0, F2 a1, F2 a2, F2 b0, F2 b1, F2 b2) {
+// Sums and differences without the final renormalisation: exact two_sum of the high parts, plain sum of
+// the low parts.
+__device__ __forceinline__ F2 addl(F2 a, F2 b) {
+    const F2 s = two_sum(a.hi, b.hi);
+    return F2{s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo))};
+}
+__device__ __forceinline__ F2 subl(F2 a, F2 b) { return addl(a, neg(b)); }
+// 1 - a for 0 <= a <= 1 (1 - a.hi and its rounding error are exact), and for any a
+__device__ __forceinline__ F2 one_minus(F2 a) {
+    const float s = __fsub_rn(1.0f, a.hi);
+    return F2{s, __fsub_rn(__fsub_rn(__fsub_rn(1.0f, s), a.hi), a.lo)};
+}
+__device__ __forceinline__ F2 one_minus_any(F2 a) {
+    const F2 s = two_sum(1.0f, -a.hi);
+    return F2{s.hi, __fsub_rn(s.lo, a.lo)};
+}
+// acc += a b: the product's leading part by an exact two_sum, everything else into the low part
+__device__ __forceinline__ void acc_mul(F2& acc, F2 a, F2 b) { acc_add(acc, mull(a, b)); }
+// a0 b0 + a1 b1 + a2 b2, unnormalised: the low part is within a few 2^-24 of the largest product, so what a
+// later lazy product drops stays below 2^-46 of the factors' own scale even where the sum cancels
+__device__ __forceinline__ F2 dot3l(F2 a0, F2 a1, F2 a2, F2 b0, F2 b1, F2 b2) {
     const F2 p0 = two_prod(a0.hi, b0.hi), p1 = two_prod(a1.hi, b1.hi), p2 = two_prod(a2.hi, b2.hi);
     const F2 s = two_sum(p0.hi, p1.hi);
     const F2 t = two_sum(s.hi, p2.hi);
@@ -180,51 +199,43 @@ __device__ __forceinline__ F2 dot3(F2 a0, F2 a1, F2 a2, F2 b0, F2 b1, F2 b2) {
     e = __fmaf_rn(a0.hi, b0.lo, __fmaf_rn(a0.lo, b0.hi, e));
     e = __fmaf_rn(a1.hi, b1.lo, __fmaf_rn(a1.lo, b1.hi, e));
     e = __fmaf_rn(a2.hi, b2.lo, __fmaf_rn(a2.lo, b2.hi, e));
-    return fast_two_sum(t.hi, e);
+    return F2{t.hi, e};
 }
-// 1/sqrt(x): SFU seed y0 (rel. err < 2^-22), one Newton step y0 + y0 (1 - x y0^2)/2 in float-float
+// a0^2 + a1^2 + a2^2, unnormalised (the two halves of each cross product are equal)
+__device__ __forceinline__ F2 sq3l(F2 a0, F2 a1, F2 a2) {
+    const F2 p0 = two_prod(a0.hi, a0.hi), p1 = two_prod(a1.hi, a1.hi), p2 = two_prod(a2.hi, a2.hi);
+    const F2 s = two_sum(p0.hi, p1.hi);
+    const F2 t = two_sum(s.hi, p2.hi);
+    const float x = __fmaf_rn(a2.hi, a2.lo, __fmaf_rn(a1.hi, a1.lo, __fmul_rn(a0.hi, a0.lo)));
+    const float e = __fadd_rn(__fadd_rn(p0.lo, p1.lo), __fadd_rn(p2.lo, __fadd_rn(s.lo, t.lo)));
+    return F2{t.hi, __fmaf_rn(2.0f, x, e)};
+}
+// 1/sqrt(x), normalised: SFU seed y (rel. err < 2^-22), its residual e = 1 - x y^2 (1 - x.hi w is exact, the
+// rest follows in FP32), y + y e (1/2 + 3/8 e): truncation below 2^-64
 __device__ __forceinline__ F2 rsqrt_ff(F2 x) {
-    const float y0 = rsqrt_sfu(x.hi);
-    const F2 t = mul(x, two_prod(y0, y0));
-    const float e = __fsub_rn(__fsub_rn(1.0f, t.hi), t.lo);
-    return fast_two_sum(y0, __fmul_rn(__fmul_rn(0.5f, y0), e));
+    const float y = rsqrt_sfu(x.hi);
+    const F2 w = two_prod(y, y);
+    const float t = __fmul_rn(x.hi, w.hi);
+    const float l = __fmaf_rn(x.lo, w.hi, __fmaf_rn(x.hi, w.lo, __fmaf_rn(x.hi, w.hi, -t)));
+    const float e = __fsub_rn(__fsub_rn(1.0f, t), l);
+    return fast_two_sum(y, __fmul_rn(__fmul_rn(__fmul_rn(0.5f, y), e), __fmaf_rn(0.75f, e, 1.0f)));
 }
-// e^{-x}, x >= 0: x = k/1024 + f (k nearest), e^{-x} = e^{-(k>>10)} e^{-(k&1023)/1024} e^{-f},
-// e^{-f} = 1 - f + f^2 (1/2 - f/6 + f^2/24) for |f| <= 1/2048 (truncation < 3e-19)
-__device__ __forceinline__ F2 exp_neg_ff(F2 x, const float2* tab) {
-    float xh = x.hi, xl = x.lo;
-    if (xh > 63.9f) {
-        xh = 63.9f;
-        xl = 0.f;
-    }
-    const float t = __fmaf_rn(xh, 1024.f, 12582912.f);   // 1.5 * 2^23: round(x * 1024) in the mantissa
-    const int k = min(max(__float_as_int(t) - 0x4B400000, 0), kExpHi * kExpLo - 1);   // in range for any input
-    const float kf = __fsub_rn(t, 12582912.f);
-    const F2 f = two_sum(__fmaf_rn(kf, -1.0f / 1024.f, xh), xl);   // the first term is exact
-    const float fh = f.hi;
-    const float poly = __fmaf_rn(__fmaf_rn(fh, 1.0f / 24.0f, -1.0f / 6.0f), fh, 0.5f);
-    const float q = __fmul_rn(__fmul_rn(fh, fh), poly);
-    const F2 omf = fast_two_sum(1.0f, -fh);
-    const F2 ef = fast_two_sum(omf.hi, __fadd_rn(__fsub_rn(omf.lo, f.lo), q));
-    return mul(mul(f2(tab[k >> 10]), f2(tab[kExpHi + (k & 1023)])), ef);
-}
-// The same with lazy products (for the symmetric pair terms).
+// e^{-x}, x >= 0: x = k/1024 + a + x.lo (k nearest to 1024 x.hi, a exact), e^{-x} = e^{-(k>>10)} e^{-(k&1023)/1024} e^{-f},
+// e^{-f} = 1 - a - x.lo + q with q = f^2 (1/2 - f/6 + f^2/24), f = a + x.lo, |f| <= 1/2048 (truncation < 3e-19).
+// x is capped at 63.9, where e^{-x} < 2e-28: the cap keeps the table index in range for any input
+// (fminf returns the number when the other operand is a NaN).  Lazy result.
 __device__ __forceinline__ F2 exp_neg_ffl(F2 x, const float2* tab) {
-    float xh = x.hi, xl = x.lo;
-    if (xh > 63.9f) {
-        xh = 63.9f;
-        xl = 0.f;
-    }
-    const float t = __fmaf_rn(xh, 1024.f, 12582912.f);
-    const int k = min(max(__float_as_int(t) - 0x4B400000, 0), kExpHi * kExpLo - 1);
-    const float kf = __fsub_rn(t, 12582912.f);
-    const F2 f = two_sum(__fmaf_rn(kf, -1.0f / 1024.f, xh), xl);
-    const float fh = f.hi;
-    const float poly = __fmaf_rn(__fmaf_rn(fh, 1.0f / 24.0f, -1.0f / 6.0f), fh, 0.5f);
-    const float q = __fmul_rn(__fmul_rn(fh, fh), poly);
-    const F2 omf = fast_two_sum(1.0f, -fh);
-    const F2 ef = fast_two_sum(omf.hi, __fadd_rn(__fsub_rn(omf.lo, f.lo), q));
-    return mull(mull(f2(tab[k >> 10]), f2(tab[kExpHi + (k & 1023)])), ef);
+    const float xh = fminf(x.hi, 63.9f);
+    const float xl = x.hi > 63.9f ? 0.f : x.lo;
+    const float t = __fmaf_rn(xh, 1024.f, 12582912.f);   // 1.5 * 2^23: round(x * 1024) in the mantissa
+    const int k = __float_as_int(t) - 0x4B400000;
+    const float a = __fmaf_rn(__fsub_rn(t, 12582912.f), -1.0f / 1024.f, xh);
+    const float f = __fadd_rn(a, xl);
+    const float poly = __fmaf_rn(__fmaf_rn(f, 1.0f / 24.0f, -1.0f / 6.0f), f, 0.5f);
+    const float q = __fmul_rn(__fmul_rn(f, f), poly);
+    const float s = __fsub_rn(1.0f, a);
+    const float l = __fadd_rn(__fsub_rn(__fsub_rn(__fsub_rn(1.0f, s), a), xl), q);
+    return mull(mull(f2(tab[k >> 10]), f2(tab[kExpHi + (k & (kExpLo - 1))])), F2{s, l});
 }
 
 // ------------------------------------------------------------------ exact node accumulators
@@ -337,9 +348,12 @@ __device__ __forceinline__ void fx_read(unsigned long long* __restrict__ acc, in
 // and acc1 += a K11 - b K12, acc2 += a K21 - b K22.
 struct Fp32Policy {
     using Src = float4;
+    static constexpr int kMinBlocks = 2;   // resident blocks per SM the registers are limited for
     static constexpr int kVec = 2;    // Src per node
     static constexpr int kTile = 256; // nodes per tile (8 KB)
     static constexpr bool kTables = false;
+    static constexpr bool kRenorm = false;   // running sums need no renormalisation
+    static constexpr bool kStepTranspose = false;
     static constexpr int kSymStep = 32;   // symmetric chunk fully unrolled
     struct Tgt {
         float px, py, pz, qx, qy, qz, wa, wb;
@@ -412,9 +426,12 @@ struct Fp32Policy {
 //                -a2 += ((-b_t) s)(d.n_y) t2n + ((-a_t) s) X   (negated; jfinal restores the sign).
 struct Fp32x2Policy {
     using Src = ulonglong2;
+    static constexpr int kMinBlocks = 2;   // resident blocks per SM the registers are limited for
     static constexpr int kVec = 4;      // Src per node (64 B)
     static constexpr int kTile = 256;   // nodes per tile (16 KB)
     static constexpr bool kTables = false;
+    static constexpr bool kRenorm = false;   // running sums need no renormalisation
+    static constexpr bool kStepTranspose = false;
     static constexpr int kSymStep = 32;
     static constexpr int kPack = 2;
     struct Tgt {
@@ -569,9 +586,12 @@ struct Fp32x2Policy {
 
 struct Fp64Policy {
     using Src = double4;
+    static constexpr int kMinBlocks = 2;   // resident blocks per SM the registers are limited for
     static constexpr int kVec = 2;
     static constexpr int kTile = 128;   // 8 KB
     static constexpr bool kTables = false;
+    static constexpr bool kRenorm = false;   // running sums need no renormalisation
+    static constexpr bool kStepTranspose = false;
     static constexpr int kSymStep = 4;
     struct Tgt {
         double px, py, pz, qx, qy, qz, wa, wb;
@@ -673,12 +693,27 @@ struct Fp64Policy {
 };
 
 // Source node = 4 float4: {P.hi, a.hi} {P.lo, a.lo} {n.hi, b.hi} {n.lo, b.lo}.
+// Bound: the FP32 pipe (no FP64 in the pair loops).  Products and sums are lazy; renormalised are only the
+// node differences, 1/r, E and 1 - E1 (and the running sums once per step), which is what keeps every term's error at or below that of fully
+// normalised arithmetic (a pair's K11, K12, K21 against 64 bits, 2e5 pairs of an ellipsoid 0.3 to 8 apart:
+// rms 6.3e-14, 5.1e-14, 2.0e-12 of the uncancelled term; normalised throughout: 7.1e-14, 5.5e-14, 2.1e-12).
+// With u = 1 - E1, w = E kappa r, c = (d . n_x)(d . n_y)/r^2 the bracket of K21 is
+// u (n_x . n_y - 3 c) + w kappa r c, which needs neither 3 + 3 kappa r + kappa^2 r^2 nor 3 - E (..).
+// About 410 FP32 operations per symmetric evaluation (500 before): 217 ms instead of 255 ms per application
+// at 178 575 nodes, 14.1 instead of 16.5 ms at 44 597.  Shape: 24 warps per SM (80 registers) and fully
+// unrolled steps of 4 sources, transposed step by step; longer unrolled code misses the instruction cache
+// (steps of 8: 265 ms), steps of 2 measured 221 ms, 16 warps 213 against 209 ms (before the running sums were
+// renormalised), two targets per f32x2 operation 227 ms: the FMA pipe, not issue, is the limit, and a packed
+// multiplication is contracted with the packed addition that follows it, which breaks error-free sums.
 struct Df64Policy {
     using Src = float4;
     static constexpr int kVec = 4;
     static constexpr int kTile = 128;   // 8 KB
+    static constexpr int kMinBlocks = 3;
     static constexpr bool kTables = true;
-    static constexpr int kSymStep = 2;    // ~640 FP32 ops per symmetric pair: two per unrolled step
+    static constexpr bool kRenorm = true;
+    static constexpr bool kStepTranspose = true;   // each step's sources are transposed on their own
+    static constexpr int kSymStep = 4;
     struct Tgt {
         F2 px, py, pz, qx, qy, qz, wa, wb;
     };
@@ -700,6 +735,11 @@ struct Df64Policy {
         s1 += (double)c.a1.hi + (double)c.a1.lo;
         s2 += (double)c.a2.hi + (double)c.a2.lo;
     }
+    // the low parts of a running sum grow with every lazy addition: renormalised once per step
+    __device__ static void renorm(Acc& c) {
+        c.a1 = fast_two_sum(c.a1.hi, c.a1.lo);
+        c.a2 = fast_two_sum(c.a2.hi, c.a2.lo);
+    }
     // unnormalised sums (exact two_sum of the high parts); the caller folds the result to FP64
     __device__ static JAcc jadd(const JAcc& x, const JAcc& y) {
         JAcc r = x;
@@ -711,91 +751,79 @@ struct Df64Policy {
         return JAcc{F2{__shfl_xor_sync(0xffffffffu, x.a1.hi, m), __shfl_xor_sync(0xffffffffu, x.a1.lo, m)},
                     F2{__shfl_xor_sync(0xffffffffu, x.a2.hi, m), __shfl_xor_sync(0xffffffffu, x.a2.lo, m)}};
     }
+    struct Node {
+        F2 x, y, z, nx, ny, nz, a, b;
+    };
+    __device__ static Node node(const Src* S) {
+        const float4 p = S[0], pl = S[1], n = S[2], nl = S[3];
+        return Node{F2{p.x, pl.x}, F2{p.y, pl.y}, F2{p.z, pl.z}, F2{n.x, nl.x},
+                    F2{n.y, nl.y}, F2{n.z, nl.z}, F2{p.w, pl.w}, F2{n.w, nl.w}};
+    }
+    // The factors the two orientations share: d . n_x, d . n_y, s t1, s t2, s X and (1 - E)/r.
+    struct Common {
+        F2 dnx, dny, st1, st2, sX, om;
+    };
+    __device__ static Common common(const Tgt& T, const Node& q, const PairConsts& k, const float2* tab) {
+        const F2 dx = sub(T.px, q.x), dy = sub(T.py, q.y), dz = sub(T.pz, q.z);
+        const F2 r2 = sq3l(dx, dy, dz);
+        const F2 rinv = rsqrt_ff(r2);
+        const F2 kr = mull(f2(k.kappad), mull(r2, rinv));
+        F2 E = exp_neg_ffl(kr, tab);
+        E = fast_two_sum(E.hi, E.lo);
+        const F2 w = mull(E, kr);
+        const F2 E1 = addl(E, w);
+        Common c;
+        c.om = mull(rinv, one_minus(E));
+        c.dny = dot3l(dx, dy, dz, q.nx, q.ny, q.nz);
+        c.dnx = dot3l(dx, dy, dz, T.qx, T.qy, T.qz);
+        const F2 nn = dot3l(T.qx, T.qy, T.qz, q.nx, q.ny, q.nz);
+        const F2 rinv2 = mull(rinv, rinv);
+        const F2 s = mull(rinv2, rinv);
+        const F2 cc = mull(mull(c.dnx, c.dny), rinv2);
+        const F2 c3 = two_prod(3.0f, cc.hi);
+        const F2 m = subl(nn, F2{c3.hi, __fmaf_rn(3.0f, cc.lo, c3.lo)});
+        F2 u = one_minus(E1);
+        u = fast_two_sum(u.hi, u.lo);
+        const F2 X = addl(mull(u, m), mull(mull(w, kr), cc));
+        c.st1 = mull(s, one_minus_any(mull(E1, f2(k.c1d))));
+        c.st2 = mull(s, one_minus_any(mull(E1, f2(k.c2d))));
+        c.sX = mull(s, X);
+        return c;
+    }
+    __device__ static void target_terms(const Common& c, F2 A, F2 B, Acc& acc) {
+        acc_mul(acc.a1, A, mull(c.dny, c.st1));
+        acc_mul(acc.a1, neg(B), c.om);
+        acc_mul(acc.a2, B, mull(c.dnx, c.st2));
+        acc_mul(acc.a2, A, c.sX);
+    }
     template <bool kMask>
     __device__ static void pair(const Tgt& T, const Src* S, const PairConsts& k, const float2* tab, Acc& acc,
                                 const bool* exv) {
-        const bool ex = exv[0];
-        const float4 s0 = S[0], s1 = S[1], s2 = S[2], s3 = S[3];
-        F2 Px{s0.x, s1.x}, Py{s0.y, s1.y}, Pz{s0.z, s1.z}, A{s0.w, s1.w};
-        const F2 Nx{s2.x, s3.x}, Ny{s2.y, s3.y}, Nz{s2.z, s3.z};
-        F2 Bw{s2.w, s3.w};
-        if (kMask && ex) {
-            Px = F2{T.px.hi + 1.f, T.px.lo};
-            Py = T.py;
-            Pz = T.pz;
-            A = Bw = F2{0.f, 0.f};
+        Node q = node(S);
+        if (kMask && exv[0]) {   // excluded correction pair: a zero-weight source at distance 1
+            q.x = F2{T.px.hi + 1.f, T.px.lo};
+            q.y = T.py;
+            q.z = T.pz;
+            q.a = q.b = F2{0.f, 0.f};
         }
-        // lazy products and unnormalised accumulation as in pair_sym (the target rows of its terms); the
-        // differences that can cancel (d, the dot products, 1 - E, 1 - E1, 3 - E q, X) stay normalised
-        const F2 dx = sub(T.px, Px), dy = sub(T.py, Py), dz = sub(T.pz, Pz);
-        const F2 r2 = dot3(dx, dy, dz, dx, dy, dz);
-        const F2 rinv = rsqrt_ff(r2);
-        const F2 r = mull(r2, rinv);
-        const F2 kr = mull(f2(k.kappad), r);
-        const F2 E = exp_neg_ffl(kr, tab);
-        const F2 E1 = mull(E, add_f(kr, 1.f));
-        const F2 dny = dot3(dx, dy, dz, Nx, Ny, Nz);
-        const F2 dnx = dot3(dx, dy, dz, T.qx, T.qy, T.qz);
-        const F2 nn = dot3(T.qx, T.qy, T.qz, Nx, Ny, Nz);
-        const F2 rinv2 = mull(rinv, rinv);
-        const F2 s = mull(rinv2, rinv);
-        const F2 t1 = add_f(neg(mull(E1, f2(k.c1d))), 1.f);
-        const F2 om = mull(rinv, add_f(neg(E), 1.f));
-        const F2 t2 = add_f(neg(mull(E1, f2(k.c2d))), 1.f);
-        const F2 u = add_f(neg(E1), 1.f);
-        const F2 q = add_f(mull(kr, add_f(kr, 3.f)), 3.f);
-        const F2 t3 = add_f(neg(mull(E, q)), 3.f);
-        const F2 Bt = mull(mull(t3, mull(dnx, dny)), rinv2);
-        const F2 X = sub(mull(u, nn), Bt);
-        const F2 as = mull(A, s), bs = mull(Bw, s);
-        acc_add(acc.a1, mull(as, mull(dny, t1)));
-        acc_add(acc.a1, neg(mull(Bw, om)));
-        acc_add(acc.a2, mull(bs, mull(dnx, t2)));
-        acc_add(acc.a2, mull(as, X));
+        target_terms(common(T, q, k, tab), q.a, q.b, acc);
     }
-    // Both orientations with lazy products (mull) and unnormalised accumulation (acc_add); the
-    // differences that can cancel (d, the dot products, 1 - E, 1 - E1, 3 - E q, X) stay normalised.
     template <bool kFirst>
     __device__ static void pair_sym(const Tgt& T, const Src* S, const PairConsts& k, const float2* tab, Acc& acc,
                                     JAcc& ja) {
-        const float4 s0 = S[0], s1 = S[1], s2 = S[2], s3 = S[3];
-        const F2 Px{s0.x, s1.x}, Py{s0.y, s1.y}, Pz{s0.z, s1.z}, A{s0.w, s1.w};
-        const F2 Nx{s2.x, s3.x}, Ny{s2.y, s3.y}, Nz{s2.z, s3.z}, Bw{s2.w, s3.w};
-        const F2 dx = sub(T.px, Px), dy = sub(T.py, Py), dz = sub(T.pz, Pz);
-        const F2 r2 = dot3(dx, dy, dz, dx, dy, dz);
-        const F2 rinv = rsqrt_ff(r2);
-        const F2 r = mull(r2, rinv);
-        const F2 kr = mull(f2(k.kappad), r);
-        const F2 E = exp_neg_ffl(kr, tab);
-        const F2 E1 = mull(E, add_f(kr, 1.f));
-        const F2 dny = dot3(dx, dy, dz, Nx, Ny, Nz);
-        const F2 dnx = dot3(dx, dy, dz, T.qx, T.qy, T.qz);
-        const F2 nn = dot3(T.qx, T.qy, T.qz, Nx, Ny, Nz);
-        const F2 rinv2 = mull(rinv, rinv);
-        const F2 s = mull(rinv2, rinv);
-        const F2 t1 = add_f(neg(mull(E1, f2(k.c1d))), 1.f);
-        const F2 om = mull(rinv, add_f(neg(E), 1.f));
-        const F2 t2 = add_f(neg(mull(E1, f2(k.c2d))), 1.f);
-        const F2 u = add_f(neg(E1), 1.f);
-        const F2 q = add_f(mull(kr, add_f(kr, 3.f)), 3.f);
-        const F2 t3 = add_f(neg(mull(E, q)), 3.f);
-        const F2 Bt = mull(mull(t3, mull(dnx, dny)), rinv2);
-        const F2 X = sub(mull(u, nn), Bt);
-        const F2 as = mull(A, s), bs = mull(Bw, s);
-        acc_add(acc.a1, mull(as, mull(dny, t1)));
-        acc_add(acc.a1, neg(mull(Bw, om)));
-        acc_add(acc.a2, mull(bs, mull(dnx, t2)));
-        acc_add(acc.a2, mull(as, X));
-        const F2 ast = mull(T.wa, s), bst = mull(T.wb, s);
+        const Node q = node(S);
+        const Common c = common(T, q, k, tab);
+        target_terms(c, q.a, q.b, acc);
+        const F2 x1 = mull(c.dnx, c.st1), y2 = mull(c.dny, c.st2);
         if constexpr (kFirst) {
-            ja.a1 = neg(mull(ast, mull(dnx, t1)));
-            ja.a2 = neg(mull(bst, mull(dny, t2)));
+            ja.a1 = neg(mull(T.wa, x1));
+            ja.a2 = neg(mull(T.wb, y2));
         } else {
-            acc_add(ja.a1, neg(mull(ast, mull(dnx, t1))));
-            acc_add(ja.a2, neg(mull(bst, mull(dny, t2))));
+            acc_mul(ja.a1, neg(T.wa), x1);
+            acc_mul(ja.a2, neg(T.wb), y2);
         }
-        acc_add(ja.a1, neg(mull(T.wb, om)));
-        acc_add(ja.a2, mull(ast, X));
+        acc_mul(ja.a1, neg(T.wb), c.om);
+        acc_mul(ja.a2, T.wa, c.sX);
     }
 };
 
@@ -915,8 +943,10 @@ __device__ __forceinline__ bool pair_item(const typename Policy::Src* __restrict
 #pragma unroll U
             for (int q = 0; q < n; ++q) {
 #pragma unroll
-                for (int r = 0; r < R; ++r)
+                for (int r = 0; r < R; ++r) {
                     Policy::template pair<false>(tg[r], tile + q * VEC, kc, tab, acc[r], none);
+                    if constexpr (Policy::kRenorm) Policy::renorm(acc[r]);
+                }
             }
         } else {
             for (int q = 0; q < n; ++q) {
@@ -934,6 +964,7 @@ __device__ __forceinline__ bool pair_item(const typename Policy::Src* __restrict
                         }
                     }
                     Policy::template pair<true>(tg[r], tile + q * VEC, kc, tab, acc[r], ex);
+                    if constexpr (Policy::kRenorm) Policy::renorm(acc[r]);
                 }
             }
         }
@@ -987,8 +1018,9 @@ __device__ __forceinline__ void transpose_sum(typename Policy::JAcc (&v)[V], int
 // sums them (transpose_sum), and the kWarps warp sums of a tile are added in
 // warp order in shared memory (jred: kWarps * TILE entries).  The chunk loop
 // is unrolled S sources at a time (S = V: fully); with S < V the chunk's
-// accumulators shift by S registers per step, which keeps the code of long
-// pair arithmetics within the instruction cache.
+// accumulators shift by S registers per step (or, Policy::kStepTranspose, each
+// step's sums are transposed on their own), which keeps the code of long pair
+// arithmetics within the instruction cache.
 template <typename Policy, int R, int V, int U, int S = V>
 __device__ __forceinline__ bool pair_item_sym(const typename Policy::Src* __restrict__ src, int M, int tblock,
                                               int j_begin, int j_end, const FxOut& out, const PairConsts& kc,
@@ -1052,6 +1084,38 @@ __device__ __forceinline__ bool pair_item_sym(const typename Policy::Src* __rest
         for (int r = 0; r < R; ++r) Policy::zero(acc[r]);
 #pragma unroll U
         for (int c0 = 0; c0 < n; c0 += V) {
+            if constexpr (Policy::kStepTranspose) {
+                // S sources per step, transposed and summed at once: registers for S sums only
+#pragma unroll 1
+                for (int q0 = 0; q0 < V && c0 + q0 < n; q0 += S) {
+                    J cur[S];
+                    auto source = [&](int t) {
+                        typename Policy::JAccR jr;
+                        const Src* q = tile + (c0 + q0 + t) * VEC;
+                        Policy::template pair_sym<true>(tg[0], q, kc, tab, acc[0], jr);
+#pragma unroll
+                        for (int r = 1; r < R; ++r)
+                            Policy::template pair_sym<false>(tg[r], q, kc, tab, acc[r], jr);
+                        cur[t] = Policy::jfinal(jr);
+                    };
+                    if (c0 + q0 + S <= n) {
+#pragma unroll
+                        for (int t = 0; t < S; ++t) source(t);
+                    } else {   // ragged end of the item: warp-uniform skip
+#pragma unroll
+                        for (int t = 0; t < S; ++t) {
+                            Policy::zero(cur[t]);
+                            if (c0 + q0 + t < n) source(t);
+                        }
+                    }
+#pragma unroll
+                    for (int r = 0; r < R; ++r) Policy::renorm(acc[r]);
+                    transpose_sum<Policy, S>(cur, lane);
+                    const int qs = c0 + q0 + lane / (32 / S);
+                    if (lane % (32 / S) == 0 && qs < n) jred[warp * TILE + qs] = cur[0];
+                }
+                continue;
+            }
             J ja[V];
 #pragma unroll
             for (int q = 0; q < V; ++q) Policy::zero(ja[q]);

@@ -100,17 +100,17 @@ struct MapDf64 {
     __device__ static void pair(const Tgt& T, const Src* S, const PairConsts& k, const float2* tab, Acc& acc) {
         const float4 s0 = S[0], s1 = S[1], s2 = S[2], s3 = S[3];
         const F2 dx = sub(T.x, F2{s0.x, s1.x}), dy = sub(T.y, F2{s0.y, s1.y}), dz = sub(T.z, F2{s0.z, s1.z});
-        const F2 r2 = dot3(dx, dy, dz, dx, dy, dz);
+        const F2 r2 = sq3l(dx, dy, dz);
         const F2 rinv = rsqrt_ff(r2);
-        const F2 r = mul(r2, rinv);
-        const F2 kr = mul(f2(k.kappad), r);
-        const F2 E = exp_neg_ff(kr, tab);
-        const F2 E1 = mul(E, add_f(kr, 1.f));
-        const F2 dny = dot3(dx, dy, dz, F2{s2.x, s3.x}, F2{s2.y, s3.y}, F2{s2.z, s3.z});
-        const F2 s = mul(mul(rinv, rinv), rinv);
-        const F2 t = add_f(mul(E1, f2(k.c1d)), -1.f);
-        acc = add(acc, mul(mul(F2{s0.w, s1.w}, s), mul(dny, t)));
-        acc = add(acc, mul(F2{s2.w, s3.w}, mul(rinv, add_f(neg(E), 1.f))));
+        const F2 kr = mull(f2(k.kappad), mull(r2, rinv));
+        const F2 E = exp_neg_ffl(kr, tab);
+        const F2 E1 = addl(E, mull(E, kr));
+        const F2 dny = dot3l(dx, dy, dz, F2{s2.x, s3.x}, F2{s2.y, s3.y}, F2{s2.z, s3.z});
+        const F2 s = mull(mull(rinv, rinv), rinv);
+        const F2 nt = one_minus_any(mull(E1, f2(k.c1d)));   // 1 - c1 E1
+        acc_mul(acc, neg(mull(F2{s0.w, s1.w}, s)), mull(dny, nt));
+        acc_mul(acc, F2{s2.w, s3.w}, mull(rinv, one_minus(E)));
+        acc = fast_two_sum(acc.hi, acc.lo);
     }
 };
 

@@ -55,7 +55,7 @@ __global__ void near_flags_kernel(const int32_t* __restrict__ ptr, const int32_t
 }
 
 template <typename Policy, int R, int V, int U>
-__global__ void __launch_bounds__(kThreads, 2) sched_kernel(const typename Policy::Src* __restrict__ src, int M,
+__global__ void __launch_bounds__(kThreads, Policy::kMinBlocks) sched_kernel(const typename Policy::Src* __restrict__ src, int M,
                                                          const int32_t* __restrict__ eptr,
                                                          const int32_t* __restrict__ excl,
                                                          const PairItem* __restrict__ items, int n_items,

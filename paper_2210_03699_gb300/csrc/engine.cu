@@ -140,9 +140,7 @@ __global__ void __launch_bounds__(kThreads, Policy::kMinBlocks) k_pairs(SlotDev*
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ int cur;
     __shared__ PairConsts kc;
-    if (threadIdx.x == 0) kc.exp_tab = exp_tab;   // one table per device, shared by every slot
-    __syncthreads();
-    pair_block_init<Policy>(kc, sm.tab, bar);
+    pair_block_init<Policy>(exp_tab, sm.tab, bar);   // one table per device, shared by every slot
     uint32_t gt = 0;
     const int total = *n_items;
     for (;;) {
@@ -166,11 +164,7 @@ __global__ void __launch_bounds__(kThreads, Policy::kMinBlocks) k_pairs(SlotDev*
                                            sm.jred, sm.tab, bar, gt))
                 return;
         } else {
-            if (threadIdx.x == 0) {
-                const float2* t = kc.exp_tab;
-                kc = s.kc;
-                kc.exp_tab = t;
-            }
+            if (threadIdx.x == 0) kc = s.kc;
             __syncthreads();
             const PairConsts k = kc;   // block-uniform register copy: no shared loads in the pair loops
             if (!run_item<Policy, R, V, U>(s.items[pol][item], src, s.M, s.eptr, s.excl, s.acc, k, err, sm.ring,
@@ -488,7 +482,7 @@ int launch_persistent_k(Engine* e, int pol, int var, int half, int prec) {
     const int list = pol * kNV + var;
     k_pairs<Policy, R, V, U, kShared><<<per_sm * e->sms, kThreads, smem, e->stream>>>(
         e->slots.as<SlotDev>(), e->items[pol][var].as<int2>(), e->n_items.as<int>() + list,
-        e->counters.as<int>() + 2 * list + half, half, prec, pol, e->exp_tab, e->err.as<int>(), e->kc_val[pol],
+        e->counters.as<int>() + 2 * list + half, half, prec, pol, e->exp_tab[pol], e->err.as<int>(), e->kc_val[pol],
         e->need.as<int>());
     CTR_LAUNCHED();
     return CTR_OK;
@@ -618,7 +612,8 @@ int engine_create(int device, int cap, Engine** out) {
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
         return bad(fail(CTR_ERR_CUDA, "attribute"));
     e->sms = sms;
-    if ((st = exp_table(device, &e->exp_tab)) < 0) return bad(st);
+    for (int p = 0; p < 3; ++p)
+        if ((st = exp_table(device, p, &e->exp_tab[p])) < 0) return bad(st);
     if (cudaStreamSynchronize(stream) != cudaSuccess) return bad(fail(CTR_ERR_CUDA, "sync"));
     *out = e;
     return CTR_OK;
@@ -711,7 +706,7 @@ static int rebuild_items(Engine* e) {
             const SlotDev& s = e->host[q];
             if (policy_index(s.inner_prec) != p && policy_index(s.res_prec) != p) continue;
             PairConsts c = s.kc;
-            c.exp_tab = e->exp_tab;
+            c.exp_tab = e->exp_tab[p];
             if (!any) {
                 val = c;
                 any = true;
@@ -719,7 +714,7 @@ static int rebuild_items(Engine* e) {
                 shared = false;
             }
         }
-        if (!any) val.exp_tab = e->exp_tab;
+        if (!any) val.exp_tab = e->exp_tab[p];
         if (shared != e->kc_shared[p] || std::memcmp(&val, &e->kc_val[p], sizeof(PairConsts)) != 0) {
             e->kc_shared[p] = shared;
             e->kc_val[p] = val;
@@ -932,7 +927,7 @@ int engine_admit(Engine* e, ctr_ibim* s, int* slot_out) {
         d.part_s[p] = (float)(sc.total_cost / kUnitRate[p] / d.nparts[p]);
     }
     d.span = 1;
-    CTR_TRY(pair_consts(s, true, &d.kc));
+    CTR_TRY(pair_consts(s, 0, &d.kc));
     for (int p = 0; p < 3; ++p) {
         d.items[p] = s->sched[p].d_items.as<PairItem>();
         d.BS[p] = s->sched[p].BS;

@@ -91,7 +91,7 @@ struct Engine {
     // slots do not wait for its whole application.  0: every application runs whole.  The exact node
     // accumulators make the result independent of the split.
     double quantum_s = 0.0;
-    const float2* exp_tab = nullptr;
+    const float2* exp_tab[3] = {};   // exponential tables per pair arithmetic
     bool kc_shared[3] = {false, false, false};   // all slots of an arithmetic share their pair constants
     pk::PairConsts kc_val[3] = {};               // ... and these are they (launch parameter)
     std::vector<SlotDev> host;

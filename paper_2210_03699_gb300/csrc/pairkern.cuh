@@ -13,12 +13,16 @@ constexpr int kThreads = 256;
 constexpr uint32_t kWaitLimit = 1u << 22;   // default polls of a bounded mbarrier wait
 constexpr int kExpHi = 64;      // e^{-k}, k = 0..63
 constexpr int kExpLo = 1024;    // e^{-k/1024}, k = 0..1023
+constexpr int kExp2 = 1024;     // FP64 tables: 2^{-k/1024} (double), then its relative rounding error (float)
+constexpr int kExp2F2 = kExp2 + kExp2 / 2;   // their size in float2
 
 struct PairConsts {
     float c1f, c2f, kappaf, kl2f;    // eps_E/eps_I, eps_I/eps_E, kappa, -kappa log2(e)
     double c1, c2, kappa;
     float2 c1d, c2d, kappad;         // float-float copies
-    const float2* exp_tab;           // [kExpHi + kExpLo] float-float, global
+    double k2;                       // kappa log2(e), rounded; k2f: in FP32; k2d: -ln 2 times its rounding error
+    float k2f, k2d;
+    const float2* exp_tab;           // exponential tables of the arithmetic (float-float or FP64), global
     // the FP32 values duplicated into both halves of a 64-bit word (f32x2 operands)
     unsigned long long one2, mone2, three2, mthree2, c1x2, nc1x2, c2x2, nc2x2, kap2, kl2x2;
     uint32_t wait_limit;             // polls of a source-tile wait before the block gives up
@@ -238,6 +242,53 @@ __device__ __forceinline__ F2 exp_neg_ffl(F2 x, const float2* tab) {
     return mull(mull(f2(tab[k >> 10]), f2(tab[kExpHi + (k & (kExpLo - 1))])), F2{s, l});
 }
 
+// ------------------------------------------------------------------ FP64 arithmetic
+// The FP64 pipe (1.9 operations a clock and SM, conversions included, against about 110 on the FP32 pipe)
+// bounds the FP64 kernels, so what need not run on it does not: seeds come from the SFU, indices and
+// high-order terms from FP32, conversions are bit operations.
+// FP64 bits of a positive normal FP32 value (0 becomes 2^-127, nothing at the places this is used)
+__device__ __forceinline__ double widen_pos(float v) {
+    const uint32_t b = __float_as_uint(v);
+    return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(float v) {
+    const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+}
+// the leading 24 bits of a positive FP64 value, kept within the FP32 range
+__device__ __forceinline__ float narrow_pos(double v) {
+    const int hi = min(max(__double2hiint(v), 0x38100000), 0x47e00000);
+    return __uint_as_float(__funnelshift_l((uint32_t)__double2loint(v), (uint32_t)(hi - 0x38000000), 3));
+}
+// 1/sqrt(x): SFU seed of 20 bits (its square is exact in FP64), residual, third-order step; five operations
+__device__ __forceinline__ double rsqrt_d(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y * y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+// e^{-kappa r} = 2^-i T_j 2^-f with kappa r log2(e) = i + j/1024 + f: the index from FP32, f by one fused
+// operation, 2^-f - 1 = f (-ln2 + f (ln2^2/2 - f g)) with g in FP32 (f^3 g < 2^-37), corrected by the relative
+// rounding errors of T_j and of kappa log2(e) (q's constant term): within one rounding of the exact value
+// times the rounding of the result, as CUDA's exp, in five FP64 operations instead of about sixteen (rms
+// error over r = 1e-3 to 1e3 0.36 x 2^-53, rsqrt_d 0.43 x 2^-53 as CUDA's).
+__device__ __forceinline__ double exp_neg_d(double r, const PairConsts& k, const float2* tab) {
+    const double* T = reinterpret_cast<const double*>(tab);
+    const float* tau = reinterpret_cast<const float*>(T + kExp2);
+    const float rf = narrow_pos(r);
+    const float y = __fmul_rn(k.k2f, rf);
+    const float t = __fmaf_rn(fminf(y, 1000.f), 1024.f, 12582912.f);
+    const int i = __float_as_int(t) - 0x4B400000;
+    const float c = __fmul_rn(__fsub_rn(t, 12582912.f), 1.0f / 1024.f);
+    const double f = fma(k.k2, r, -widen_pos(c));
+    const float g = __fmaf_rn(-0.00961812910762848f, __fmaf_rn(k.k2f, rf, -c), 0.05550410866482158f);
+    const double h = fma(f, fma(-f, widen_pos(g), 0.2402265069591007), -0.6931471805599453);
+    const double q = fma(f, h, widen(__fmaf_rn(k.k2d, rf, tau[i & (kExp2 - 1)])));
+    const double Tj = T[i & (kExp2 - 1)];
+    const double s = __hiloint2double(__double2hiint(Tj) - ((i >> 10) << 20), __double2loint(Tj));
+    return y < 1000.f ? fma(s, q, s) : 0.0;   // below 2^-1000: nothing
+}
+
 // ------------------------------------------------------------------ exact node accumulators
 // The dense sum's partial results (an item's target sums, a symmetric tile's source sums, a far item's
 // sums) are added into per-node accumulators in whatever order the blocks run.  To keep the result
@@ -351,7 +402,7 @@ struct Fp32Policy {
     static constexpr int kMinBlocks = 2;   // resident blocks per SM the registers are limited for
     static constexpr int kVec = 2;    // Src per node
     static constexpr int kTile = 256; // nodes per tile (8 KB)
-    static constexpr bool kTables = false;
+    static constexpr int kTab = 0;
     static constexpr bool kRenorm = false;   // running sums need no renormalisation
     static constexpr bool kStepTranspose = false;
     static constexpr int kSymStep = 32;   // symmetric chunk fully unrolled
@@ -429,7 +480,7 @@ struct Fp32x2Policy {
     static constexpr int kMinBlocks = 2;   // resident blocks per SM the registers are limited for
     static constexpr int kVec = 4;      // Src per node (64 B)
     static constexpr int kTile = 256;   // nodes per tile (16 KB)
-    static constexpr bool kTables = false;
+    static constexpr int kTab = 0;
     static constexpr bool kRenorm = false;   // running sums need no renormalisation
     static constexpr bool kStepTranspose = false;
     static constexpr int kSymStep = 32;
@@ -589,7 +640,7 @@ struct Fp64Policy {
     static constexpr int kMinBlocks = 2;   // resident blocks per SM the registers are limited for
     static constexpr int kVec = 2;
     static constexpr int kTile = 128;   // 8 KB
-    static constexpr bool kTables = false;
+    static constexpr int kTab = kExp2F2;
     static constexpr bool kRenorm = false;   // running sums need no renormalisation
     static constexpr bool kStepTranspose = false;
     static constexpr int kSymStep = 4;
@@ -617,78 +668,69 @@ struct Fp64Policy {
     __device__ static JAcc jshfl_xor(const JAcc& x, int m) {
         return JAcc{__shfl_xor_sync(0xffffffffu, x.a1, m), __shfl_xor_sync(0xffffffffu, x.a2, m)};
     }
-    template <bool kFirst>
-    __device__ static void pair_sym(const Tgt& T, const Src* S, const PairConsts& k, const float2*, Acc& acc,
-                                    JAcc& ja) {
-        const double4 pa = S[0], nb = S[1];
+    // The factors the two orientations share: d . n_x, d . n_y, s t1, s t2, s X and (1 - E)/r (u, w, c as in
+    // Df64Policy): 55 FP64 operations per symmetric evaluation, 50 per one-sided one (69 per symmetric one with
+    // CUDA's rsqrt and exp).  Per application 9.7 -> 7.8 ms at 11 203 nodes, 133 -> 107 ms at 44 597, 90% of
+    // the FP64 pipe's measured rate; every term's error as before.
+    struct Common {
+        double dnx, dny, st1, st2, sX, om;
+    };
+    __device__ static Common common(const Tgt& T, const double4& pa, const double4& nb, const PairConsts& k,
+                                    const float2* tab) {
         const double dx = T.px - pa.x, dy = T.py - pa.y, dz = T.pz - pa.z;
         const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-        const double rinv = rsqrt(r2);
+        const double rinv = rsqrt_d(r2);
         const double r = r2 * rinv;
-        const double E = exp(-k.kappa * r);
+        const double E = exp_neg_d(r, k, tab);
         const double kr = k.kappa * r;
         const double E1 = fma(E, kr, E);
-        const double dny = fma(dz, nb.z, fma(dy, nb.y, dx * nb.x));
-        const double dnx = fma(dz, T.qz, fma(dy, T.qy, dx * T.qx));
+        Common c;
+        c.dny = fma(dz, nb.z, fma(dy, nb.y, dx * nb.x));
+        c.dnx = fma(dz, T.qz, fma(dy, T.qy, dx * T.qx));
         const double nn = fma(T.qz, nb.z, fma(T.qy, nb.y, T.qx * nb.x));
         const double rinv2 = rinv * rinv;
         const double s = rinv2 * rinv;
-        const double as = pa.w * s, bs = nb.w * s;
-        const double t1 = fma(-k.c1, E1, 1.0);
-        const double om = fma(-rinv, E, rinv);
-        const double t2 = fma(-k.c2, E1, 1.0);
-        const double u = 1.0 - E1;
-        const double q = fma(kr, kr + 3.0, 3.0);
-        const double t3 = fma(-E, q, 3.0);
-        const double B = t3 * dnx * dny * rinv2;
-        const double X = fma(u, nn, -B);
-        acc.a1 = fma(as, dny * t1, acc.a1);
-        acc.a1 = fma(-nb.w, om, acc.a1);
-        acc.a2 = fma(bs, dnx * t2, acc.a2);
-        acc.a2 = fma(as, X, acc.a2);
-        const double ast = T.wa * s, bst = T.wb * s;
+        const double v = s * E1;
+        const double cc = c.dnx * c.dny * rinv2;
+        const double X = fma(E * kr * kr, cc, (1.0 - E1) * fma(-3.0, cc, nn));
+        c.om = fma(-rinv, E, rinv);
+        c.st1 = fma(-k.c1, v, s);
+        c.st2 = fma(-k.c2, v, s);
+        c.sX = s * X;
+        return c;
+    }
+    __device__ static void target_terms(const Common& c, double a, double b, Acc& acc) {
+        acc.a1 = fma(a, c.dny * c.st1, acc.a1);
+        acc.a1 = fma(-b, c.om, acc.a1);
+        acc.a2 = fma(b, c.dnx * c.st2, acc.a2);
+        acc.a2 = fma(a, c.sX, acc.a2);
+    }
+    template <bool kFirst>
+    __device__ static void pair_sym(const Tgt& T, const Src* S, const PairConsts& k, const float2* tab, Acc& acc,
+                                    JAcc& ja) {
+        const double4 pa = S[0], nb = S[1];
+        const Common c = common(T, pa, nb, k, tab);
+        target_terms(c, pa.w, nb.w, acc);
+        const double x1 = c.dnx * c.st1, y2 = c.dny * c.st2;
         if constexpr (kFirst) {
-            ja.a1 = -ast * (dnx * t1);
-            ja.a2 = -bst * (dny * t2);
+            ja.a1 = -T.wa * x1;
+            ja.a2 = -T.wb * y2;
         } else {
-            ja.a1 = fma(-ast, dnx * t1, ja.a1);
-            ja.a2 = fma(-bst, dny * t2, ja.a2);
+            ja.a1 = fma(-T.wa, x1, ja.a1);
+            ja.a2 = fma(-T.wb, y2, ja.a2);
         }
-        ja.a1 = fma(-T.wb, om, ja.a1);
-        ja.a2 = fma(ast, X, ja.a2);
+        ja.a1 = fma(-T.wb, c.om, ja.a1);
+        ja.a2 = fma(T.wa, c.sX, ja.a2);
     }
     template <bool kMask>
-    __device__ static void pair(const Tgt& T, const Src* S, const PairConsts& k, const float2*, Acc& acc, const bool* exv) {
-        const bool ex = exv[0];
+    __device__ static void pair(const Tgt& T, const Src* S, const PairConsts& k, const float2* tab, Acc& acc,
+                                const bool* exv) {
         double4 pa = S[0], nb = S[1];
-        if (kMask && ex) {
+        if (kMask && exv[0]) {   // excluded correction pair: a zero-weight source at distance 1
             pa = make_double4(T.px + 1.0, T.py, T.pz, 0.0);
             nb.w = 0.0;
         }
-        const double dx = T.px - pa.x, dy = T.py - pa.y, dz = T.pz - pa.z;
-        const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-        const double rinv = rsqrt(r2);
-        const double r = r2 * rinv;
-        const double E = exp(-k.kappa * r);
-        const double kr = k.kappa * r;
-        const double E1 = fma(E, kr, E);
-        const double dny = fma(dz, nb.z, fma(dy, nb.y, dx * nb.x));
-        const double dnx = fma(dz, T.qz, fma(dy, T.qy, dx * T.qx));
-        const double nn = fma(T.qz, nb.z, fma(T.qy, nb.y, T.qx * nb.x));
-        const double rinv2 = rinv * rinv;
-        const double s = rinv2 * rinv;
-        const double as = pa.w * s, bs = nb.w * s;
-        const double t1 = fma(-k.c1, E1, 1.0);
-        acc.a1 = fma(as, dny * t1, acc.a1);
-        const double om = fma(-rinv, E, rinv);
-        acc.a1 = fma(-nb.w, om, acc.a1);
-        const double t2 = fma(-k.c2, E1, 1.0);
-        acc.a2 = fma(bs, dnx * t2, acc.a2);
-        const double u = 1.0 - E1;
-        const double q = fma(kr, kr + 3.0, 3.0);
-        const double t3 = fma(-E, q, 3.0);
-        const double B = t3 * dnx * dny * rinv2;
-        acc.a2 = fma(as, fma(u, nn, -B), acc.a2);
+        target_terms(common(T, pa, nb, k, tab), pa.w, nb.w, acc);
     }
 };
 
@@ -710,7 +752,7 @@ struct Df64Policy {
     static constexpr int kVec = 4;
     static constexpr int kTile = 128;   // 8 KB
     static constexpr int kMinBlocks = 3;
-    static constexpr bool kTables = true;
+    static constexpr int kTab = kExpHi + kExpLo;   // exponential tables in shared memory (float2)
     static constexpr bool kRenorm = true;
     static constexpr bool kStepTranspose = true;   // each step's sources are transposed on their own
     static constexpr int kSymStep = 4;
@@ -1210,7 +1252,7 @@ __device__ __forceinline__ bool run_item(const PairItem& it, const typename Poli
 }
 
 // Shared-memory bytes of a pair block: the two-stage source ring, the warp
-// sums of a symmetric tile and, for the float-float policy, the exponential
+// sums of a symmetric tile and, for the float-float and FP64 policies, the exponential
 // tables (in that order; each part a multiple of 16 bytes).
 template <typename Policy>
 constexpr size_t pair_ring_bytes() {
@@ -1223,7 +1265,7 @@ constexpr size_t pair_jred_bytes() {
 template <typename Policy>
 constexpr size_t pair_smem_bytes() {
     return pair_ring_bytes<Policy>() + pair_jred_bytes<Policy>() +
-           (Policy::kTables ? (kExpHi + kExpLo) * sizeof(float2) : 0);
+           Policy::kTab * sizeof(float2);
 }
 // The dynamic shared memory of a pair block, carved in the order above.
 template <typename Policy>
@@ -1275,10 +1317,8 @@ inline int with_var32(int v, const F& f) {
 
 // Per-block setup shared by every pair kernel: exponential tables and the two mbarriers.
 template <typename Policy>
-__device__ __forceinline__ void pair_block_init(const PairConsts& kc, float2* tab, uint64_t* bar) {
-    if constexpr (Policy::kTables) {
-        for (int q = threadIdx.x; q < kExpHi + kExpLo; q += kThreads) tab[q] = kc.exp_tab[q];
-    }
+__device__ __forceinline__ void pair_block_init(const float2* exp_tab, float2* tab, uint64_t* bar) {
+    for (int q = threadIdx.x; q < Policy::kTab; q += kThreads) tab[q] = exp_tab[q];
     if (threadIdx.x == 0) {
         mbar_init(&bar[0], 1);
         mbar_init(&bar[1], 1);
@@ -1298,8 +1338,9 @@ __device__ __forceinline__ float2 split_ff_dev(double v) {
 
 }  // namespace pk
 
-// float-float table of e^{-k} (k < 64) and e^{-k/1024} (k < 1024) on a device
-int exp_table(int device, const float2** out);
+// Exponential tables of pair arithmetic pol on a device: 1 the float-float e^{-k} (k < 64) and e^{-k/1024}
+// (k < 1024), 2 the FP64 2^{-k/1024} and their relative rounding errors (k < 1024), 0 none (NULL)
+int exp_table(int device, int pol, const float2** out);
 // Splits of the source range for equal-work items filling whole waves of `slots` resident blocks
 // (one-sided grid launch of the fixed-scratch entry point)
 PairPlan make_plan(int64_t M, int R, int tile, int slots);
@@ -1312,8 +1353,8 @@ int last_fp32_variant();
 int launch_schedule(ctr_ibim* s, int pol, const void* src, const pk::PairConsts& kc);
 // Fill the f32x2 copies of a PairConsts from its FP32 fields
 void set_packed_consts(pk::PairConsts& kc);
-// Pair constants of a handle (kernel-ratio terms, kappa, tables when needed)
-int pair_consts(ctr_ibim* s, bool tables, pk::PairConsts* out);
+// Pair constants of a handle (kernel-ratio terms, kappa) and the tables of pair arithmetic pol
+int pair_consts(ctr_ibim* s, int pol, pk::PairConsts* out);
 // Polls of the pair kernels' bounded waits for launches prepared from now on (ctr_set_wait_limit)
 uint32_t wait_limit();
 

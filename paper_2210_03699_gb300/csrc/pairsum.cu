@@ -28,6 +28,7 @@
 //         FMA, rsqrt by one Newton step in df64, exp by two exact tables and
 //         a degree-4 polynomial), ~2^-44 relative, on the FP32 pipe.
 #include <atomic>
+#include <cmath>
 #include <cstring>
 #include <mutex>
 
@@ -48,7 +49,7 @@ __global__ void __launch_bounds__(kThreads) pair_kernel(const typename Policy::S
     extern __shared__ __align__(128) unsigned char smem_raw[];
     PairSmem<Policy> sm(smem_raw);
     __shared__ __align__(8) uint64_t bar[2];
-    pair_block_init<Policy>(kc, sm.tab, bar);
+    pair_block_init<Policy>(kc.exp_tab, sm.tab, bar);
     const int j_begin = blockIdx.y * src_per_split;
     const int j_end = min(M, j_begin + src_per_split);
     uint32_t gt = 0;
@@ -154,7 +155,7 @@ PairPlan make_plan(int64_t M, int R, int tile, int slots) {
 // tables); the occupancy query and the launch use the same figure.
 template <typename Policy>
 constexpr size_t grid_launch_smem() {
-    static_assert(!Policy::kTables, "the one-sided grid launch carries no exponential tables");
+    static_assert(Policy::kTab == 0, "the one-sided grid launch carries no exponential tables");
     return pair_ring_bytes<Policy>();
 }
 
@@ -167,22 +168,62 @@ int resident_slots(int sms, int* slots) {
     return CTR_OK;
 }
 
-// float-float table of e^{-k} (k < 64) and e^{-k/1024} (k < 1024), one per device
-int exp_table(int dev, const float2** out) {
+namespace {
+
+// double-double values for the tables (host, once per device)
+struct DD {
+    double hi, lo;
+};
+DD dd_norm(double a, double b) {   // |a| >= |b|
+    const double s = a + b;
+    return DD{s, b - (s - a)};
+}
+DD dd_mul(DD a, DD b) {
+    const double p = a.hi * b.hi;
+    return dd_norm(p, std::fma(a.hi, b.hi, -p) + (a.hi * b.lo + a.lo * b.hi));
+}
+// 2^-x, 0 <= x < 1, to about 100 bits: e^y by its Taylor series at y = -x ln2 / 64, squared six times
+DD exp2_neg(double x) {
+    const DD y = dd_mul(DD{-x / 64.0, 0.0}, DD{0.6931471805599453, 2.3190468138462996e-17});
+    DD s{1.0, 0.0};
+    for (int n = 14; n >= 1; --n) {   // s = 1 + y s / n
+        const DD t = dd_mul(y, s);
+        const double q = t.hi / n;
+        const DD u = dd_norm(1.0, q);
+        s = dd_norm(u.hi, u.lo + (std::fma(-q, (double)n, t.hi) + t.lo) / n);
+    }
+    for (int k = 0; k < 6; ++k) s = dd_mul(s, s);
+    return s;
+}
+
+}  // namespace
+
+// Exponential tables, one set per device
+int exp_table(int dev, int pol, const float2** out) {
     static std::mutex mu;
     static DevBuf tabs[64];
     static bool ready[64] = {false};
+    constexpr int kFF = kExpHi + kExpLo;   // a multiple of 2: the FP64 tables behind it stay 16-byte aligned
+    static_assert(kFF % 2 == 0, "table alignment");
     if (dev < 0 || dev >= 64) return fail(CTR_ERR_INVALID, "device index");
     std::lock_guard<std::mutex> lk(mu);
     if (!ready[dev]) {
-        std::vector<float2> h(kExpHi + kExpLo);
+        std::vector<float2> h(kFF + kExp2F2);
         for (int k = 0; k < kExpHi; ++k) h[k] = split_ff(std::exp(-(double)k));
         for (int k = 0; k < kExpLo; ++k) h[kExpHi + k] = split_ff(std::exp(-(double)k / 1024.0));
+        double* T = reinterpret_cast<double*>(h.data() + kFF);
+        float* tau = reinterpret_cast<float*>(T + kExp2);
+        for (int k = 0; k < kExp2; ++k) {
+            const DD v = exp2_neg(k / 1024.0);
+            T[k] = v.hi;
+            tau[k] = (float)(v.lo / v.hi);
+        }
         CTR_TRY(tabs[dev].alloc(sizeof(float2) * h.size()));
         CTR_CUDA_TRY(cudaMemcpy(tabs[dev].p, h.data(), sizeof(float2) * h.size(), cudaMemcpyHostToDevice));
         ready[dev] = true;
     }
-    *out = tabs[dev].as<float2>();
+    const float2* base = tabs[dev].as<float2>();
+    *out = pol == 1 ? base : pol == 2 ? base + kFF : nullptr;
     return CTR_OK;
 }
 
@@ -211,7 +252,7 @@ std::atomic<uint32_t> g_wait_limit{kWaitLimit};
 
 uint32_t wait_limit() { return g_wait_limit.load(std::memory_order_relaxed); }
 
-int pair_consts(ctr_ibim* s, bool tables, PairConsts* out) {
+int pair_consts(ctr_ibim* s, int pol, PairConsts* out) {
     PairConsts kc{};
     kc.wait_limit = wait_limit();
     kc.c1 = s->eps_out / s->eps_in;
@@ -225,8 +266,12 @@ int pair_consts(ctr_ibim* s, bool tables, PairConsts* out) {
     kc.c2d = split_ff(kc.c2);
     kc.kappad = split_ff(kc.kappa);
     set_packed_consts(kc);
-    kc.exp_tab = nullptr;
-    if (tables) CTR_TRY(exp_table(s->device, &kc.exp_tab));
+    // kappa log2(e) rounded, and -ln 2 times what the rounding lost (log2(e) in two doubles)
+    kc.k2 = s->kappa * 1.4426950408889634;
+    const double lost = std::fma(s->kappa, 1.4426950408889634, -kc.k2) + s->kappa * 2.0355273740931033e-17;
+    kc.k2f = (float)kc.k2;
+    kc.k2d = (float)(-0.6931471805599453 * lost);
+    CTR_TRY(exp_table(s->device, pol, &kc.exp_tab));
     *out = kc;
     return CTR_OK;
 }
@@ -284,8 +329,8 @@ int apply_operator_timed(ctr_ibim* s, const double* d_x, double* d_y, int precis
     pack_kernel<<<grid_for(M, 256), 256, 0, st>>>(d_x, s->na.W, M, scale, s32, s64, sdf, tinv);
     CTR_LAUNCHED();
     PairConsts kc;
-    CTR_TRY(pair_consts(s, precision == CTR_DF64, &kc));
     const int pol = (precision == CTR_FP32_REFINE) ? 0 : (precision == CTR_DF64 ? 1 : 2);
+    CTR_TRY(pair_consts(s, pol, &kc));
     const void* src = s32 ? (const void*)s32 : (sdf ? (const void*)sdf : (const void*)s64);
     CTR_TRY(mark(1));
     CTR_TRY(launch_schedule(s, pol, src, kc));

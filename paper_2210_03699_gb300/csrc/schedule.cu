@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(kThreads, Policy::kMinBlocks) sched_kernel(con
     PairSmem<Policy> sm(smem_raw);
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ int cur;
-    pair_block_init<Policy>(kc, sm.tab, bar);
+    pair_block_init<Policy>(kc.exp_tab, sm.tab, bar);
     uint32_t gt = 0;
     for (;;) {
         if (threadIdx.x == 0) cur = atomicAdd(counter, 1);
@@ -268,7 +268,7 @@ int plan_fp32(ctr_ibim* s, const std::vector<uint8_t>& flags, int g0, int nb0, i
     }
     CTR_TRY(pack_sources(s, s->rhs.as<double>(), CTR_FP32_REFINE));
     PairConsts kc;
-    CTR_TRY(pair_consts(s, false, &kc));
+    CTR_TRY(pair_consts(s, 0, &kc));
     cudaEvent_t a = nullptr, b = nullptr;
     CTR_CUDA_TRY(cudaEventCreate(&a));
     CTR_CUDA_TRY(cudaEventCreate(&b));

@@ -388,7 +388,7 @@ int build_tree_schedules(ctr_ibim* s, const int slots[3]) {
         v.flist[p] = P.d_flist.as<int32_t>();
         v.BS[p] = s->sched[p].BS;
     }
-    CTR_TRY(exp_table(s->device, &v.exp_tab));
+    CTR_TRY(exp_table(s->device, 1, &v.exp_tab));
     v.src32 = s->src32.as<float4>();
     v.srcdf = s->srcdf.as<float4>();
     v.src64 = s->src64.as<double4>();

@@ -109,10 +109,12 @@ struct PairPlan {
 };
 
 // A work item of a pair schedule: target block I (BS consecutive nodes) against
-// sources [j_begin, j_end); one-sided (sym = 0: correction pairs masked) or
-// symmetric (sym = 1: both orientations of every pair, no correction pair in
-// the item).  Its target sums (and a symmetric item's source sums) are added
-// into the handle's exact per-node accumulators.
+// sources [j_begin, j_end); one-sided (kItemOne: correction pairs masked),
+// symmetric (kItemSym: both orientations of every pair, no correction pair in
+// the item) or near symmetric (kItemNear: both orientations, each correction
+// pair left out of the rows that omit it).  Its target sums (and a symmetric item's
+// source sums) are added into the handle's exact per-node accumulators.
+enum : int32_t { kItemOne = 0, kItemSym = 1, kItemNear = 2 };
 struct PairItem {
     int32_t I, j_begin, j_end, sym;
 };
@@ -244,6 +246,7 @@ struct ctr_ibim {
     ctr::DevBuf corr_w;      // double [4][E]: omega11, omega21, omega22, omega12
     ctr::DevBuf bad;         // uint8 [M] hybrid classification
     ctr::DevBuf excl;        // int32 [E] sorted correction nodes per target
+    ctr::DevBuf cl_begin, cl_end, cl_list;   // int32: closed exclusion lists of direct handles (pk::Exclusions)
     ctr::DevBuf rhs;         // double [2M]
     ctr::DevBuf charges;     // double [4][nc]: x, y, z, q
     ctr::DevBuf acc;         // exact accumulators of the dense sum: pk::kFxWords x M 64-bit words

@@ -143,70 +143,53 @@ __global__ void __launch_bounds__(kThreads, Policy::kMinBlocks) k_pairs(SlotDev*
     pair_block_init<Policy>(exp_tab, sm.tab, bar);   // one table per device, shared by every slot
     uint32_t gt = 0;
     const int total = *n_items;
-    for (;;) {
-        if (threadIdx.x == 0) cur = atomicAdd(counter, 1);
-        __syncthreads();
-        const int it = cur;
-        __syncthreads();
-        if (it >= total) break;
+    for (int it = blockIdx.x; it < total;) {   // the first entries need no counter
         const int2 w = items[it];   // slot, item | part << kPartShift
         const SlotDev& s = S[w.x];
         const bool want = half == 0 ? (inner_active(s) && s.inner_prec == prec)
                                     : (update_active(s) && res_arith(s) == prec);
         const int pe = w.y >> kPartShift;
-        if (!want || pe < s.part || pe >= s.part + s.span) continue;
-        const int item = w.y & kItemMask;
-        const Src* src = reinterpret_cast<const Src*>(prec == CTR_FP32_REFINE ? (const void*)s.src32
-                                                      : prec == CTR_DF64 ? (const void*)s.srcdf
-                                                                         : (const void*)s.src64);
-        if constexpr (kShared) {
-            if (!run_item<Policy, R, V, U>(s.items[pol][item], src, s.M, s.eptr, s.excl, s.acc, pkc, err, sm.ring,
-                                           sm.jred, sm.tab, bar, gt))
-                return;
-        } else {
-            if (threadIdx.x == 0) kc = s.kc;
-            __syncthreads();
-            const PairConsts k = kc;   // block-uniform register copy: no shared loads in the pair loops
-            if (!run_item<Policy, R, V, U>(s.items[pol][item], src, s.M, s.eptr, s.excl, s.acc, k, err, sm.ring,
-                                           sm.jred, sm.tab, bar, gt))
-                return;
+        if (want && pe >= s.part && pe < s.part + s.span) {
+            const int item = w.y & kItemMask;
+            const Src* src = reinterpret_cast<const Src*>(prec == CTR_FP32_REFINE ? (const void*)s.src32
+                                                          : prec == CTR_DF64 ? (const void*)s.srcdf
+                                                                             : (const void*)s.src64);
+            if constexpr (kShared) {
+                if (!run_item<Policy, R, V, U>(s.items[pol][item], src, s.M, s.excl, s.acc, pkc, err, sm.ring,
+                                               sm.jred, sm.tab, bar, gt))
+                    return;
+            } else {
+                if (threadIdx.x == 0) kc = s.kc;
+                __syncthreads();
+                const PairConsts k = kc;   // block-uniform register copy: no shared loads in the pair loops
+                if (!run_item<Policy, R, V, U>(s.items[pol][item], src, s.M, s.excl, s.acc, k, err, sm.ring,
+                                               sm.jred, sm.tab, bar, gt))
+                    return;
+            }
         }
+        if (threadIdx.x == 0) cur = gridDim.x + atomicAdd(counter, 1);
+        __syncthreads();
+        it = cur;
         __syncthreads();
     }
 }
 
 // finish: diag + the node's accumulated dense sum (read and cleared) + correction of the applied vector;
 // inner: w = V_{j+1} = A z;   update: r = g - A x, or r = r - A d (residual update, d in z)
-__global__ void k_finish(SlotDev* S, int half) {
+__global__ void __launch_bounds__(kFinishThreads) k_finish(SlotDev* S, int half) {
     const SlotDev& s = S[blockIdx.y];
     if (half == 0 ? !inner_active(s) : !update_active(s)) return;
-    const int64_t M = s.M, E = s.E;
+    const int64_t M = s.M;
     const bool upd = (half == 1) && s.upd;
     const double* x = (half == 0 || upd) ? s.z : s.x;
     double* out = (half == 0) ? s.V + (size_t)(s.j + 1) * s.n : s.r;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M; i += (int64_t)gridDim.x * blockDim.x) {
-        double s1, s2;
-        fx_read(s.acc + (s.tinv ? (int64_t)s.tinv[i] : i), M, true, s1, s2);
-        double c1 = 0.0, c2 = 0.0;
-        for (int e = s.cptr[i]; e < s.cptr[i + 1]; ++e) {
-            const int m = s.cnode[e];
-            const double Wm = s.W[m], r1 = x[m], r2 = x[M + m];
-            c1 += Wm * (s.h2 * s.cw[e] * r1 - s.h3 * s.cw[3 * E + e] * r2);
-            c2 += Wm * (s.h2 * s.cw[E + e] * r1 - s.h2 * s.cw[2 * E + e] * r2);
-        }
-        const double y1 = s.lam1 * x[i] + s1 + c1;
-        const double y2 = s.lam2 * x[M + i] + s2 + c2;
-        if (half == 0) {
-            out[i] = y1;
-            out[M + i] = y2;
-        } else if (upd) {   // out is r: each thread updates its own two entries
-            out[i] -= y1;
-            out[M + i] -= y2;
-        } else {
-            out[i] = s.g[i] - y1;
-            out[M + i] = s.g[M + i] - y2;
-        }
-    }
+    finish_rows(s.fin, s.acc, s.tinv, x, [&](int64_t i, int c, double v) {
+        const int64_t q = (int64_t)c * M + i;
+        const double y = (c == 0 ? s.lam1 : s.lam2) * x[q] + v;
+        if (half == 0) out[q] = y;
+        else if (upd) out[q] -= y;   // out is r: each thread updates its own entry
+        else out[q] = s.g[q] - y;
+    });
 }
 
 // ---------------------------------------------------------------- batched reductions (same chunking as alone)
@@ -775,6 +758,7 @@ static int enqueue_step(Engine* e) {
     const int cap = e->cap;
     const int mx = e->max_nblk;
     const dim3 vec(e->vec_blocks, cap);
+    const dim3 rows(2 * e->vec_blocks, cap);   // half as many rows per block
     const unsigned one = grid_for(cap, 128);
     k_plan_step<<<1, kVecThreads, 0, st>>>(S, cap);
     CTR_LAUNCHED();
@@ -791,7 +775,7 @@ static int enqueue_step(Engine* e) {
     CTR_TRY(launch_trees(e, 0));
     k_part<<<one, 128, 0, st>>>(S, cap, 0);
     CTR_LAUNCHED();
-    k_finish<<<vec, kVecThreads, 0, st>>>(S, 0);
+    k_finish<<<rows, kFinishThreads, 0, st>>>(S, 0);
     CTR_LAUNCHED();
     for (int pass = 0; pass < 2; ++pass) {
         k_dots_partial<<<dim3(mx, cap), kVecThreads, 0, st>>>(S, pass);
@@ -824,7 +808,7 @@ static int enqueue_step(Engine* e) {
     CTR_TRY(launch_trees(e, 1));
     k_part<<<one, 128, 0, st>>>(S, cap, 1);
     CTR_LAUNCHED();
-    k_finish<<<vec, kVecThreads, 0, st>>>(S, 1);
+    k_finish<<<rows, kFinishThreads, 0, st>>>(S, 1);
     CTR_LAUNCHED();
     k_dots_partial<<<dim3(mx, cap), kVecThreads, 0, st>>>(S, 3);
     CTR_LAUNCHED();
@@ -878,15 +862,11 @@ int engine_admit(Engine* e, ctr_ibim* s, int* slot_out) {
     SlotDev d{};
     d.M = (int)s->M;
     d.n = 2 * s->M;
-    d.E = (int)s->E;
     d.m = s->kr.m;
     d.nblk = s->kr.nblk;
     d.W = s->na.W;
-    d.cptr = s->corr_ptr.as<int32_t>();
-    d.cnode = s->corr_node.as<int32_t>();
-    d.cw = s->corr_w.as<double>();
-    d.excl = s->tree ? s->tree->d_excl.as<int32_t>() : s->excl.as<int32_t>();
-    d.eptr = s->tree ? s->tree->d_eptr.as<int32_t>() : s->corr_ptr.as<int32_t>();
+    d.fin = finish_rows_of(s);
+    d.excl = exclusions_of(s);
     d.tinv = s->tree ? s->tree->d_tinv.as<int32_t>() : nullptr;
     if (s->tree) d.tv = s->tree->view;
     d.src32 = s->src32.as<float4>();
@@ -898,8 +878,6 @@ int engine_admit(Engine* e, ctr_ibim* s, int* slot_out) {
     d.lam2 = 0.5 * (1.0 + s->eps_in / s->eps_out);
     d.il1 = 2.0 / (1.0 + s->eps_out / s->eps_in);
     d.il2 = 2.0 / (1.0 + s->eps_in / s->eps_out);
-    d.h2 = s->h * s->h;
-    d.h3 = s->h * s->h * s->h;
     d.scale = s->h * s->h * s->h / (4.0 * kPi);
     d.refine = (s->opt.precision == CTR_FP32_REFINE) ? 1 : 0;
     d.inner_prec = s->opt.precision;

@@ -35,7 +35,7 @@ struct SlotStat {
 struct SlotDev {
     SlotStat stat;
     int j, m, kdone, cycle_end;
-    int M, E, nblk;
+    int M, nblk;
     int64_t n;
     int refine, inner_prec, res_prec, max_refine;
     int res_update;          // refinement residuals after the first: r -= A d in the inner arithmetic
@@ -47,18 +47,15 @@ struct SlotDev {
     int64_t budget;
     // system (owned by the handle)
     const double* W;
-    const int32_t* cptr;
-    const int32_t* cnode;
-    const double* cw;
-    const int32_t* excl;     // excluded sources of each target, in the order of the packed sources
-    const int32_t* eptr;     // ... and their row pointers (cptr, or the treecode's tree-order lists)
+    pk::FinishRows fin;      // correction rows
+    pk::Exclusions excl;     // sources left out, in the order of the packed sources
     const int32_t* tinv;     // treecode: node -> tree position of the packed sources (else NULL)
     float4* src32;
     double4* src64;
     float4* srcdf;
     unsigned long long* acc;   // exact node accumulators of the dense sum
     const double* g;
-    double lam1, lam2, il1, il2, h2, h3, scale;
+    double lam1, lam2, il1, il2, scale;
     pk::PairConsts kc;
     // pair schedules of the three arithmetics ([0] FP32, [1] float-float, [2] FP64; owned by the handle)
     const PairItem* items[3];

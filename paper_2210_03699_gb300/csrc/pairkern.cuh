@@ -16,6 +16,9 @@ constexpr int kExpLo = 1024;    // e^{-k/1024}, k = 0..1023
 constexpr int kExp2 = 1024;     // FP64 tables: 2^{-k/1024} (double), then its relative rounding error (float)
 constexpr int kExp2F2 = kExp2 + kExp2 / 2;   // their size in float2
 
+// Flags of an excluded pair (Exclusions): the source is left out of the target's row, the target of the source's
+enum : int { kOutTarget = 1, kOutSource = 2 };
+
 struct PairConsts {
     float c1f, c2f, kappaf, kl2f;    // eps_E/eps_I, eps_I/eps_E, kappa, -kappa log2(e)
     double c1, c2, kappa;
@@ -343,6 +346,18 @@ __device__ __forceinline__ void fx_add(unsigned long long* __restrict__ acc, int
 // positive minus negative, one rounding.  The node's words of that sum are cleared when `clear`.
 __device__ __forceinline__ double fx_read_one(unsigned long long* __restrict__ acc, int64_t stride, int c,
                                               bool clear) {
+    unsigned long long wp[kFxChunks], wn[kFxChunks];   // every load in flight before the first use
+    unsigned long long* ap = acc + (int64_t)(2 * c) * kFxChunks * stride;
+    unsigned long long* an = ap + (int64_t)kFxChunks * stride;
+#pragma unroll
+    for (int k = 0; k < kFxChunks; ++k) {
+        wp[k] = ap[(int64_t)k * stride];
+        wn[k] = an[(int64_t)k * stride];
+    }
+    if (clear) {
+#pragma unroll
+        for (int k = 0; k < kFxChunks; ++k) ap[(int64_t)k * stride] = an[(int64_t)k * stride] = 0ull;
+    }
     uint32_t D[kFxChunks + 1];
     unsigned long long cp = 0, cn = 0;
     long long borrow = 0;
@@ -350,11 +365,8 @@ __device__ __forceinline__ double fx_read_one(unsigned long long* __restrict__ a
     for (int k = 0; k <= kFxChunks; ++k) {
         unsigned long long tp = cp, tn = cn;
         if (k < kFxChunks) {
-            unsigned long long* ap = acc + (int64_t)((2 * c) * kFxChunks + k) * stride;
-            unsigned long long* an = acc + (int64_t)((2 * c + 1) * kFxChunks + k) * stride;
-            tp += *ap;
-            tn += *an;
-            if (clear) *ap = *an = 0ull;
+            tp += wp[k];
+            tn += wn[k];
         }
         cp = tp >> 32;
         cn = tn >> 32;
@@ -379,16 +391,73 @@ __device__ __forceinline__ double fx_read_one(unsigned long long* __restrict__ a
     return neg ? -v : v;
 }
 
-// Both sums of the node at acc (NaN when a contribution was marked); clears the node's words when `clear`.
-__device__ __forceinline__ void fx_read(unsigned long long* __restrict__ acc, int64_t stride, bool clear, double& s1,
-                                        double& s2) {
-    unsigned long long* mark = acc + (int64_t)(4 * kFxChunks) * stride;
-    const bool bad = *mark != 0ull;
-    s1 = fx_read_one(acc, stride, 0, clear);
-    s2 = fx_read_one(acc, stride, 1, clear);
-    if (clear) *mark = 0ull;
-    if (bad) s1 = s2 = __longlong_as_double(0x7ff8000000000000ll);
+// ------------------------------------------------------------------ finishing a row
+// What the finishing kernels need besides the accumulated sum: the correction rows (CSR, weights omega11,
+// omega21, omega22, omega12 of E entries each).
+struct FinishRows {
+    const int32_t* ptr;
+    const int32_t* node;
+    const double* w;
+    const double* W;
+    int64_t M, E;
+    double h2, h3;
+};
+
+// Component c (0: omega11, omega12; 1: omega21, omega22) of row i applied to x, without the diagonal:
+// accumulated sum (read and cleared) + correction.  NaN when a contribution was marked (`bad`).
+__device__ __forceinline__ double finish_row(const FinishRows& f, unsigned long long* __restrict__ acc,
+                                             int64_t pos, int64_t i, int c, const double* __restrict__ x, bool bad) {
+    const int64_t M = f.M, E = f.E;
+    const int e0 = f.ptr[i], e1 = f.ptr[i + 1];
+    const double* wa = f.w + (c == 0 ? 0 : E);
+    const double* wb = f.w + (c == 0 ? 3 : 2) * E;
+    const double hb = c == 0 ? f.h3 : f.h2;
+    const double s = fx_read_one(acc + pos, M, c, true);
+    double v = 0.0;
+    for (int e = e0; e < e1; e += 4) {   // four entries (a row has about four) with their gathers in flight
+        int m[4];
+        double a[4], b[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int q = min(e + k, e1 - 1);
+            m[k] = f.node[q];
+            a[k] = wa[q];
+            b[k] = wb[q];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const double t = f.W[m[k]] * (f.h2 * a[k] * x[m[k]] - hb * b[k] * x[M + m[k]]);
+            if (e + k < e1) v += t;
+        }
+    }
+    return bad ? __longlong_as_double(0x7ff8000000000000ll) : s + v;
 }
+
+// The rows of a finishing kernel: a block of kFinishThreads takes kFinishRows rows, the two components of a
+// row in different warps (half the serial chain of one thread per row, and twice the threads for the small
+// systems, where the chain's latency is the whole kernel: 15 -> 9 us at 3 214 nodes, 74 -> 40 us at 178 575).
+// put(i, c, value) receives the results.
+constexpr int kFinishThreads = 256, kFinishRows = kFinishThreads / 2;
+template <typename Put>
+__device__ __forceinline__ void finish_rows(const FinishRows& f, unsigned long long* __restrict__ acc,
+                                            const int32_t* __restrict__ tinv, const double* __restrict__ x,
+                                            const Put& put) {
+    const int c = threadIdx.x / kFinishRows, at = threadIdx.x % kFinishRows;
+    for (int64_t base = (int64_t)blockIdx.x * kFinishRows; base < f.M; base += (int64_t)gridDim.x * kFinishRows) {
+        const int64_t i = base + at;
+        bool bad = false;
+        unsigned long long* mark = nullptr;
+        if (i < f.M) {
+            const int64_t pos = tinv ? (int64_t)tinv[i] : i;
+            mark = acc + (int64_t)(4 * kFxChunks) * f.M + pos;
+            bad = *mark != 0ull;
+            put(i, c, finish_row(f, acc, pos, i, c, x, bad));
+        }
+        __syncthreads();   // both components have read the mark
+        if (bad && c == 0) *mark = 0ull;
+    }
+}
+
 
 // ------------------------------------------------------------------ pair policies
 // Fp32: 4 pi K terms, d = x - y, s = 1/r^3, E = e^{-kappa r}, E1 = E (1 + kappa r):
@@ -484,6 +553,7 @@ struct Fp32x2Policy {
     static constexpr bool kRenorm = false;   // running sums need no renormalisation
     static constexpr bool kStepTranspose = false;
     static constexpr int kSymStep = 32;
+    static constexpr int kNearStep = 4;   // sources per transposed step of a near symmetric item
     static constexpr int kPack = 2;
     struct Tgt {
         u64 px, py, pz, qx, qy, qz, nwa, nwb;
@@ -541,13 +611,34 @@ struct Fp32x2Policy {
     __device__ static JAcc jshfl_xor(const JAcc& x, int m) {
         return JAcc{__shfl_xor_sync(0xffffffffu, x.a1, m), __shfl_xor_sync(0xffffffffu, x.a2, m)};
     }
-    // The terms shared by both orientations for the two targets of T and source S.
+    struct Node {
+        u64 x, y, z, nx, ny, nz, a, nb;
+    };
+    __device__ static Node node(const Src* S) {
+        const ulonglong2 v0 = S[0], v1 = S[1], v2 = S[2], v3 = S[3];
+        return Node{v0.x, v0.y, v1.x, v2.x, v2.y, v3.x, v1.y, v3.y};
+    }
+    // The halves of `other` where excluded, else of `mine`.
+    __device__ static u64 pick(const bool* ex, u64 mine, u64 other) {
+        float m0, m1, o0, o1;
+        up2(mine, m0, m1);
+        up2(other, o0, o1);
+        return pk2(ex[0] ? o0 : m0, ex[1] ? o1 : m1);
+    }
+    // Excluded pairs (per half): a zero-weight source at distance 1 of the target.
+    __device__ static void exclude(const Tgt& T, Node& q, const bool* ex, u64 one2) {
+        q.x = pick(ex, q.x, add2(T.px, one2));
+        q.y = pick(ex, q.y, T.py);
+        q.z = pick(ex, q.z, T.pz);
+        q.a = pick(ex, q.a, 0ull);
+        q.nb = pick(ex, q.nb, 0ull);
+    }
+    // The terms shared by both orientations for the two targets of T and source q.
     struct Common {
         u64 dnx, dny, om, t1, t2n, X, s;
     };
-    __device__ static Common common(const Tgt& T, u64 Sx, u64 Sy, u64 Sz, u64 Nx, u64 Ny, u64 Nz,
-                                    const PairConsts& k) {
-        const u64 dx = sub2(T.px, Sx), dy = sub2(T.py, Sy), dz = sub2(T.pz, Sz);
+    __device__ static Common common(const Tgt& T, const Node& q, const PairConsts& k) {
+        const u64 dx = sub2(T.px, q.x), dy = sub2(T.py, q.y), dz = sub2(T.pz, q.z);
         const u64 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
         const u64 rinv = rsqrt2(r2);
         const u64 r = mul2(r2, rinv);
@@ -555,17 +646,17 @@ struct Fp32x2Policy {
         const u64 kr = mul2(k.kap2, r);
         const u64 E1 = fma2(E, kr, E);
         Common c;
-        c.dny = fma2(dz, Nz, fma2(dy, Ny, mul2(dx, Nx)));
+        c.dny = fma2(dz, q.nz, fma2(dy, q.ny, mul2(dx, q.nx)));
         c.dnx = fma2(dz, T.qz, fma2(dy, T.qy, mul2(dx, T.qx)));
-        const u64 nn = fma2(T.qz, Nz, fma2(T.qy, Ny, mul2(T.qx, Nx)));
+        const u64 nn = fma2(T.qz, q.nz, fma2(T.qy, q.ny, mul2(T.qx, q.nx)));
         const u64 rinv2 = mul2(rinv, rinv);
         c.s = mul2(rinv2, rinv);
         c.t1 = fma2(k.nc1x2, E1, k.one2);
         c.t2n = fma2(k.c2x2, E1, k.mone2);
         c.om = mul2(rinv, sub2(k.one2, E));
         const u64 u = sub2(k.one2, E1);
-        const u64 q = fma2(kr, add2(kr, k.three2), k.three2);
-        const u64 t3n = fma2(E, q, k.mthree2);
+        const u64 p = fma2(kr, add2(kr, k.three2), k.three2);
+        const u64 t3n = fma2(E, p, k.mthree2);
         const u64 Bn = mul2(mul2(mul2(t3n, c.dnx), c.dny), rinv2);
         c.X = fma2(u, nn, Bn);
         return c;
@@ -580,58 +671,47 @@ struct Fp32x2Policy {
     template <bool kMask>
     __device__ static void pair(const Tgt& T, const Src* S, const PairConsts& k, const float2*, Acc& acc,
                                 const bool* ex) {
-        const ulonglong2 v0 = S[0], v1 = S[1], v2 = S[2], v3 = S[3];
-        u64 Sx = v0.x, Sy = v0.y, Sz = v1.x, Sa = v1.y, Snb = v3.y;
-        if (kMask && (ex[0] || ex[1])) {   // excluded correction pair: a zero-weight source at distance 1
-            float x[2], y[2], z[2], a[2], b[2], tx[2], ty[2], tz[2];
-            up2(Sx, x[0], x[1]);
-            up2(Sy, y[0], y[1]);
-            up2(Sz, z[0], z[1]);
-            up2(Sa, a[0], a[1]);
-            up2(Snb, b[0], b[1]);
-            up2(T.px, tx[0], tx[1]);
-            up2(T.py, ty[0], ty[1]);
-            up2(T.pz, tz[0], tz[1]);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                if (ex[h]) {
-                    x[h] = tx[h] + 1.f;
-                    y[h] = ty[h];
-                    z[h] = tz[h];
-                    a[h] = b[h] = 0.f;
-                }
-            }
-            Sx = pk2(x[0], x[1]);
-            Sy = pk2(y[0], y[1]);
-            Sz = pk2(z[0], z[1]);
-            Sa = pk2(a[0], a[1]);
-            Snb = pk2(b[0], b[1]);
-        }
-        const Common c = common(T, Sx, Sy, Sz, v2.x, v2.y, v3.x, k);
-        target_terms(c, Sa, Snb, acc);
+        Node q = node(S);
+        if (kMask && (ex[0] || ex[1])) exclude(T, q, ex, k.one2);
+        target_terms(common(T, q, k), q.a, q.nb, acc);
     }
     // Both orientations: s is folded once into the factors the two share (s t1, s t2n, s X), which
     // saves one f32x2 operation per pair against forming a s, b s and the targets' (-a) s, (-b) s.
-    template <bool kFirst>
+    // kMask: flags per half (Exclusions); a pair left out of both rows is moved to distance 1 (no NaN).
+    template <bool kFirst, bool kMask = false>
     __device__ static void pair_sym(const Tgt& T, const Src* S, const PairConsts& k, const float2*, Acc& acc,
-                                    JAccR& ja) {
-        const ulonglong2 v0 = S[0], v1 = S[1], v2 = S[2], v3 = S[3];
-        const Common c = common(T, v0.x, v0.y, v1.x, v2.x, v2.y, v3.x, k);
-        const u64 st1 = mul2(c.s, c.t1), st2n = mul2(c.s, c.t2n), sX = mul2(c.s, c.X);
-        const u64 Sa = v1.y, Snb = v3.y;
-        acc.a1 = fma2(mul2(Sa, c.dny), st1, acc.a1);
-        acc.a1 = fma2(Snb, c.om, acc.a1);
-        acc.a2 = fma2(mul2(Snb, c.dnx), st2n, acc.a2);
-        acc.a2 = fma2(Sa, sX, acc.a2);
-        if constexpr (kFirst) {
-            ja.a1 = mul2(mul2(T.nwa, c.dnx), st1);
-            ja.a2 = mul2(mul2(T.nwb, c.dny), st2n);   // ja.a2 holds -a2 until jfinal
-        } else {
-            ja.a1 = fma2(mul2(T.nwa, c.dnx), st1, ja.a1);
-            ja.a2 = fma2(mul2(T.nwb, c.dny), st2n, ja.a2);
+                                    JAccR& ja, const int* ex = nullptr) {
+        Node q = node(S);
+        u64 nwa = T.nwa, nwb = T.nwb;
+        if constexpr (kMask) {
+            if (ex[0] | ex[1]) {
+                const bool both[2] = {ex[0] == 3, ex[1] == 3};
+                const bool out_t[2] = {(ex[0] & kOutTarget) != 0, (ex[1] & kOutTarget) != 0};
+                const bool out_s[2] = {(ex[0] & kOutSource) != 0, (ex[1] & kOutSource) != 0};
+                q.x = pick(both, q.x, add2(T.px, k.one2));
+                q.y = pick(both, q.y, T.py);
+                q.z = pick(both, q.z, T.pz);
+                q.a = pick(out_t, q.a, 0ull);
+                q.nb = pick(out_t, q.nb, 0ull);
+                nwa = pick(out_s, nwa, 0ull);
+                nwb = pick(out_s, nwb, 0ull);
+            }
         }
-        ja.a1 = fma2(T.nwb, c.om, ja.a1);
-        ja.a2 = fma2(T.nwa, sX, ja.a2);
+        const Common c = common(T, q, k);
+        const u64 st1 = mul2(c.s, c.t1), st2n = mul2(c.s, c.t2n), sX = mul2(c.s, c.X);
+        acc.a1 = fma2(mul2(q.a, c.dny), st1, acc.a1);
+        acc.a1 = fma2(q.nb, c.om, acc.a1);
+        acc.a2 = fma2(mul2(q.nb, c.dnx), st2n, acc.a2);
+        acc.a2 = fma2(q.a, sX, acc.a2);
+        if constexpr (kFirst) {
+            ja.a1 = mul2(mul2(nwa, c.dnx), st1);
+            ja.a2 = mul2(mul2(nwb, c.dny), st2n);   // ja.a2 holds -a2 until jfinal
+        } else {
+            ja.a1 = fma2(mul2(nwa, c.dnx), st1, ja.a1);
+            ja.a2 = fma2(mul2(nwb, c.dny), st2n, ja.a2);
+        }
+        ja.a1 = fma2(nwb, c.om, ja.a1);
+        ja.a2 = fma2(nwa, sX, ja.a2);
     }
 };
 
@@ -644,6 +724,7 @@ struct Fp64Policy {
     static constexpr bool kRenorm = false;   // running sums need no renormalisation
     static constexpr bool kStepTranspose = false;
     static constexpr int kSymStep = 4;
+    static constexpr int kNearStep = 2;
     struct Tgt {
         double px, py, pz, qx, qy, qz, wa, wb;
     };
@@ -705,31 +786,39 @@ struct Fp64Policy {
         acc.a2 = fma(b, c.dnx * c.st2, acc.a2);
         acc.a2 = fma(a, c.sX, acc.a2);
     }
-    template <bool kFirst>
+    // kMask: flags (Exclusions); a pair left out of both rows is moved to distance 1 (no NaN).
+    template <bool kFirst, bool kMask = false>
     __device__ static void pair_sym(const Tgt& T, const Src* S, const PairConsts& k, const float2* tab, Acc& acc,
-                                    JAcc& ja) {
-        const double4 pa = S[0], nb = S[1];
+                                    JAcc& ja, const int* ex = nullptr) {
+        double4 pa = S[0], nb = S[1];
+        double wa = T.wa, wb = T.wb;
+        if constexpr (kMask) {
+            if (*ex == 3) exclude(T, pa, nb);
+            if (*ex & kOutTarget) pa.w = nb.w = 0.0;
+            if (*ex & kOutSource) wa = wb = 0.0;
+        }
         const Common c = common(T, pa, nb, k, tab);
         target_terms(c, pa.w, nb.w, acc);
         const double x1 = c.dnx * c.st1, y2 = c.dny * c.st2;
         if constexpr (kFirst) {
-            ja.a1 = -T.wa * x1;
-            ja.a2 = -T.wb * y2;
+            ja.a1 = -wa * x1;
+            ja.a2 = -wb * y2;
         } else {
-            ja.a1 = fma(-T.wa, x1, ja.a1);
-            ja.a2 = fma(-T.wb, y2, ja.a2);
+            ja.a1 = fma(-wa, x1, ja.a1);
+            ja.a2 = fma(-wb, y2, ja.a2);
         }
-        ja.a1 = fma(-T.wb, c.om, ja.a1);
-        ja.a2 = fma(T.wa, c.sX, ja.a2);
+        ja.a1 = fma(-wb, c.om, ja.a1);
+        ja.a2 = fma(wa, c.sX, ja.a2);
+    }
+    __device__ static void exclude(const Tgt& T, double4& pa, double4& nb) {
+        pa = make_double4(T.px + 1.0, T.py, T.pz, 0.0);
+        nb.w = 0.0;
     }
     template <bool kMask>
     __device__ static void pair(const Tgt& T, const Src* S, const PairConsts& k, const float2* tab, Acc& acc,
                                 const bool* exv) {
         double4 pa = S[0], nb = S[1];
-        if (kMask && exv[0]) {   // excluded correction pair: a zero-weight source at distance 1
-            pa = make_double4(T.px + 1.0, T.py, T.pz, 0.0);
-            nb.w = 0.0;
-        }
+        if (kMask && exv[0]) exclude(T, pa, nb);
         target_terms(common(T, pa, nb, k, tab), pa.w, nb.w, acc);
     }
 };
@@ -756,6 +845,7 @@ struct Df64Policy {
     static constexpr bool kRenorm = true;
     static constexpr bool kStepTranspose = true;   // each step's sources are transposed on their own
     static constexpr int kSymStep = 4;
+    static constexpr int kNearStep = 2;
     struct Tgt {
         F2 px, py, pz, qx, qy, qz, wa, wb;
     };
@@ -842,30 +932,38 @@ struct Df64Policy {
     __device__ static void pair(const Tgt& T, const Src* S, const PairConsts& k, const float2* tab, Acc& acc,
                                 const bool* exv) {
         Node q = node(S);
-        if (kMask && exv[0]) {   // excluded correction pair: a zero-weight source at distance 1
-            q.x = F2{T.px.hi + 1.f, T.px.lo};
-            q.y = T.py;
-            q.z = T.pz;
-            q.a = q.b = F2{0.f, 0.f};
-        }
+        if (kMask && exv[0]) exclude(T, q);
         target_terms(common(T, q, k, tab), q.a, q.b, acc);
     }
-    template <bool kFirst>
+    __device__ static void exclude(const Tgt& T, Node& q) {   // a zero-weight source at distance 1
+        q.x = F2{T.px.hi + 1.f, T.px.lo};
+        q.y = T.py;
+        q.z = T.pz;
+        q.a = q.b = F2{0.f, 0.f};
+    }
+    // kMask: flags (Exclusions); a pair left out of both rows is moved to distance 1 (no NaN).
+    template <bool kFirst, bool kMask = false>
     __device__ static void pair_sym(const Tgt& T, const Src* S, const PairConsts& k, const float2* tab, Acc& acc,
-                                    JAcc& ja) {
-        const Node q = node(S);
+                                    JAcc& ja, const int* ex = nullptr) {
+        Node q = node(S);
+        F2 wa = T.wa, wb = T.wb;
+        if constexpr (kMask) {
+            if (*ex == 3) exclude(T, q);
+            if (*ex & kOutTarget) q.a = q.b = F2{0.f, 0.f};
+            if (*ex & kOutSource) wa = wb = F2{0.f, 0.f};
+        }
         const Common c = common(T, q, k, tab);
         target_terms(c, q.a, q.b, acc);
         const F2 x1 = mull(c.dnx, c.st1), y2 = mull(c.dny, c.st2);
         if constexpr (kFirst) {
-            ja.a1 = neg(mull(T.wa, x1));
-            ja.a2 = neg(mull(T.wb, y2));
+            ja.a1 = neg(mull(wa, x1));
+            ja.a2 = neg(mull(wb, y2));
         } else {
-            acc_mul(ja.a1, neg(T.wa), x1);
-            acc_mul(ja.a2, neg(T.wb), y2);
+            acc_mul(ja.a1, neg(wa), x1);
+            acc_mul(ja.a2, neg(wb), y2);
         }
-        acc_mul(ja.a1, neg(T.wb), c.om);
-        acc_mul(ja.a2, T.wa, c.sX);
+        acc_mul(ja.a1, neg(wb), c.om);
+        acc_mul(ja.a2, wa, c.sX);
     }
 };
 
@@ -906,6 +1004,44 @@ struct FxOut {
     }
 };
 
+// What the items leave out, by target position i, ascending.
+//   own: the correction nodes N(i), own_list[own_begin[i] .. own_begin[i + 1]): the one-sided items' masks.
+//   closed: every node j with j in N(i) or i in N(j), as 4 j + flags (kOutTarget: j is left out of row i,
+//   kOutSource: i is left out of row j), list[begin[i] .. end[i]): the near symmetric items' masks (direct
+//   handles; NULL for treecode handles, which have no such items).
+struct Exclusions {
+    const int32_t* own_begin;
+    const int32_t* own_list;
+    const int32_t* begin;
+    const int32_t* end;
+    const int32_t* list;
+};
+
+// The first two entries of the ascending list[b .. e) that are >= j (INT_MAX where there is none) and the
+// first one's position; eight entries (few lists are longer) are read at a time, their latencies overlapping.
+__device__ __forceinline__ void first_excluded(const int32_t* __restrict__ list, int b, int e, int j, int& pos,
+                                               int& next, int& after) {
+    pos = b;
+    next = after = INT_MAX;
+    while (pos < e) {
+        int v[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) v[k] = pos + k < e ? list[pos + k] : INT_MAX;
+        int below = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) below += v[k] < j;
+#pragma unroll
+        for (int k = 7; k >= 0; --k) {
+            if (v[k] >= j) {
+                after = v[k + 1];
+                next = v[k];
+            }
+        }
+        pos += below;
+        if (below < 8) break;
+    }
+}
+
 // One one-sided work item of the dense pair sum: target block `tblock`
 // (kThreads * R targets) against sources [j_begin, j_end), with the correction
 // pairs masked; the sums of target i go to `out` (RegionOut or FxOut).
@@ -915,8 +1051,7 @@ struct FxOut {
 // set; the caller must return).
 template <typename Policy, int R, int U = 2, typename Out = FxOut>
 __device__ __forceinline__ bool pair_item(const typename Policy::Src* __restrict__ src, int M,
-                                          const int32_t* __restrict__ eptr, const int32_t* __restrict__ excl,
-                                          int tblock, int j_begin, int j_end, const Out& out,
+                                          const Exclusions& cl, int tblock, int j_begin, int j_end, const Out& out,
                                           const PairConsts& kc,
                                           int* __restrict__ err, typename Policy::Src* ring, const float2* tab,
                                           uint64_t* bar, uint32_t& gt) {
@@ -930,18 +1065,15 @@ __device__ __forceinline__ bool pair_item(const typename Policy::Src* __restrict
 
     typename Policy::Tgt tg[R];
     double s1[RP], s2[RP];
-    int ti[RP], epos[RP], eend[RP], enext[RP];
+    int ti[RP], epos[RP], eend[RP], enext[RP], eafter[RP];   // the entry after the next one is read ahead
 #pragma unroll
     for (int a = 0; a < RP; ++a) {
         ti[a] = tblock * (kThreads * RP) + a * kThreads + tid;
         const int t = min(ti[a], M - 1);
         s1[a] = 0.0;
         s2[a] = 0.0;
-        int e = eptr[t], ee = eptr[t + 1];
-        while (e < ee && excl[e] < j_begin) ++e;
-        epos[a] = e;
-        eend[a] = ee;
-        enext[a] = (e < ee) ? excl[e] : INT_MAX;
+        eend[a] = cl.own_begin[t + 1];
+        first_excluded(cl.own_list, cl.own_begin[t], eend[a], j_begin, epos[a], enext[a], eafter[a]);
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) tg[r] = load_targets<Policy>(src, M, &ti[r * P]);
@@ -1002,7 +1134,8 @@ __device__ __forceinline__ bool pair_item(const typename Policy::Src* __restrict
                         ex[h] = (j == enext[a]);
                         if (ex[h]) {
                             ++epos[a];
-                            enext[a] = (epos[a] < eend[a]) ? excl[epos[a]] : INT_MAX;
+                            enext[a] = eafter[a];
+                            eafter[a] = (epos[a] + 1 < eend[a]) ? cl.own_list[epos[a] + 1] : INT_MAX;
                         }
                     }
                     Policy::template pair<true>(tg[r], tile + q * VEC, kc, tab, acc[r], ex);
@@ -1234,21 +1367,145 @@ __device__ __forceinline__ bool pair_item_sym(const typename Policy::Src* __rest
     return true;
 }
 
+// One symmetric work item with correction pairs among its pairs: as pair_item_sym, but an excluded pair adds
+// nothing to the row(s) that leave it out.  A target is compared with its next excluded node at every source;
+// kNearStep sources are transposed at a time, which keeps the code short (a few per cent of the pairs of a
+// large system come here, most of a small one's).
+template <typename Policy, int R>
+__device__ __forceinline__ bool pair_item_near(const typename Policy::Src* __restrict__ src, int M, const Exclusions& cl,
+                                               int tblock, int j_begin, int j_end, const FxOut& out,
+                                               const PairConsts& kc, int* __restrict__ err, typename Policy::Src* ring,
+                                               typename Policy::JAcc* jred, const float2* tab, uint64_t* bar,
+                                               uint32_t& gt) {
+    using Src = typename Policy::Src;
+    using J = typename Policy::JAcc;
+    constexpr int TILE = Policy::kTile;
+    constexpr int VEC = Policy::kVec;
+    constexpr int P = Policy::kPack;
+    constexpr int RP = R * P;
+    constexpr int BS = kThreads * RP;
+    constexpr int kWarps = kThreads / 32;
+    constexpr int S = Policy::kNearStep;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int ntiles = (j_end - j_begin + TILE - 1) / TILE;
+
+    typename Policy::Tgt tg[R];
+    double s1[RP], s2[RP];
+    int ti[RP], epos[RP], eend[RP], enext[RP], eafter[RP];
+#pragma unroll
+    for (int a = 0; a < RP; ++a) {
+        ti[a] = tblock * BS + a * kThreads + tid;
+        s1[a] = 0.0;
+        s2[a] = 0.0;
+        const int t = min(ti[a], M - 1);
+        eend[a] = cl.end[t];
+        first_excluded(cl.list, cl.begin[t], eend[a], 4 * j_begin, epos[a], enext[a], eafter[a]);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) tg[r] = load_targets<Policy>(src, M, &ti[r * P]);
+    auto issue = [&](int k) {
+        const uint32_t g = gt + (uint32_t)k;
+        const int j0 = j_begin + k * TILE;
+        const int n = min(TILE, j_end - j0);
+        const uint32_t bytes = (uint32_t)(n * VEC * sizeof(Src));
+        Src* dst = ring + (g & 1) * TILE * VEC;
+        fence_proxy_async();
+        mbar_expect_tx(&bar[g & 1], bytes);
+        bulk_load(dst, src + (size_t)VEC * j0, bytes, &bar[g & 1]);
+    };
+    if (tid == 0 && ntiles > 0) issue(0);
+
+    for (int k = 0; k < ntiles; ++k) {
+        const uint32_t g = gt + (uint32_t)k;
+        if (tid == 0 && k + 1 < ntiles) issue(k + 1);
+        const bool ok = mbar_wait(&bar[g & 1], (g >> 1) & 1, kc.wait_limit);
+        if (__syncthreads_or(!ok)) {
+            if (tid == 0) {   // as in pair_item: flag, drain both copies in flight, return
+                atomicOr(err, kErrWait);
+                (void)mbar_wait(&bar[g & 1], (g >> 1) & 1);
+                if (k + 1 < ntiles) (void)mbar_wait(&bar[(g + 1) & 1], ((g + 1) >> 1) & 1);
+            }
+            return false;
+        }
+        const Src* tile = ring + (g & 1) * TILE * VEC;
+        const int j0 = j_begin + k * TILE;
+        const int n = min(TILE, j_end - j0);
+        typename Policy::Acc acc[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) Policy::zero(acc[r]);
+#pragma unroll 1
+        for (int c0 = 0; c0 < n; c0 += S) {
+            J cur[S];
+#pragma unroll
+            for (int t = 0; t < S; ++t) {
+                Policy::zero(cur[t]);
+                const int q = c0 + t;
+                if (q < n) {   // warp-uniform
+                    typename Policy::JAccR jr;
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        int ex[P];
+#pragma unroll
+                        for (int h = 0; h < P; ++h) {
+                            const int a = r * P + h;
+                            ex[h] = 0;
+                            if (j0 + q == enext[a] >> 2) {
+                                ex[h] = enext[a] & 3;
+                                ++epos[a];
+                                enext[a] = eafter[a];
+                                eafter[a] = (epos[a] + 1 < eend[a]) ? cl.list[epos[a] + 1] : INT_MAX;
+                            }
+                        }
+                        if (r == 0) Policy::template pair_sym<true, true>(tg[r], tile + q * VEC, kc, tab, acc[r], jr, ex);
+                        else Policy::template pair_sym<false, true>(tg[r], tile + q * VEC, kc, tab, acc[r], jr, ex);
+                    }
+                    cur[t] = Policy::jfinal(jr);
+                }
+            }
+            if constexpr (Policy::kRenorm) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) Policy::renorm(acc[r]);
+            }
+            transpose_sum<Policy, S>(cur, lane);
+            const int qs = c0 + lane / (32 / S);
+            if (lane % (32 / S) == 0 && qs < n) jred[warp * TILE + qs] = cur[0];
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) fold_targets<Policy>(acc[r], &s1[r * P], &s2[r * P]);
+        __syncthreads();   // all warp sums of this tile are in jred
+        if (tid < n) {
+            J t = jred[tid];
+#pragma unroll
+            for (int w = 1; w < kWarps; ++w) t = Policy::jadd(t, jred[w * TILE + tid]);
+            double d1 = 0.0, d2 = 0.0;
+            Policy::fold(t, d1, d2);
+            out.put(j0 + tid, d1, d2);
+        }
+        __syncthreads();   // jred and the buffer of this tile are free again
+    }
+    gt += (uint32_t)ntiles;
+#pragma unroll
+    for (int a = 0; a < RP; ++a)
+        if (ti[a] < M) out.put(ti[a], s1[a], s2[a]);
+    return true;
+}
+
 // Runs one item of a schedule (dispatch on its kind); its sums go into the nodes' exact accumulators
 // (acc, M words per accumulator word, fx_add).
 template <typename Policy, int R, int V, int U>
 __device__ __forceinline__ bool run_item(const PairItem& it, const typename Policy::Src* __restrict__ src, int M,
-                                         const int32_t* __restrict__ eptr, const int32_t* __restrict__ excl,
-                                         unsigned long long* __restrict__ acc, const PairConsts& kc,
-                                         int* __restrict__ err, typename Policy::Src* ring,
+                                         const Exclusions& cl, unsigned long long* __restrict__ acc,
+                                         const PairConsts& kc, int* __restrict__ err, typename Policy::Src* ring,
                                          typename Policy::JAcc* jred, const float2* tab, uint64_t* bar,
                                          uint32_t& gt) {
     constexpr int S = Policy::kSymStep < V ? Policy::kSymStep : V;
     const FxOut out{acc, (int64_t)M};
-    if (it.sym)
+    if (it.sym == kItemNear)
+        return pair_item_near<Policy, R>(src, M, cl, it.I, it.j_begin, it.j_end, out, kc, err, ring, jred, tab, bar, gt);
+    if (it.sym == kItemSym)
         return pair_item_sym<Policy, R, V, U, S>(src, M, it.I, it.j_begin, it.j_end, out, kc, err, ring, jred, tab,
                                                  bar, gt);
-    return pair_item<Policy, R, U>(src, M, eptr, excl, it.I, it.j_begin, it.j_end, out, kc, err, ring, tab, bar, gt);
+    return pair_item<Policy, R, U>(src, M, cl, it.I, it.j_begin, it.j_end, out, kc, err, ring, tab, bar, gt);
 }
 
 // Shared-memory bytes of a pair block: the two-stage source ring, the warp
@@ -1341,6 +1598,10 @@ __device__ __forceinline__ float2 split_ff_dev(double v) {
 // Exponential tables of pair arithmetic pol on a device: 1 the float-float e^{-k} (k < 64) and e^{-k/1024}
 // (k < 1024), 2 the FP64 2^{-k/1024} and their relative rounding errors (k < 1024), 0 none (NULL)
 int exp_table(int device, int pol, const float2** out);
+// What a handle's pair items leave out
+pk::Exclusions exclusions_of(const ctr_ibim* s);
+// The finishing kernels' view of a handle's rows
+pk::FinishRows finish_rows_of(const ctr_ibim* s);
 // Splits of the source range for equal-work items filling whole waves of `slots` resident blocks
 // (one-sided grid launch of the fixed-scratch entry point)
 PairPlan make_plan(int64_t M, int R, int tile, int slots);

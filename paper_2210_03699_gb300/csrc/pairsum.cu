@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(kThreads) pair_kernel(const typename Policy::S
     const int j_end = min(M, j_begin + src_per_split);
     uint32_t gt = 0;
     const RegionOut out{partial + (size_t)blockIdx.y * 2 * M, M, 0};
-    (void)pair_item<Policy, R, 2, RegionOut>(src, M, eptr, excl, blockIdx.x, j_begin, j_end, out, kc, err, sm.ring,
+    (void)pair_item<Policy, R, 2, RegionOut>(src, M, Exclusions{eptr, excl, nullptr, nullptr, nullptr}, blockIdx.x, j_begin, j_end, out, kc, err, sm.ring,
                                              sm.tab, bar, gt);
 }
 
@@ -86,23 +86,14 @@ __global__ void pack_kernel(const double* __restrict__ x, const double* __restri
 }
 
 // y = diag + the node's accumulated dense sum (read and cleared) + correction (FP64)
-__global__ void finish_kernel(int64_t M, unsigned long long* __restrict__ acc, const double* __restrict__ x,
-                              double* __restrict__ y, const double* __restrict__ W, const int32_t* __restrict__ ptr,
-                              const int32_t* __restrict__ node, const double* __restrict__ w, int64_t E,
-                              double lam1, double lam2, double h2, double h3, const int32_t* __restrict__ tinv) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= M) return;
-    double s1, s2;
-    fx_read(acc + (tinv ? (int64_t)tinv[i] : i), M, true, s1, s2);
-    double c1 = 0.0, c2 = 0.0;
-    for (int e = ptr[i]; e < ptr[i + 1]; ++e) {
-        const int m = node[e];
-        const double Wm = W[m], r1 = x[m], r2 = x[M + m];
-        c1 += Wm * (h2 * w[e] * r1 - h3 * w[3 * E + e] * r2);
-        c2 += Wm * (h2 * w[E + e] * r1 - h2 * w[2 * E + e] * r2);
-    }
-    y[i] = lam1 * x[i] + s1 + c1;
-    y[M + i] = lam2 * x[M + i] + s2 + c2;
+__global__ void __launch_bounds__(kFinishThreads) finish_kernel(const FinishRows f, unsigned long long* __restrict__ acc,
+                                                              const double* __restrict__ x, double* __restrict__ y,
+                                                              double lam1, double lam2,
+                                                              const int32_t* __restrict__ tinv) {
+    finish_rows(f, acc, tinv, x, [&](int64_t i, int c, double v) {
+        const int64_t q = (int64_t)c * f.M + i;
+        y[q] = (c == 0 ? lam1 : lam2) * x[q] + v;
+    });
 }
 
 // float-float static source data {P.hi}{P.lo}{n.hi}{n.lo} (weights filled per application)
@@ -276,6 +267,19 @@ int pair_consts(ctr_ibim* s, int pol, PairConsts* out) {
     return CTR_OK;
 }
 
+FinishRows finish_rows_of(const ctr_ibim* s) {
+    FinishRows f{};
+    f.ptr = s->corr_ptr.as<int32_t>();
+    f.node = s->corr_node.as<int32_t>();
+    f.w = s->corr_w.as<double>();
+    f.W = s->na.W;
+    f.M = s->M;
+    f.E = s->E;
+    f.h2 = s->h * s->h;
+    f.h3 = s->h * s->h * s->h;
+    return f;
+}
+
 int pack_sources(ctr_ibim* s, const double* d_x, int precision) {
     const int64_t M = s->M;
     const double scale = s->h * s->h * s->h / (4.0 * kPi);
@@ -337,13 +341,9 @@ int apply_operator_timed(ctr_ibim* s, const double* d_x, double* d_y, int precis
     CTR_TRY(mark(2));
     CTR_TRY(launch_tree(s, pol));
     CTR_TRY(mark(3));
-    const double h2 = s->h * s->h;
-    const double h3 = s->h * s->h * s->h;
-    finish_kernel<<<grid_for(M, 256), 256, 0, st>>>(M, s->acc.as<unsigned long long>(), d_x, d_y, s->na.W,
-                                                   s->corr_ptr.as<int32_t>(), s->corr_node.as<int32_t>(),
-                                                   s->corr_w.as<double>(), s->E,
-                                                   0.5 * (1.0 + s->eps_out / s->eps_in),
-                                                   0.5 * (1.0 + s->eps_in / s->eps_out), h2, h3, tinv);
+    finish_kernel<<<grid_for(M, kFinishRows), kFinishThreads, 0, st>>>(
+        finish_rows_of(s), s->acc.as<unsigned long long>(), d_x, d_y, 0.5 * (1.0 + s->eps_out / s->eps_in),
+        0.5 * (1.0 + s->eps_in / s->eps_out), tinv);
     CTR_LAUNCHED();
     CTR_TRY(mark(4));
     return CTR_OK;

@@ -5,16 +5,19 @@
 // r = |P_i - P_j|, e^{-kappa r}, the three dot products of d = P_i - P_j with
 // n_i and n_j, and n_i . n_j, whichever of the two nodes is the target.  A
 // symmetric item evaluates each pair of its (target block, source range) once
-// for both orientations (pairkern.cuh, pair_item_sym); a one-sided item
-// evaluates target rows only and masks the correction pairs N(i), which the
-// dense sum omits.  N(i) is not symmetric (j in N(i) does not imply i in N(j)),
-// so every block pair (I, J) in which some correction pair occurs in either
-// direction is "near" and gets one-sided items from both sides; every other
-// block pair with J > I gets symmetric items.  Since the correction nodes of i
-// lie within a few h of P_i, near pairs form a band around the diagonal.
+// for both orientations (pairkern.cuh, pair_item_sym).  The correction pairs,
+// which the dense sum omits, are not symmetric (j in N(i) does not imply i in
+// N(j)), so a block pair (I, J), J > I, with a correction pair in either
+// direction gets near symmetric items: each excluded pair is masked for the
+// row(s) that leave it out (closed exclusion lists, built here).  Block pairs
+// without one get plain symmetric items, diagonal blocks one-sided ones.
+// Since the correction nodes of i lie within a few h of P_i, near pairs form
+// a band around the diagonal: 6% of the pairs of a large system (1024-node
+// blocks at 178 575 nodes), most of a small one's.
 //
 // Items are split to at most a quarter-wave of work each, and to at most
-// kItemSeconds of one resident block's time, and sorted by cost for the
+// kItemSeconds of one resident block's time (small systems: to pieces of one
+// length that fill whole waves), and sorted by cost for the
 // atomic-counter scheduler.  Every item adds its sums into the nodes'
 // exact accumulators (pairkern.cuh, fx_add: integer addition, so the order in
 // which blocks add does not change a bit of the result).
@@ -40,6 +43,13 @@ constexpr int kMaxBaseBlocks = 8192; // near-flag matrix side (bytes: its square
 // one-sided one, per arithmetic: extra terms of the second orientation plus the
 // in-warp transposed sums.
 constexpr double kSymCost[3] = {1.25, 1.20, 1.15};
+constexpr double kNearCost[3] = {1.45, 1.25, 1.17};   // ... with excluded pairs masked
+
+// Small systems: pieces of a multiple of kPieceStep sources, and the cost of starting an item (target and list
+// loads, the first tile's latency, the sums' atomics) in sources of a 256-target block, per arithmetic.
+
+constexpr int kPieceStep = 16;
+constexpr double kItemStart[3] = {16.0, 1.5, 0.5};
 
 __global__ void near_flags_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ excl, int64_t M,
                                   int g0, int nb0, uint8_t* __restrict__ flags) {
@@ -54,10 +64,65 @@ __global__ void near_flags_kernel(const int32_t* __restrict__ ptr, const int32_t
     }
 }
 
+// Closed exclusion lists (Exclusions): every correction pair (i, m) counts once for i and once for m, which
+// bounds row i's list by its own entries plus the rows it appears in; the lists keep that room.
+__global__ void closure_count_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ excl, int64_t M,
+                                     int32_t* __restrict__ count) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= M) return;
+    const int e0 = ptr[i], e1 = ptr[i + 1];
+    atomicAdd(&count[i], e1 - e0);
+    for (int e = e0; e < e1; ++e) atomicAdd(&count[excl[e]], 1);
+}
+// rows in which node m appears, behind the room of its own entries (order: as the blocks run, sorted below)
+__global__ void closure_scatter_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ excl, int64_t M,
+                                       const int32_t* __restrict__ begin, int32_t* __restrict__ fill,
+                                       int32_t* __restrict__ list) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= M) return;
+    for (int e = ptr[i]; e < ptr[i + 1]; ++e) {
+        const int m = excl[e];
+        list[begin[m] + (ptr[m + 1] - ptr[m]) + atomicAdd(&fill[m], 1)] = (int32_t)i;
+    }
+}
+// sorts the scattered rows of node i and merges them with N(i) into the flagged list
+__global__ void closure_merge_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ excl, int64_t M,
+                                     const int32_t* __restrict__ begin, const int32_t* __restrict__ fill,
+                                     int32_t* __restrict__ list, int32_t* __restrict__ end) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= M) return;
+    int e = ptr[i];
+    const int e1 = ptr[i + 1], b = begin[i], n = fill[i];
+    int32_t* t = list + b + (e1 - e);   // at or behind every place the merge writes to
+    for (int p = 1; p < n; ++p) {
+        const int32_t v = t[p];
+        int q = p;
+        while (q > 0 && t[q - 1] > v) {
+            t[q] = t[q - 1];
+            --q;
+        }
+        t[q] = v;
+    }
+    int w = b, p = 0;
+    while (e < e1 || p < n) {
+        const int32_t own = e < e1 ? excl[e] : INT_MAX, other = p < n ? t[p] : INT_MAX;
+        int flags = 0;
+        if (own <= other) {
+            flags |= kOutTarget;
+            ++e;
+        }
+        if (other <= own) {
+            flags |= kOutSource;
+            ++p;
+        }
+        list[w++] = 4 * min(own, other) + flags;
+    }
+    end[i] = w;
+}
+
 template <typename Policy, int R, int V, int U>
 __global__ void __launch_bounds__(kThreads, Policy::kMinBlocks) sched_kernel(const typename Policy::Src* __restrict__ src, int M,
-                                                         const int32_t* __restrict__ eptr,
-                                                         const int32_t* __restrict__ excl,
+                                                         const Exclusions cl,
                                                          const PairItem* __restrict__ items, int n_items,
                                                          int* __restrict__ counter,
                                                          unsigned long long* __restrict__ acc, PairConsts kc,
@@ -68,15 +133,15 @@ __global__ void __launch_bounds__(kThreads, Policy::kMinBlocks) sched_kernel(con
     __shared__ int cur;
     pair_block_init<Policy>(kc.exp_tab, sm.tab, bar);
     uint32_t gt = 0;
-    for (;;) {
-        if (threadIdx.x == 0) cur = atomicAdd(counter, 1);
-        __syncthreads();
-        const int it = cur;
-        __syncthreads();
+    for (int it = blockIdx.x;;) {   // the first items need no counter
         if (it >= n_items) break;
-        if (!run_item<Policy, R, V, U>(items[it], src, M, eptr, excl, acc, kc, err, sm.ring, sm.jred, sm.tab, bar,
+        if (!run_item<Policy, R, V, U>(items[it], src, M, cl, acc, kc, err, sm.ring, sm.jred, sm.tab, bar,
                                        gt))
             return;
+        if (threadIdx.x == 0) cur = gridDim.x + atomicAdd(counter, 1);
+        __syncthreads();
+        it = cur;
+        __syncthreads();
     }
 }
 
@@ -110,16 +175,17 @@ int sched_launch(ctr_ibim* s, int pol, const void* src, const PairConsts& kc, in
     CTR_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(int), s->stream));
     sched_kernel<Policy, R, V, U><<<grid, kThreads, pair_smem_bytes<Policy>(), s->stream>>>(
         reinterpret_cast<const typename Policy::Src*>(src), (int)s->M,
-        s->tree ? s->tree->d_eptr.as<int32_t>() : s->corr_ptr.as<int32_t>(),
-        s->tree ? s->tree->d_excl.as<int32_t>() : s->excl.as<int32_t>(), p.d_items.as<PairItem>(),
+        exclusions_of(s), p.d_items.as<PairItem>(),
         (int)p.items.size(), counter, s->acc.as<unsigned long long>(), kc, s->err.as<int>());
     CTR_LAUNCHED();
     return CTR_OK;
 }
 
-// Items of one arithmetic for a system of M nodes with the given near-flag matrix.
-void plan_schedule(PairSchedule& p, int64_t M, int R, int tile, double sym_cost, double item_cost,
-                   const std::vector<uint8_t>& flags, int g0, int nb0, int slots) {
+// Items of one arithmetic (pol) for a system of M nodes with the given near-flag matrix.
+void plan_schedule(PairSchedule& p, int pol, int64_t M, int R, int tile, const std::vector<uint8_t>& flags, int g0,
+                   int nb0, int slots) {
+    const double costs[3] = {1.0, kSymCost[pol], kNearCost[pol]};   // by item kind
+    const double item_cost = kUnitRate[pol] * kItemSeconds[pol];
     p.R = R;
     p.BS = kThreads * R;
     p.tile = tile;
@@ -145,39 +211,55 @@ void plan_schedule(PairSchedule& p, int64_t M, int R, int tile, double sym_cost,
     std::vector<Run> runs;
     double total = 0.0;
     for (int I = 0; I < nb; ++I) {
-        int J = 0;
+        int J = I;
         while (J < nb) {
-            if (near(I, J)) {
-                int J1 = J;
-                while (J1 < nb && near(I, J1)) ++J1;
-                runs.push_back(Run{I, (int)((int64_t)J * BS), (int)std::min<int64_t>(M, (int64_t)J1 * BS), 0});
-                J = J1;
-            } else if (J > I) {
-                int J1 = J;
-                while (J1 < nb && !near(I, J1)) ++J1;
-                runs.push_back(Run{I, (int)((int64_t)J * BS), (int)std::min<int64_t>(M, (int64_t)J1 * BS), 1});
-                J = J1;
-            } else {
-                ++J;
-            }
+            const int kind = J == I ? kItemOne : near(I, J) ? kItemNear : kItemSym;
+            int J1 = J + 1;
+            if (kind != kItemOne)
+                while (J1 < nb && near(I, J1) == (kind == kItemNear)) ++J1;
+            runs.push_back(Run{I, (int)((int64_t)J * BS), (int)std::min<int64_t>(M, (int64_t)J1 * BS), kind});
+            J = J1;
         }
     }
-    for (const Run& r : runs) total += (double)BS * (r.j1 - r.j0) * (r.sym ? sym_cost : 1.0);
+    for (const Run& r : runs) total += (double)BS * (r.j1 - r.j0) * costs[r.sym];
     // split runs into items of at most a quarter-wave of work and kItemSeconds of one block (item_cost:
     // the arithmetic's rate x kItemSeconds; whole tiles, at least two when possible)
     const double nslots = (double)std::max(1, slots);
     const double cmax = std::max(1.0, std::min(total / ((double)kItemsPerSlot * nslots), item_cost / nslots));
+    // A system with less than eight tiles of work per resident block cannot be cut that way (few items, the
+    // last wave nearly empty): its pieces have one common length, the one with the shortest estimated makespan
+    // (waves of equal pieces, each with the cost of starting it).  The FP64 kernel is bound by one pipe per
+    // SM whatever the blocks on it, so there the waves are counted in SMs.
+    int64_t piece = 0;
+    const double servers = pol == 2 ? std::max(1.0, nslots / 2.0) : nslots;
+    if (total < 8.0 * tile * BS * nslots) {
+        double best = 1e300;
+        const double start = kItemStart[pol] * kThreads / BS;
+        for (int64_t len = kPieceStep; len <= 2 * tile; len += kPieceStep) {
+            int64_t n = 0;
+            for (const Run& r : runs) n += (r.j1 - r.j0 + len - 1) / len;
+            const double waves = std::ceil((double)n / servers);
+            const double t = waves * ((double)len + start);
+            if (t < 0.99 * best) {   // the longer pieces unless shorter ones gain
+                best = t;
+                piece = len;
+            }
+        }
+    }
     p.total_cost = total;
     p.items.clear();
     p.cost.clear();
     p.pairs_sym = p.pairs_one = 0;
     for (const Run& r : runs) {
         const int64_t len = r.j1 - r.j0;
-        const double unit = (double)BS * (r.sym ? sym_cost : 1.0);
-        int64_t pieces = std::max<int64_t>(1, (int64_t)std::ceil(unit * (double)len / cmax));
-        int64_t plen = (len + pieces - 1) / pieces;
-        plen = ((plen + tile - 1) / tile) * tile;
-        plen = std::max<int64_t>(plen, std::min<int64_t>(len, 2 * (int64_t)tile));
+        const double unit = (double)BS * costs[r.sym];
+        int64_t plen = piece;
+        if (piece == 0) {
+            const int64_t pieces = std::max<int64_t>(1, (int64_t)std::ceil(unit * (double)len / cmax));
+            plen = (len + pieces - 1) / pieces;
+            plen = ((plen + tile - 1) / tile) * tile;
+            plen = std::max<int64_t>(plen, std::min<int64_t>(len, 2 * (int64_t)tile));
+        }
         for (int64_t a = r.j0; a < r.j1; a += plen) {
             PairItem it{};
             it.I = r.I;
@@ -241,8 +323,7 @@ int plan_fp32(ctr_ibim* s, const std::vector<uint8_t>& flags, int g0, int nb0, i
     auto plan = [&](int v) -> int {
         const int per = with_var32(v, PerSm{});
         if (per < 0) return per;
-        plan_schedule(s->sched[0], M, kVar32[v].R * Fp32x2Policy::kPack, kVar32[v].tile, kSymCost[0],
-                      kUnitRate[0] * kItemSeconds[0], flags, g0, nb0, per * sms);
+        plan_schedule(s->sched[0], 0, M, kVar32[v].R * Fp32x2Policy::kPack, kVar32[v].tile, flags, g0, nb0, per * sms);
         CTR_TRY(upload_schedule(s->sched[0], M, s->stream));
         s->sched[0].var = v;
         return CTR_OK;
@@ -321,6 +402,13 @@ int schedule_slots(int sms, int slots[3]) {
     return CTR_OK;
 }
 
+Exclusions exclusions_of(const ctr_ibim* s) {
+    if (s->tree)
+        return Exclusions{s->tree->d_eptr.as<int32_t>(), s->tree->d_excl.as<int32_t>(), nullptr, nullptr, nullptr};
+    return Exclusions{s->corr_ptr.as<int32_t>(), s->excl.as<int32_t>(), s->cl_begin.as<int32_t>(),
+                      s->cl_end.as<int32_t>(), s->cl_list.as<int32_t>()};
+}
+
 int launch_schedule(ctr_ibim* s, int pol, const void* src, const PairConsts& kc) {
     CTR_TRY(ensure_schedule(s, pol));
     int sms = 0;
@@ -352,10 +440,36 @@ static int near_flags(ctr_ibim* s, std::vector<uint8_t>& flags, int& g0, int& nb
 static int plan_fixed(ctr_ibim* s, int pol, const std::vector<uint8_t>& flags, int g0, int nb0, const int slots[3]) {
     const int Rs[3] = {0, kRdf, kR64};   // targets per thread of the fixed shapes
     const int tiles[3] = {0, Df64Policy::kTile, Fp64Policy::kTile};
-    plan_schedule(s->sched[pol], s->M, Rs[pol], tiles[pol], kSymCost[pol], kUnitRate[pol] * kItemSeconds[pol], flags,
-                  g0, nb0, slots[pol]);
+    plan_schedule(s->sched[pol], pol, s->M, Rs[pol], tiles[pol], flags, g0, nb0, slots[pol]);
     CTR_TRY(upload_schedule(s->sched[pol], s->M, s->stream));
     s->sched[pol].planned = true;
+    return CTR_OK;
+}
+
+static int build_closure(ctr_ibim* s) {
+    const int64_t M = s->M, E = s->E;
+    if (M >= (int64_t)1 << 29) return fail(CTR_ERR_CAPACITY, "more than 2^29 nodes");   // 4 j + flags in an int32
+    cudaStream_t st = s->stream;
+    const int32_t* ptr = s->corr_ptr.as<int32_t>();
+    const int32_t* excl = s->excl.as<int32_t>();
+    DevBuf scratch, work;
+    CTR_TRY(s->cl_begin.alloc(sizeof(int32_t) * (M + 1)));
+    CTR_TRY(s->cl_end.alloc(sizeof(int32_t) * M));
+    CTR_TRY(s->cl_list.alloc(sizeof(int32_t) * std::max<int64_t>(1, 2 * E)));
+    CTR_TRY(work.alloc(sizeof(int32_t) * 2 * M));
+    int32_t* count = work.as<int32_t>();
+    int32_t* fill = count + M;
+    CTR_CUDA_TRY(cudaMemsetAsync(count, 0, sizeof(int32_t) * 2 * M, st));
+    closure_count_kernel<<<grid_for(M, 256), 256, 0, st>>>(ptr, excl, M, count);
+    CTR_LAUNCHED();
+    CTR_TRY(exclusive_scan_i32(count, s->cl_begin.as<int32_t>(), M, st, scratch));
+    closure_scatter_kernel<<<grid_for(M, 256), 256, 0, st>>>(ptr, excl, M, s->cl_begin.as<int32_t>(), fill,
+                                                            s->cl_list.as<int32_t>());
+    CTR_LAUNCHED();
+    closure_merge_kernel<<<grid_for(M, 256), 256, 0, st>>>(ptr, excl, M, s->cl_begin.as<int32_t>(), fill,
+                                                          s->cl_list.as<int32_t>(), s->cl_end.as<int32_t>());
+    CTR_LAUNCHED();
+    CTR_CUDA_TRY(cudaStreamSynchronize(st));   // `work` is freed on return
     return CTR_OK;
 }
 
@@ -364,6 +478,7 @@ static int plan_fixed(ctr_ibim* s, int pol, const std::vector<uint8_t>& flags, i
 int build_schedules(ctr_ibim* s, const int slots[3]) {
     std::vector<uint8_t> flags;
     int g0 = 0, nb0 = 0;
+    CTR_TRY(build_closure(s));
     CTR_TRY(near_flags(s, flags, g0, nb0));
     CTR_TRY(alloc_accumulators(s));
     CTR_TRY(s->counter.alloc(sizeof(int) * 4));

@@ -43,3 +43,22 @@ def test_operator_at_ragged_sizes(ctr, oracle_tables, name, kappa):
     with ctr.CtrIbim.from_problem(prob) as G:
         for precision, tol in ((ctr.DF64, 1e-12), (ctr.FP64, 1e-12), (ctr.FP32_REFINE, 2e-5)):
             assert np.max(np.abs(G.matvec(x, precision) - ref)) / scale < tol
+
+
+@pytest.mark.parametrize("block", [512, 1024])
+@pytest.mark.parametrize("name", ["kreg_sphere", "molecule"])
+def test_excluded_pairs_of_symmetric_items(ctr, oracle_tables, name, block):
+    """Rows with long and one-sided exclusion lists (K-reg cylinders; hybrid rows beside them): a pair that
+    only one of its two rows leaves out is in the other's sum."""
+    prob = syn.sphere_problem(h=0.25) if name == "kreg_sphere" else syn.molecule_problem(n_atoms=20, seed=1, h=0.5)
+    kreg = name == "kreg_sphere"
+    S = OracleSystem.from_problem(prob, tables=oracle_tables, method="kreg" if kreg else "hyb")
+    sets = [set(S.excl_idx[S.excl_ptr[i]:S.excl_ptr[i + 1]].tolist()) for i in range(S.M)]
+    assert sum(i not in sets[j] for i in range(S.M) for j in sets[i]) > 0   # one-way pairs exist
+    x = syn.random_density(S.M, seed=5)
+    ref = S.matvec(x)
+    scale = np.max(np.abs(ref))
+    opts = ctr.Options(tube_halfwidth=prob.tube, method=ctr.METHOD_KREG if kreg else ctr.METHOD_HYB, fp32_block=block)
+    with ctr.CtrIbim.from_problem(prob, options=opts) as G:
+        for precision, tol in ((ctr.DF64, 1e-12), (ctr.FP64, 1e-12), (ctr.FP32_REFINE, 2e-5)):
+            assert np.max(np.abs(G.matvec(x, precision) - ref)) / scale < tol

@@ -25,9 +25,11 @@ struct PairConsts {
     float2 c1d, c2d, kappad;         // float-float copies
     double k2;                       // kappa log2(e), rounded; k2f: in FP32; k2d: -ln 2 times its rounding error
     float k2f, k2d;
+    double c1kap;                    // (eps_E/eps_I) kappa
     const float2* exp_tab;           // exponential tables of the arithmetic (float-float or FP64), global
     // the FP32 values duplicated into both halves of a 64-bit word (f32x2 operands)
     unsigned long long one2, mone2, three2, mthree2, c1x2, nc1x2, c2x2, nc2x2, kap2, kl2x2;
+    unsigned long long c1kap2;       // (eps_E/eps_I) kappa
     uint32_t wait_limit;             // polls of a source-tile wait before the block gives up
     uint32_t pad_;
 };
@@ -106,6 +108,8 @@ __device__ __forceinline__ u64 sub2(u64 a, u64 b) {
     asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
+// -v as -0 - v: folded into the operand of the instruction that uses it (measured: no slot of its own)
+__device__ __forceinline__ u64 neg2(u64 v) { return sub2(0x8000000080000000ull, v); }
 __device__ __forceinline__ u64 mul2(u64 a, u64 b) {
     u64 d;
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
@@ -537,13 +541,12 @@ struct Fp32Policy {
 // Packed FP32: the Fp32 terms for two targets at once (lanes of f32x2 operations).  A thread slot
 // holds targets a, b (lanes x, y); a source node is stored with every value duplicated,
 // {(x,x),(y,y)} {(z,z),(a,a)} {(nx,nx),(ny,ny)} {(nz,nz),(-b,-b)} (64 B), so a broadcast
-// shared-memory load gives ready operands.  Signs are arranged so that every step is a plain
-// add/sub/mul or a*b + c (the f32x2 forms take no negated operands):
-//   t1 = 1 - c1 E1, t1n = -t1, t2 = 1 - c2 E1, t2n = -t2, om = (1 - E)/r, u = 1 - E1,
+// shared-memory load gives ready operands.  The signs sit in the stored weights:
+//   s t1 = s - c1 s E1, s t2n = c2 s E1 - s, om = (1 - E)/r, u = 1 - E1,
 //   t3n = E q - 3, Bn = t3n (d.n_x)(d.n_y)/r^2, X = u n_x.n_y + Bn,
-//   target rows: a1 += a s (d.n_y) t1 + (-b) om,   a2 += (-b s)(d.n_x) t2n + a s X;
-//   source rows: a1 += ((-a_t) s)(d.n_x) t1 + (-b_t) om,
-//                -a2 += ((-b_t) s)(d.n_y) t2n + ((-a_t) s) X   (negated; jfinal restores the sign).
+//   target rows: a1 += a (d.n_y) s t1 + (-b) om,   a2 += (-b)(d.n_x) s t2n + a s X;
+//   source rows: a1 += (-a_t)(d.n_x) s t1 + (-b_t) om,
+//                -a2 += (-b_t)(d.n_y) s t2n + (-a_t) s X   (negated; jfinal restores the sign).
 struct Fp32x2Policy {
     using Src = ulonglong2;
     static constexpr int kMinBlocks = 2;   // resident blocks per SM the registers are limited for
@@ -635,7 +638,7 @@ struct Fp32x2Policy {
     }
     // The terms shared by both orientations for the two targets of T and source q.
     struct Common {
-        u64 dnx, dny, om, t1, t2n, X, s;
+        u64 dnx, dny, om, st1, st2n, sX;
     };
     __device__ static Common common(const Tgt& T, const Node& q, const PairConsts& k) {
         const u64 dx = sub2(T.px, q.x), dy = sub2(T.py, q.y), dz = sub2(T.pz, q.z);
@@ -650,23 +653,23 @@ struct Fp32x2Policy {
         c.dnx = fma2(dz, T.qz, fma2(dy, T.qy, mul2(dx, T.qx)));
         const u64 nn = fma2(T.qz, q.nz, fma2(T.qy, q.ny, mul2(T.qx, q.nx)));
         const u64 rinv2 = mul2(rinv, rinv);
-        c.s = mul2(rinv2, rinv);
-        c.t1 = fma2(k.nc1x2, E1, k.one2);
-        c.t2n = fma2(k.c2x2, E1, k.mone2);
-        c.om = mul2(rinv, sub2(k.one2, E));
+        const u64 s = mul2(rinv2, rinv);
+        const u64 v = mul2(s, E1);
+        c.st1 = fma2(k.nc1x2, v, s);
+        c.st2n = fma2(k.c2x2, v, neg2(s));
+        c.om = fma2(neg2(rinv), E, rinv);
         const u64 u = sub2(k.one2, E1);
         const u64 p = fma2(kr, add2(kr, k.three2), k.three2);
         const u64 t3n = fma2(E, p, k.mthree2);
         const u64 Bn = mul2(mul2(mul2(t3n, c.dnx), c.dny), rinv2);
-        c.X = fma2(u, nn, Bn);
+        c.sX = mul2(s, fma2(u, nn, Bn));
         return c;
     }
     __device__ static void target_terms(const Common& c, u64 Sa, u64 Snb, Acc& acc) {
-        const u64 as = mul2(Sa, c.s), nbs = mul2(Snb, c.s);
-        acc.a1 = fma2(mul2(as, c.dny), c.t1, acc.a1);
+        acc.a1 = fma2(mul2(Sa, c.dny), c.st1, acc.a1);
         acc.a1 = fma2(Snb, c.om, acc.a1);
-        acc.a2 = fma2(mul2(nbs, c.dnx), c.t2n, acc.a2);
-        acc.a2 = fma2(as, c.X, acc.a2);
+        acc.a2 = fma2(mul2(Snb, c.dnx), c.st2n, acc.a2);
+        acc.a2 = fma2(Sa, c.sX, acc.a2);
     }
     template <bool kMask>
     __device__ static void pair(const Tgt& T, const Src* S, const PairConsts& k, const float2*, Acc& acc,
@@ -675,8 +678,8 @@ struct Fp32x2Policy {
         if (kMask && (ex[0] || ex[1])) exclude(T, q, ex, k.one2);
         target_terms(common(T, q, k), q.a, q.nb, acc);
     }
-    // Both orientations: s is folded once into the factors the two share (s t1, s t2n, s X), which
-    // saves one f32x2 operation per pair against forming a s, b s and the targets' (-a) s, (-b) s.
+    // Both orientations: the factors s t1, s t2n, s X and (1 - E)/r are formed once (39 operations per one-sided
+    // evaluation, 47 per symmetric one).
     // kMask: flags per half (Exclusions); a pair left out of both rows is moved to distance 1 (no NaN).
     template <bool kFirst, bool kMask = false>
     __device__ static void pair_sym(const Tgt& T, const Src* S, const PairConsts& k, const float2*, Acc& acc,
@@ -698,20 +701,16 @@ struct Fp32x2Policy {
             }
         }
         const Common c = common(T, q, k);
-        const u64 st1 = mul2(c.s, c.t1), st2n = mul2(c.s, c.t2n), sX = mul2(c.s, c.X);
-        acc.a1 = fma2(mul2(q.a, c.dny), st1, acc.a1);
-        acc.a1 = fma2(q.nb, c.om, acc.a1);
-        acc.a2 = fma2(mul2(q.nb, c.dnx), st2n, acc.a2);
-        acc.a2 = fma2(q.a, sX, acc.a2);
+        target_terms(c, q.a, q.nb, acc);
         if constexpr (kFirst) {
-            ja.a1 = mul2(mul2(nwa, c.dnx), st1);
-            ja.a2 = mul2(mul2(nwb, c.dny), st2n);   // ja.a2 holds -a2 until jfinal
+            ja.a1 = mul2(mul2(nwa, c.dnx), c.st1);
+            ja.a2 = mul2(mul2(nwb, c.dny), c.st2n);   // ja.a2 holds -a2 until jfinal
         } else {
-            ja.a1 = fma2(mul2(nwa, c.dnx), st1, ja.a1);
-            ja.a2 = fma2(mul2(nwb, c.dny), st2n, ja.a2);
+            ja.a1 = fma2(mul2(nwa, c.dnx), c.st1, ja.a1);
+            ja.a2 = fma2(mul2(nwb, c.dny), c.st2n, ja.a2);
         }
         ja.a1 = fma2(nwb, c.om, ja.a1);
-        ja.a2 = fma2(nwa, sX, ja.a2);
+        ja.a2 = fma2(nwa, c.sX, ja.a2);
     }
 };
 

@@ -235,6 +235,7 @@ void set_packed_consts(PairConsts& kc) {
     kc.nc2x2 = dup(-kc.c2f);
     kc.kap2 = dup(kc.kappaf);
     kc.kl2x2 = dup(kc.kl2f);
+    kc.c1kap2 = dup((float)(kc.c1 * kc.kappa));
 }
 
 namespace {
@@ -261,6 +262,7 @@ int pair_consts(ctr_ibim* s, int pol, PairConsts* out) {
     kc.k2 = s->kappa * 1.4426950408889634;
     const double lost = std::fma(s->kappa, 1.4426950408889634, -kc.k2) + s->kappa * 2.0355273740931033e-17;
     kc.k2f = (float)kc.k2;
+    kc.c1kap = kc.c1 * kc.kappa;
     kc.k2d = (float)(-0.6931471805599453 * lost);
     CTR_TRY(exp_table(s->device, pol, &kc.exp_tab));
     *out = kc;

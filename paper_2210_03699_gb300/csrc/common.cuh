@@ -246,7 +246,7 @@ struct ctr_ibim {
     ctr::DevBuf corr_w;      // double [4][E]: omega11, omega21, omega22, omega12
     ctr::DevBuf bad;         // uint8 [M] hybrid classification
     ctr::DevBuf excl;        // int32 [E] sorted correction nodes per target
-    ctr::DevBuf cl_begin, cl_end, cl_list;   // int32: closed exclusion lists of direct handles (pk::Exclusions)
+    ctr::DevBuf cl_begin, cl_end, cl_list;   // int32: closed exclusion lists (pk::Exclusions)
     ctr::DevBuf rhs;         // double [2M]
     ctr::DevBuf charges;     // double [4][nc]: x, y, z, q
     ctr::DevBuf acc;         // exact accumulators of the dense sum: pk::kFxWords x M 64-bit words
@@ -278,6 +278,12 @@ int build_tree_schedules(ctr_ibim* s, const int slots[3]);
 int launch_tree(ctr_ibim* s, int pol);
 int64_t tree_bytes(const ctr_ibim* s);
 // schedule.cu: symmetric / one-sided pair schedules of a handle
+constexpr int kMaxBaseBlocks = 8192;   // side of a block-pair matrix (bytes: its square)
+// items of p (BS and tile set) from runs: target block, source range, kind; then their device copy
+void cut_runs(PairSchedule& p, int pol, int64_t M, const std::vector<PairItem>& runs, int slots);
+int upload_schedule(PairSchedule& p, cudaStream_t st);
+// the closed exclusion lists (pk::Exclusions) of correction rows ptr, excl (device, ascending in each row)
+int build_closure(ctr_ibim* s, const int32_t* ptr, const int32_t* excl);
 int build_schedules(ctr_ibim* s, const int slots[3]);
 int ensure_schedule(ctr_ibim* s, int pol);   // plans pair arithmetic `pol` if it has not been planned yet
 // the handle's exact node accumulators, allocated and cleared (pairsum.cu)

@@ -1006,8 +1006,8 @@ struct FxOut {
 // What the items leave out, by target position i, ascending.
 //   own: the correction nodes N(i), own_list[own_begin[i] .. own_begin[i + 1]): the one-sided items' masks.
 //   closed: every node j with j in N(i) or i in N(j), as 4 j + flags (kOutTarget: j is left out of row i,
-//   kOutSource: i is left out of row j), list[begin[i] .. end[i]): the near symmetric items' masks (direct
-//   handles; NULL for treecode handles, which have no such items).
+//   kOutSource: i is left out of row j), list[begin[i] .. end[i]): the near symmetric items' masks.
+// (Positions: node ids, or tree positions in a treecode handle.)
 struct Exclusions {
     const int32_t* own_begin;
     const int32_t* own_list;

@@ -37,7 +37,6 @@ using namespace pk;
 namespace {
 
 constexpr int kItemsPerSlot = 4;     // items per resident block in a single-system launch
-constexpr int kMaxBaseBlocks = 8192; // near-flag matrix side (bytes: its square)
 
 // Relative cost of one symmetric pair evaluation (two orientations) against a
 // one-sided one, per arithmetic: extra terms of the second orientation plus the
@@ -50,6 +49,14 @@ constexpr double kNearCost[3] = {1.45, 1.25, 1.17};   // ... with excluded pairs
 
 constexpr int kPieceStep = 16;
 constexpr double kItemStart[3] = {16.0, 1.5, 0.5};
+
+// Larger systems: the part of each run cut into pieces of full length; the rest goes into pieces of a quarter of
+// it (kFineMin sources or more), which come last and even out the end of the launch.  With full pieces only,
+// the SMs of an FP32 application at 44 597 nodes idle 14% of the time; 1.79 -> 1.64 ms there (1024-node
+// blocks), 4.07 -> 3.90 at 69 793, 25.2 -> 24.7 at 178 575.  Fractions of 0.5 to 0.8 and divisors of 2 to 8
+// measured within 2% of each other.
+constexpr double kCoarse = 0.7;
+constexpr int kFineDiv = 4, kFineMin = 64;
 
 __global__ void near_flags_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ excl, int64_t M,
                                   int g0, int nb0, uint8_t* __restrict__ flags) {
@@ -74,7 +81,7 @@ __global__ void closure_count_kernel(const int32_t* __restrict__ ptr, const int3
     atomicAdd(&count[i], e1 - e0);
     for (int e = e0; e < e1; ++e) atomicAdd(&count[excl[e]], 1);
 }
-// rows in which node m appears, behind the room of its own entries (order: as the blocks run, sorted below)
+// the rows in which node m appears, in the order the blocks run
 __global__ void closure_scatter_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ excl, int64_t M,
                                        const int32_t* __restrict__ begin, int32_t* __restrict__ fill,
                                        int32_t* __restrict__ list) {
@@ -82,40 +89,48 @@ __global__ void closure_scatter_kernel(const int32_t* __restrict__ ptr, const in
     if (i >= M) return;
     for (int e = ptr[i]; e < ptr[i + 1]; ++e) {
         const int m = excl[e];
-        list[begin[m] + (ptr[m + 1] - ptr[m]) + atomicAdd(&fill[m], 1)] = (int32_t)i;
+        list[begin[m] + atomicAdd(&fill[m], 1)] = (int32_t)i;
     }
 }
-// sorts the scattered rows of node i and merges them with N(i) into the flagged list
+// ... in ascending order: a warp per node, every entry to the place its rank gives (K-reg rows have a hundred
+// entries and more, where one thread's insertion sort takes milliseconds)
+__global__ void closure_sort_kernel(int64_t M, const int32_t* __restrict__ begin, const int32_t* __restrict__ fill,
+                                    const int32_t* __restrict__ list, int32_t* __restrict__ sorted) {
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i >= M) return;
+    const int32_t* t = list + begin[i];
+    const int n = fill[i];
+    for (int p = threadIdx.x & 31; p < n; p += 32) {
+        const int32_t v = t[p];
+        int rank = 0;
+        for (int q = 0; q < n; ++q) rank += t[q] < v;   // entries are distinct
+        sorted[begin[i] + rank] = v;
+    }
+}
+// merges them with N(i) into the flagged list
 __global__ void closure_merge_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ excl, int64_t M,
                                      const int32_t* __restrict__ begin, const int32_t* __restrict__ fill,
-                                     int32_t* __restrict__ list, int32_t* __restrict__ end) {
+                                     const int32_t* __restrict__ sorted, int32_t* __restrict__ list,
+                                     int32_t* __restrict__ end) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= M) return;
-    int e = ptr[i];
-    const int e1 = ptr[i + 1], b = begin[i], n = fill[i];
-    int32_t* t = list + b + (e1 - e);   // at or behind every place the merge writes to
-    for (int p = 1; p < n; ++p) {
-        const int32_t v = t[p];
-        int q = p;
-        while (q > 0 && t[q - 1] > v) {
-            t[q] = t[q - 1];
-            --q;
-        }
-        t[q] = v;
-    }
-    int w = b, p = 0;
-    while (e < e1 || p < n) {
-        const int32_t own = e < e1 ? excl[e] : INT_MAX, other = p < n ? t[p] : INT_MAX;
+    int e = ptr[i], p = begin[i], w = begin[i];
+    const int e1 = ptr[i + 1], p1 = p + fill[i];
+    int32_t own = e < e1 ? excl[e] : INT_MAX, other = p < p1 ? sorted[p] : INT_MAX;
+    while (own != INT_MAX || other != INT_MAX) {
+        const int32_t v = min(own, other);
         int flags = 0;
-        if (own <= other) {
+        if (own == v) {
             flags |= kOutTarget;
             ++e;
+            own = e < e1 ? excl[e] : INT_MAX;
         }
-        if (other <= own) {
+        if (other == v) {
             flags |= kOutSource;
             ++p;
+            other = p < p1 ? sorted[p] : INT_MAX;
         }
-        list[w++] = 4 * min(own, other) + flags;
+        list[w++] = 4 * v + flags;
     }
     end[i] = w;
 }
@@ -184,8 +199,6 @@ int sched_launch(ctr_ibim* s, int pol, const void* src, const PairConsts& kc, in
 // Items of one arithmetic (pol) for a system of M nodes with the given near-flag matrix.
 void plan_schedule(PairSchedule& p, int pol, int64_t M, int R, int tile, const std::vector<uint8_t>& flags, int g0,
                    int nb0, int slots) {
-    const double costs[3] = {1.0, kSymCost[pol], kNearCost[pol]};   // by item kind
-    const double item_cost = kUnitRate[pol] * kItemSeconds[pol];
     p.R = R;
     p.BS = kThreads * R;
     p.tile = tile;
@@ -205,11 +218,7 @@ void plan_schedule(PairSchedule& p, int pol, int64_t M, int R, int tile, const s
                 if (flags[(size_t)a * nb0 + b]) return true;
         return false;
     };
-    struct Run {
-        int I, j0, j1, sym;
-    };
-    std::vector<Run> runs;
-    double total = 0.0;
+    std::vector<PairItem> runs;
     for (int I = 0; I < nb; ++I) {
         int J = I;
         while (J < nb) {
@@ -217,85 +226,11 @@ void plan_schedule(PairSchedule& p, int pol, int64_t M, int R, int tile, const s
             int J1 = J + 1;
             if (kind != kItemOne)
                 while (J1 < nb && near(I, J1) == (kind == kItemNear)) ++J1;
-            runs.push_back(Run{I, (int)((int64_t)J * BS), (int)std::min<int64_t>(M, (int64_t)J1 * BS), kind});
+            runs.push_back(PairItem{I, (int)((int64_t)J * BS), (int)std::min<int64_t>(M, (int64_t)J1 * BS), kind});
             J = J1;
         }
     }
-    for (const Run& r : runs) total += (double)BS * (r.j1 - r.j0) * costs[r.sym];
-    // split runs into items of at most a quarter-wave of work and kItemSeconds of one block (item_cost:
-    // the arithmetic's rate x kItemSeconds; whole tiles, at least two when possible)
-    const double nslots = (double)std::max(1, slots);
-    const double cmax = std::max(1.0, std::min(total / ((double)kItemsPerSlot * nslots), item_cost / nslots));
-    // A system with less than eight tiles of work per resident block cannot be cut that way (few items, the
-    // last wave nearly empty): its pieces have one common length, the one with the shortest estimated makespan
-    // (waves of equal pieces, each with the cost of starting it).  The FP64 kernel is bound by one pipe per
-    // SM whatever the blocks on it, so there the waves are counted in SMs.
-    int64_t piece = 0;
-    const double servers = pol == 2 ? std::max(1.0, nslots / 2.0) : nslots;
-    if (total < 8.0 * tile * BS * nslots) {
-        double best = 1e300;
-        const double start = kItemStart[pol] * kThreads / BS;
-        for (int64_t len = kPieceStep; len <= 2 * tile; len += kPieceStep) {
-            int64_t n = 0;
-            for (const Run& r : runs) n += (r.j1 - r.j0 + len - 1) / len;
-            const double waves = std::ceil((double)n / servers);
-            const double t = waves * ((double)len + start);
-            if (t < 0.99 * best) {   // the longer pieces unless shorter ones gain
-                best = t;
-                piece = len;
-            }
-        }
-    }
-    p.total_cost = total;
-    p.items.clear();
-    p.cost.clear();
-    p.pairs_sym = p.pairs_one = 0;
-    for (const Run& r : runs) {
-        const int64_t len = r.j1 - r.j0;
-        const double unit = (double)BS * costs[r.sym];
-        int64_t plen = piece;
-        if (piece == 0) {
-            const int64_t pieces = std::max<int64_t>(1, (int64_t)std::ceil(unit * (double)len / cmax));
-            plen = (len + pieces - 1) / pieces;
-            plen = ((plen + tile - 1) / tile) * tile;
-            plen = std::max<int64_t>(plen, std::min<int64_t>(len, 2 * (int64_t)tile));
-        }
-        for (int64_t a = r.j0; a < r.j1; a += plen) {
-            PairItem it{};
-            it.I = r.I;
-            it.j_begin = (int32_t)a;
-            it.j_end = (int32_t)std::min<int64_t>(r.j1, a + plen);
-            it.sym = r.sym;
-            const int64_t tgt = std::min<int64_t>(BS, M - (int64_t)r.I * BS);
-            if (r.sym) p.pairs_sym += tgt * (it.j_end - it.j_begin);
-            else p.pairs_one += tgt * (it.j_end - it.j_begin);
-            p.items.push_back(it);
-            p.cost.push_back(unit * (double)(it.j_end - it.j_begin));
-        }
-    }
-}
-
-// Device copy of the items sorted by decreasing cost (afterwards the host copy is in that order too).
-int upload_schedule(PairSchedule& p, int64_t M, cudaStream_t st) {
-    std::vector<int> order(p.items.size());
-    std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return p.cost[a] > p.cost[b]; });
-    std::vector<PairItem> sorted(p.items.size());
-    std::vector<double> sorted_cost(p.items.size());
-    for (size_t k = 0; k < order.size(); ++k) {
-        sorted[k] = p.items[order[k]];
-        sorted_cost[k] = p.cost[order[k]];
-    }
-    CTR_TRY(p.d_items.alloc(sizeof(PairItem) * std::max<size_t>(1, sorted.size())));
-    if (!sorted.empty())
-        CTR_CUDA_TRY(cudaMemcpyAsync(p.d_items.p, sorted.data(), sizeof(PairItem) * sorted.size(),
-                                     cudaMemcpyHostToDevice, st));
-    CTR_CUDA_TRY(cudaStreamSynchronize(st));   // the host vectors above go out of scope
-    // the host copy follows the device order: the engine's work entries index the device list
-    p.items.swap(sorted);
-    p.cost.swap(sorted_cost);
-    (void)M;
-    return CTR_OK;
+    cut_runs(p, pol, M, runs, slots);
 }
 
 std::atomic<int> g_last_var32{-1};
@@ -324,7 +259,7 @@ int plan_fp32(ctr_ibim* s, const std::vector<uint8_t>& flags, int g0, int nb0, i
         const int per = with_var32(v, PerSm{});
         if (per < 0) return per;
         plan_schedule(s->sched[0], 0, M, kVar32[v].R * Fp32x2Policy::kPack, kVar32[v].tile, flags, g0, nb0, per * sms);
-        CTR_TRY(upload_schedule(s->sched[0], M, s->stream));
+        CTR_TRY(upload_schedule(s->sched[0], s->stream));
         s->sched[0].var = v;
         return CTR_OK;
     };
@@ -387,6 +322,93 @@ int plan_fp32(ctr_ibim* s, const std::vector<uint8_t>& flags, int g0, int nb0, i
 
 }  // namespace
 
+// The items of a schedule (its block size and tile set) from runs: a target block against a source range of
+// one kind.
+void cut_runs(PairSchedule& p, int pol, int64_t M, const std::vector<PairItem>& runs, int slots) {
+    const double costs[3] = {1.0, kSymCost[pol], kNearCost[pol]};   // by item kind
+    const double item_cost = kUnitRate[pol] * kItemSeconds[pol];
+    const int BS = p.BS, tile = p.tile;
+    double total = 0.0;
+    for (const PairItem& r : runs) total += (double)BS * (r.j_end - r.j_begin) * costs[r.sym];
+    // split runs into items of at most a quarter-wave of work and kItemSeconds of one block (item_cost:
+    // the arithmetic's rate x kItemSeconds; whole tiles, at least two when possible)
+    const double nslots = (double)std::max(1, slots);
+    const double cmax = std::max(1.0, std::min(total / ((double)kItemsPerSlot * nslots), item_cost / nslots));
+    // A system with less than eight tiles of work per resident block cannot be cut that way (few items, the
+    // last wave nearly empty): its pieces have one common length, the one with the shortest estimated makespan
+    // (waves of equal pieces, each with the cost of starting it).  The FP64 kernel is bound by one pipe per
+    // SM whatever the blocks on it, so there the waves are counted in SMs.
+    int64_t piece = 0;
+    const double servers = pol == 2 ? std::max(1.0, nslots / 2.0) : nslots;
+    if (total < 8.0 * tile * BS * nslots) {
+        double best = 1e300;
+        const double start = kItemStart[pol] * kThreads / BS;
+        for (int64_t len = kPieceStep; len <= 2 * tile; len += kPieceStep) {
+            int64_t n = 0;
+            for (const PairItem& r : runs) n += (r.j_end - r.j_begin + len - 1) / len;
+            const double waves = std::ceil((double)n / servers);
+            const double t = waves * ((double)len + start);
+            if (t < 0.99 * best) {   // the longer pieces unless shorter ones gain
+                best = t;
+                piece = len;
+            }
+        }
+    }
+    p.total_cost = total;
+    p.items.clear();
+    p.cost.clear();
+    p.pairs_sym = p.pairs_one = 0;
+    for (const PairItem& r : runs) {
+        const int64_t len = r.j_end - r.j_begin;
+        const double unit = (double)BS * costs[r.sym];
+        int64_t plen = piece;
+        if (piece == 0) {
+            const int64_t pieces = std::max<int64_t>(1, (int64_t)std::ceil(unit * (double)len / cmax));
+            plen = (len + pieces - 1) / pieces;
+            plen = ((plen + tile - 1) / tile) * tile;
+            plen = std::max<int64_t>(plen, std::min<int64_t>(len, 2 * (int64_t)tile));
+        }
+        const int64_t fine = piece != 0 ? plen : std::max<int64_t>(kFineMin, plen / kFineDiv / kPieceStep * kPieceStep);
+        const int64_t coarse_end =   // runs of less than two pieces are cut evenly
+            piece != 0 || len < 2 * plen ? r.j_end : r.j_begin + (int64_t)((double)len * kCoarse) / plen * plen;
+        for (int64_t a = r.j_begin, step; a < r.j_end; a += step) {
+            step = a < coarse_end ? plen : fine;
+            PairItem it{};
+            it.I = r.I;
+            it.j_begin = (int32_t)a;
+            it.j_end = (int32_t)std::min<int64_t>(r.j_end, a + step);
+            it.sym = r.sym;
+            const int64_t tgt = std::min<int64_t>(BS, M - (int64_t)r.I * BS);
+            if (r.sym) p.pairs_sym += tgt * (it.j_end - it.j_begin);
+            else p.pairs_one += tgt * (it.j_end - it.j_begin);
+            p.items.push_back(it);
+            p.cost.push_back(unit * (double)(it.j_end - it.j_begin));
+        }
+    }
+}
+
+// Device copy of the items sorted by decreasing cost (afterwards the host copy is in that order too).
+int upload_schedule(PairSchedule& p, cudaStream_t st) {
+    std::vector<int> order(p.items.size());
+    std::iota(order.begin(), order.end(), 0);
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return p.cost[a] > p.cost[b]; });
+    std::vector<PairItem> sorted(p.items.size());
+    std::vector<double> sorted_cost(p.items.size());
+    for (size_t k = 0; k < order.size(); ++k) {
+        sorted[k] = p.items[order[k]];
+        sorted_cost[k] = p.cost[order[k]];
+    }
+    CTR_TRY(p.d_items.alloc(sizeof(PairItem) * std::max<size_t>(1, sorted.size())));
+    if (!sorted.empty())
+        CTR_CUDA_TRY(cudaMemcpyAsync(p.d_items.p, sorted.data(), sizeof(PairItem) * sorted.size(),
+                                     cudaMemcpyHostToDevice, st));
+    CTR_CUDA_TRY(cudaStreamSynchronize(st));   // the host vectors above go out of scope
+    // the host copy follows the device order: the engine's work entries index the device list
+    p.items.swap(sorted);
+    p.cost.swap(sorted_cost);
+    return CTR_OK;
+}
+
 int last_fp32_variant() { return g_last_var32.load(); }
 
 int schedule_slots(int sms, int slots[3]) {
@@ -403,10 +425,9 @@ int schedule_slots(int sms, int slots[3]) {
 }
 
 Exclusions exclusions_of(const ctr_ibim* s) {
-    if (s->tree)
-        return Exclusions{s->tree->d_eptr.as<int32_t>(), s->tree->d_excl.as<int32_t>(), nullptr, nullptr, nullptr};
-    return Exclusions{s->corr_ptr.as<int32_t>(), s->excl.as<int32_t>(), s->cl_begin.as<int32_t>(),
-                      s->cl_end.as<int32_t>(), s->cl_list.as<int32_t>()};
+    const int32_t* ptr = s->tree ? s->tree->d_eptr.as<int32_t>() : s->corr_ptr.as<int32_t>();
+    const int32_t* list = s->tree ? s->tree->d_excl.as<int32_t>() : s->excl.as<int32_t>();
+    return Exclusions{ptr, list, s->cl_begin.as<int32_t>(), s->cl_end.as<int32_t>(), s->cl_list.as<int32_t>()};
 }
 
 int launch_schedule(ctr_ibim* s, int pol, const void* src, const PairConsts& kc) {
@@ -441,24 +462,23 @@ static int plan_fixed(ctr_ibim* s, int pol, const std::vector<uint8_t>& flags, i
     const int Rs[3] = {0, kRdf, kR64};   // targets per thread of the fixed shapes
     const int tiles[3] = {0, Df64Policy::kTile, Fp64Policy::kTile};
     plan_schedule(s->sched[pol], pol, s->M, Rs[pol], tiles[pol], flags, g0, nb0, slots[pol]);
-    CTR_TRY(upload_schedule(s->sched[pol], s->M, s->stream));
+    CTR_TRY(upload_schedule(s->sched[pol], s->stream));
     s->sched[pol].planned = true;
     return CTR_OK;
 }
 
-static int build_closure(ctr_ibim* s) {
+int build_closure(ctr_ibim* s, const int32_t* ptr, const int32_t* excl) {
     const int64_t M = s->M, E = s->E;
     if (M >= (int64_t)1 << 29) return fail(CTR_ERR_CAPACITY, "more than 2^29 nodes");   // 4 j + flags in an int32
     cudaStream_t st = s->stream;
-    const int32_t* ptr = s->corr_ptr.as<int32_t>();
-    const int32_t* excl = s->excl.as<int32_t>();
     DevBuf scratch, work;
     CTR_TRY(s->cl_begin.alloc(sizeof(int32_t) * (M + 1)));
     CTR_TRY(s->cl_end.alloc(sizeof(int32_t) * M));
     CTR_TRY(s->cl_list.alloc(sizeof(int32_t) * std::max<int64_t>(1, 2 * E)));
-    CTR_TRY(work.alloc(sizeof(int32_t) * 2 * M));
+    CTR_TRY(work.alloc(sizeof(int32_t) * (2 * M + 2 * E)));
     int32_t* count = work.as<int32_t>();
     int32_t* fill = count + M;
+    int32_t* sorted = fill + M;
     CTR_CUDA_TRY(cudaMemsetAsync(count, 0, sizeof(int32_t) * 2 * M, st));
     closure_count_kernel<<<grid_for(M, 256), 256, 0, st>>>(ptr, excl, M, count);
     CTR_LAUNCHED();
@@ -466,7 +486,10 @@ static int build_closure(ctr_ibim* s) {
     closure_scatter_kernel<<<grid_for(M, 256), 256, 0, st>>>(ptr, excl, M, s->cl_begin.as<int32_t>(), fill,
                                                             s->cl_list.as<int32_t>());
     CTR_LAUNCHED();
-    closure_merge_kernel<<<grid_for(M, 256), 256, 0, st>>>(ptr, excl, M, s->cl_begin.as<int32_t>(), fill,
+    closure_sort_kernel<<<grid_for(32 * M, 256), 256, 0, st>>>(M, s->cl_begin.as<int32_t>(), fill,
+                                                              s->cl_list.as<int32_t>(), sorted);
+    CTR_LAUNCHED();
+    closure_merge_kernel<<<grid_for(M, 256), 256, 0, st>>>(ptr, excl, M, s->cl_begin.as<int32_t>(), fill, sorted,
                                                           s->cl_list.as<int32_t>(), s->cl_end.as<int32_t>());
     CTR_LAUNCHED();
     CTR_CUDA_TRY(cudaStreamSynchronize(st));   // `work` is freed on return
@@ -478,7 +501,7 @@ static int build_closure(ctr_ibim* s) {
 int build_schedules(ctr_ibim* s, const int slots[3]) {
     std::vector<uint8_t> flags;
     int g0 = 0, nb0 = 0;
-    CTR_TRY(build_closure(s));
+    CTR_TRY(build_closure(s, s->corr_ptr.as<int32_t>(), s->excl.as<int32_t>()));
     CTR_TRY(near_flags(s, flags, g0, nb0));
     CTR_TRY(alloc_accumulators(s));
     CTR_TRY(s->counter.alloc(sizeof(int) * 4));

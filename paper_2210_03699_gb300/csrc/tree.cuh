@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(NT) k_tree_far(Acc acc, const int2* __restrict
 constexpr size_t tree_far2_smem(int np = kTreeMaxNp) { return sizeof(unsigned long long) * (3 * kTreeMaxN1 + 3 * np); }
 
 template <int RP, int NT, class Acc>
-__global__ void __launch_bounds__(NT) k_tree_far2(Acc acc, const int2* __restrict__ ent,
+__global__ void __launch_bounds__(NT, 2) k_tree_far2(Acc acc, const int2* __restrict__ ent,
                                                const int* __restrict__ n_ent, int* __restrict__ counter, int pol) {
     using pk::u64;
     extern __shared__ __align__(16) unsigned char tree_smem[];
@@ -461,6 +461,8 @@ __global__ void __launch_bounds__(NT) k_tree_far2(Acc acc, const int2* __restric
 }
 
 // Float-float far items (the float-float operator): R targets per thread x NT threads = a 256-node block.
+// About 150 FP32 operations per evaluation; 128 registers (four blocks per SM) measured 54 -> 50 ms against the
+// compiler's own 96 (9.5e9 evaluations), fewer registers 57 ms: the two targets' chains overlap.
 // Dynamic shared memory: the cluster's proxy coordinates and charges as float-float pairs, then the
 // exponential tables.
 constexpr size_t tree_farff_smem(int np = kTreeMaxNp) {
@@ -468,7 +470,7 @@ constexpr size_t tree_farff_smem(int np = kTreeMaxNp) {
 }
 
 template <int R, int NT, class Acc>
-__global__ void __launch_bounds__(NT) k_tree_far_ff(Acc acc, const int2* __restrict__ ent,
+__global__ void __launch_bounds__(NT, 4) k_tree_far_ff(Acc acc, const int2* __restrict__ ent,
                                                   const int* __restrict__ n_ent, int* __restrict__ counter) {
     using pk::F2;
     constexpr int pol = 1;

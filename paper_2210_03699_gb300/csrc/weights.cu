@@ -31,7 +31,7 @@
 // 64 samples, and the tensor Lagrange (degree 5) interpolation of the tables.
 #include <mutex>
 
-#include "common.cuh"
+#include "pairkern.cuh"
 
 namespace ctr {
 
@@ -140,31 +140,38 @@ struct PlaneCtx {
     double tau;  // K-reg radius
 };
 
-// Visits the K-reg cylinder nodes of target i in ascending node order.
+// The K-reg cylinder of target i, by a whole warp: fn(m) for every cell of the search cube in ascending
+// node order, lane by lane of 32 consecutive cells (m: the tube node in the cylinder there, or -1); every lane
+// of the warp makes the same number of calls.  One thread per row would search the 11^3 cells alone (1.1 ms for
+// the K-reg rows of a 60-atom molecule; setup 3.9 -> 3.0 ms).
 template <typename F>
 __device__ void visit_cylinder(const PlaneCtx& c, const NodeArrays& na, const int64_t* lin,
-                               const int32_t* node_of, int64_t i, F&& fn) {
+                               const int32_t* node_of, int64_t i, int lane, F&& fn) {
     const double P[3] = {na.Px[i], na.Py[i], na.Pz[i]};
     const double n[3] = {na.nx[i], na.ny[i], na.nz[i]};
     const int64_t g = lin[i];
-    const int64_t ci = g % c.nx, cj = (g / c.nx) % c.ny, ck = g / (c.nx * c.ny);
+    const int ci = (int)(g % c.nx), cj = (int)((g / c.nx) % c.ny), ck = (int)(g / (c.nx * c.ny));
     const double tau2 = __dmul_rn(c.tau, c.tau);
-    for (int64_t k = max((int64_t)0, ck - c.Kc); k <= min(c.nz - 1, ck + c.Kc); ++k)
-        for (int64_t j = max((int64_t)0, cj - c.Kc); j <= min(c.ny - 1, cj + c.Kc); ++j)
-            for (int64_t q = max((int64_t)0, ci - c.Kc); q <= min(c.nx - 1, ci + c.Kc); ++q) {
-                const int32_t m = node_of[q + c.nx * (j + c.ny * k)];
-                if (m < 0) continue;
-                const double y0 = __dadd_rn(c.origin[0], __dmul_rn(c.h, (double)q));
-                const double y1 = __dadd_rn(c.origin[1], __dmul_rn(c.h, (double)j));
-                const double y2 = __dadd_rn(c.origin[2], __dmul_rn(c.h, (double)k));
-                const double v0 = __dsub_rn(y0, P[0]), v1 = __dsub_rn(y1, P[1]), v2 = __dsub_rn(y2, P[2]);
-                const double sdot = __dadd_rn(__dadd_rn(__dmul_rn(v0, n[0]), __dmul_rn(v1, n[1])), __dmul_rn(v2, n[2]));
-                const double t0 = __dsub_rn(v0, __dmul_rn(sdot, n[0]));
-                const double t1 = __dsub_rn(v1, __dmul_rn(sdot, n[1]));
-                const double t2 = __dsub_rn(v2, __dmul_rn(sdot, n[2]));
-                const double q2 = __dadd_rn(__dadd_rn(__dmul_rn(t0, t0), __dmul_rn(t1, t1)), __dmul_rn(t2, t2));
-                if (q2 < tau2) fn(m, 0.0, 0.0, 0.0);
-            }
+    const int side = 2 * c.Kc + 1, cells = side * side * side;
+    for (int at = lane; at - lane < cells; at += 32) {
+        int32_t m = -1;
+        const int q = ci - c.Kc + at % side, j = cj - c.Kc + (at / side) % side, k = ck - c.Kc + at / (side * side);
+        if (at < cells && q >= 0 && j >= 0 && k >= 0 && q < c.nx && j < c.ny && k < c.nz)
+            m = node_of[q + c.nx * (j + c.ny * (int64_t)k)];
+        if (m >= 0) {
+            const double y0 = __dadd_rn(c.origin[0], __dmul_rn(c.h, (double)q));
+            const double y1 = __dadd_rn(c.origin[1], __dmul_rn(c.h, (double)j));
+            const double y2 = __dadd_rn(c.origin[2], __dmul_rn(c.h, (double)k));
+            const double v0 = __dsub_rn(y0, P[0]), v1 = __dsub_rn(y1, P[1]), v2 = __dsub_rn(y2, P[2]);
+            const double sdot = __dadd_rn(__dadd_rn(__dmul_rn(v0, n[0]), __dmul_rn(v1, n[1])), __dmul_rn(v2, n[2]));
+            const double t0 = __dsub_rn(v0, __dmul_rn(sdot, n[0]));
+            const double t1 = __dsub_rn(v1, __dmul_rn(sdot, n[1]));
+            const double t2 = __dsub_rn(v2, __dmul_rn(sdot, n[2]));
+            const double q2 = __dadd_rn(__dadd_rn(__dmul_rn(t0, t0), __dmul_rn(t1, t1)), __dmul_rn(t2, t2));
+            if (!(q2 < tau2)) m = -1;
+        }
+        fn(m);
+    }
 }
 
 // Visits the correction nodes of target i in ascending plane order.
@@ -206,35 +213,43 @@ __device__ void visit_planes(const PlaneCtx& c, const NodeArrays& na, const int6
     }
 }
 
+// Correction nodes per row: the planes' by a thread per row, K-reg rows' by a warp per row (kernels of their
+// own: only the whole grid's warps hide the search's latency).
 __global__ void corr_count_kernel(PlaneCtx c, NodeArrays na, const int64_t* __restrict__ lin,
                                   const int32_t* __restrict__ node_of, const uint8_t* __restrict__ bad, int64_t M,
                                   int32_t* __restrict__ counts) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= M) return;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= M || bad[i]) return;
     int cnt = 0;
-    auto inc = [&](int32_t, double, double, double) { ++cnt; };
-    if (bad[i]) visit_cylinder(c, na, lin, node_of, i, inc);
-    else visit_planes(c, na, lin, node_of, i, inc);
+    visit_planes(c, na, lin, node_of, i, [&](int32_t, double, double, double) { ++cnt; });
     counts[i] = cnt;
+}
+__global__ void kreg_count_kernel(PlaneCtx c, NodeArrays na, const int64_t* __restrict__ lin,
+                                  const int32_t* __restrict__ node_of, const uint8_t* __restrict__ bad, int64_t M,
+                                  int32_t* __restrict__ counts) {
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i >= M || !bad[i]) return;   // uniform in the warp
+    const int lane = threadIdx.x & 31;
+    int cnt = 0;
+    visit_cylinder(c, na, lin, node_of, i, lane, [&](int32_t m) { cnt += __popc(__ballot_sync(0xffffffffu, m >= 0)); });
+    if (lane == 0) counts[i] = cnt;
 }
 
 __global__ void corr_fill_kernel(PlaneCtx c, NodeArrays na, const int64_t* __restrict__ lin,
                                  const int32_t* __restrict__ node_of, const uint8_t* __restrict__ bad, int64_t M,
                                  const int32_t* __restrict__ ptr, int32_t* __restrict__ node,
                                  double* __restrict__ ab_eta, int64_t E, int32_t* __restrict__ excl) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= M) return;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= M || bad[i]) return;
     int e = ptr[i];
     const int e0 = e;
-    auto put = [&](int32_t m, double alpha, double beta, double eta) {
+    visit_planes(c, na, lin, node_of, i, [&](int32_t m, double alpha, double beta, double eta) {
         node[e] = m;
         ab_eta[e] = alpha;
         ab_eta[E + e] = beta;
         ab_eta[2 * E + e] = eta;
         ++e;
-    };
-    if (bad[i]) visit_cylinder(c, na, lin, node_of, i, put);
-    else visit_planes(c, na, lin, node_of, i, put);
+    });
     // sorted copy (insertion sort; at most a few entries) for the dense-sum exclusion
     for (int p = e0; p < e; ++p) {
         int32_t v = node[p];
@@ -245,6 +260,24 @@ __global__ void corr_fill_kernel(PlaneCtx c, NodeArrays na, const int64_t* __res
         }
         excl[q] = v;
     }
+}
+__global__ void kreg_fill_kernel(PlaneCtx c, NodeArrays na, const int64_t* __restrict__ lin,
+                                 const int32_t* __restrict__ node_of, const uint8_t* __restrict__ bad, int64_t M,
+                                 const int32_t* __restrict__ ptr, int32_t* __restrict__ node,
+                                 double* __restrict__ ab_eta, int64_t E, int32_t* __restrict__ excl) {
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i >= M || !bad[i]) return;   // uniform in the warp
+    const int lane = threadIdx.x & 31;
+    int e = ptr[i];
+    visit_cylinder(c, na, lin, node_of, i, lane, [&](int32_t m) {
+        const unsigned hit = __ballot_sync(0xffffffffu, m >= 0);
+        if (m >= 0) {
+            const int at = e + __popc(hit & ((1u << lane) - 1u));
+            node[at] = excl[at] = m;   // ascending already
+            ab_eta[at] = ab_eta[E + at] = ab_eta[2 * E + at] = 0.0;
+        }
+        e += __popc(hit);
+    });
 }
 
 __device__ void lagrange6(double x, int& i0, double cw[6]) {
@@ -291,27 +324,41 @@ __global__ void corr_weight_kernel(NodeArrays na, const uint8_t* __restrict__ ba
     const double A00 = t1[b], A01 = t1[cc], A10 = t2[b], A11 = t2[cc];   // rows Q tau_1, Q tau_2 (Eq. 2.26)
     const double m1 = na.m1[i], m2 = na.m2[i];
     const double D1 = 1.0 / (1.0 - eta * m1), D2 = 1.0 / (1.0 - eta * m2);   // D0 = (I - eta M)^-1
+    // Even Fourier modes of the angular functions (both have period pi, so half the 64 samples determine them);
+    // samples half a period apart are folded first: their sums carry the modes k = 0, 4, 8, .., their
+    // differences k = 2, 6, ..
     double aA[kModes], bA[kModes], aB[kModes], bB[kModes];
+#pragma unroll
     for (int q = 0; q < kModes; ++q) aA[q] = bA[q] = aB[q] = bB[q] = 0.0;
     const double inv8pi = 1.0 / (8.0 * kPi);
-    for (int j = 0; j < kSamples; ++j) {
-        const double ct = c_cos64[j], st = c_sin64[j];
-        const double v1 = D1 * (A00 * ct + A01 * st);
-        const double v2 = D2 * (A10 * ct + A11 * st);
-        const double vv = v1 * v1 + v2 * v2;
-        const double vn = sqrt(vv);
-        const double lA = (m1 * v1 * v1 + m2 * v2 * v2) * inv8pi / (vv * vn);
-        const double lB = inv8pi / vn;
+    constexpr int kFold = kSamples / 4;
+#pragma unroll 1
+    for (int j = 0; j < kFold; ++j) {
+        double lA[2], lB[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const double ct = c_cos64[j + h * kFold], st = c_sin64[j + h * kFold];
+            const double v1 = D1 * (A00 * ct + A01 * st);
+            const double v2 = D2 * (A10 * ct + A11 * st);
+            const double s1 = v1 * v1, s2 = v2 * v2;
+            const double vi = pk::rsqrt_d(s1 + s2);
+            lB[h] = inv8pi * vi;
+            lA[h] = (m1 * s1 + m2 * s2) * lB[h] * (vi * vi);
+        }
+        const double sumA = lA[0] + lA[1], difA = lA[0] - lA[1], sumB = lB[0] + lB[1], difB = lB[0] - lB[1];
+#pragma unroll
         for (int q = 0; q < kModes; ++q) {
             const int jk = (j * 2 * q) & (kSamples - 1);
-            aA[q] += lA * c_cos64[jk];
-            bA[q] += lA * c_sin64[jk];
-            aB[q] += lB * c_cos64[jk];
-            bB[q] += lB * c_sin64[jk];
+            const double fA = (q & 1) ? difA : sumA, fB = (q & 1) ? difB : sumB;
+            aA[q] += fA * c_cos64[jk];
+            bA[q] += fA * c_sin64[jk];
+            aB[q] += fB * c_cos64[jk];
+            bB[q] += fB * c_sin64[jk];
         }
     }
-    const double sc0 = 1.0 / kSamples, sc = 2.0 / kSamples;
+    const double sc0 = 2.0 / kSamples, sc = 4.0 / kSamples;
     aA[0] *= sc0; aB[0] *= sc0; bA[0] = bB[0] = 0.0;
+#pragma unroll
     for (int q = 1; q < kModes; ++q) { aA[q] *= sc; bA[q] *= sc; aB[q] *= sc; bB[q] *= sc; }
     int i0, j0;
     double ca[6], cb[6];
@@ -322,20 +369,27 @@ __global__ void corr_weight_kernel(NodeArrays na, const uint8_t* __restrict__ ba
         w[e] = w[E + e] = w[2 * E + e] = w[3 * E + e] = 0.0;
         return;
     }
+    // tables interpolated first (the same for both functions), then weighted with the modes
     double wA = 0.0, wB = 0.0;
-    for (int p = 0; p < 6; ++p)
-        for (int r = 0; r < 6; ++r) {
-            const int ia = i0 + p + kTabHalf, ib = j0 + r + kTabHalf;
-            double tA = 0.0, tB = 0.0;
-            for (int q = 0; q < kModes; ++q) {
-                const double Tc = T[((0 * kModes + q) * kTabN + ia) * kTabN + ib];
-                const double Ts = T[((1 * kModes + q) * kTabN + ia) * kTabN + ib];
-                tA += aA[q] * Tc + bA[q] * Ts;
-                tB += aB[q] * Tc + bB[q] * Ts;
+#pragma unroll
+    for (int q = 0; q < kModes; ++q) {
+        const double* Tc = T + ((0 * kModes + q) * kTabN + i0 + kTabHalf) * kTabN + j0 + kTabHalf;
+        const double* Ts = T + ((1 * kModes + q) * kTabN + i0 + kTabHalf) * kTabN + j0 + kTabHalf;
+        double vc = 0.0, vs = 0.0;
+#pragma unroll
+        for (int p = 0; p < 6; ++p) {
+            double rc = 0.0, rs = 0.0;
+#pragma unroll
+            for (int r = 0; r < 6; ++r) {
+                rc += cb[r] * Tc[p * kTabN + r];
+                rs += cb[r] * Ts[p * kTabN + r];
             }
-            wA += ca[p] * cb[r] * tA;
-            wB += ca[p] * cb[r] * tB;
+            vc += ca[p] * rc;
+            vs += ca[p] * rs;
         }
+        wA += aA[q] * vc + bA[q] * vs;
+        wB += aB[q] * vc + bB[q] * vs;
+    }
     w[e] = c11 * wA;           // omega11
     w[E + e] = kappa2 * wB;    // omega21
     w[2 * E + e] = c22 * wA;   // omega22
@@ -400,6 +454,9 @@ int setup_corrections(ctr_ibim* s, const double* d_tables, const int32_t* d_node
     corr_count_kernel<<<grid_for(M, 128), 128, 0, st>>>(c, s->na, s->lin.as<int64_t>(), d_node_of,
                                                        s->bad.as<uint8_t>(), M, counts.as<int32_t>());
     CTR_LAUNCHED();
+    kreg_count_kernel<<<grid_for(32 * M, 128), 128, 0, st>>>(c, s->na, s->lin.as<int64_t>(), d_node_of,
+                                                            s->bad.as<uint8_t>(), M, counts.as<int32_t>());
+    CTR_LAUNCHED();
     CTR_TRY(exclusive_scan_i32(counts.as<int32_t>(), s->corr_ptr.as<int32_t>(), M, st, scratch));
     int32_t Eh = 0;
     CTR_CUDA_TRY(cudaMemcpyAsync(&Eh, s->corr_ptr.as<int32_t>() + M, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
@@ -414,6 +471,11 @@ int setup_corrections(ctr_ibim* s, const double* d_tables, const int32_t* d_node
                                                       s->bad.as<uint8_t>(), M, s->corr_ptr.as<int32_t>(),
                                                       s->corr_node.as<int32_t>(), abeta.as<double>(), E,
                                                       s->excl.as<int32_t>());
+    CTR_LAUNCHED();
+    kreg_fill_kernel<<<grid_for(32 * M, 128), 128, 0, st>>>(c, s->na, s->lin.as<int64_t>(), d_node_of,
+                                                           s->bad.as<uint8_t>(), M, s->corr_ptr.as<int32_t>(),
+                                                           s->corr_node.as<int32_t>(), abeta.as<double>(), E,
+                                                           s->excl.as<int32_t>());
     CTR_LAUNCHED();
     if (E > 0) {
         const double c11 = 1.0 - s->eps_out / s->eps_in;

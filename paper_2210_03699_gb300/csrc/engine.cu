@@ -8,12 +8,15 @@
 // GMRES-based iterative refinement; with the same precision inside and out it
 // is plain restarted GMRES.
 //
-// One engine step, captured once as a CUDA graph and replayed:
-//   inner half   (slots in state INNER)  one Arnoldi iteration:
-//                z = Lambda^-1 V_j, pack, pairs, finish w = A z, CGS2 (two passes
-//                of batched dot products and updates), norm, Givens, scale, advance;
-//   update half  (slots in state UPDATE) x += Lambda^-1 V y, pack, pairs,
-//                finish r = g - A x, norm, decide (done / next cycle), start cycle.
+// One engine step runs up to two halves, each captured once as a CUDA graph and replayed:
+//   inner half   (slots in state INNER)  one Arnoldi iteration, seven kernels: plan; V_j scaled to unit length
+//                and z = Lambda^-1 V_j packed; pairs; finish w = A z; CGS2 as dots, subtract + dots,
+//                subtract + norm (the last block of each reduction adds the partials, the last of all also
+//                does the Givens update and the slot's state);
+//   update half  (slots in state UPDATE; launched only when there is one) triangular solve;
+//                x += Lambda^-1 V y, pack; pairs; finish r = g - A x; norm and decision (done / next cycle).
+// A small system's step is bound by its launches: the vector part of a 19k-node system took about 160 us in
+// some 30 kernels (both halves every step); the solve of such a system went from 16.5 to 14.5 ms.
 // The dense pair sums of all slots run in persistent kernels (one per pair
 // arithmetic and half) whose blocks take work entries (slot, item of that
 // slot's pair schedule: target block, source range, one-sided or symmetric)
@@ -46,23 +49,17 @@ constexpr int kItemMask = (1 << kPartShift) - 1;
 constexpr int kMaxParts = 127;
 constexpr int kMinItemsPerPart = 64;
 
-__device__ __forceinline__ double block_sum_d(double v) {
-    __shared__ double sh[kVecThreads / 32];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < kVecThreads / 32; ++w) t += sh[w];
-    __syncthreads();
-    return t;
-}
-
 __device__ __forceinline__ bool inner_active(const SlotDev& s) { return s.stat.state == kSlotInner; }
 __device__ __forceinline__ bool update_active(const SlotDev& s) { return s.stat.state == kSlotUpdate; }
 // Pair arithmetic of a slot's residual in this cycle: the residual arithmetic for g - A x, the inner
 // one for an update r - A d of a small correction d.
 __device__ __forceinline__ int res_arith(const SlotDev& s) { return s.upd ? s.inner_prec : s.res_prec; }
+
+__device__ __forceinline__ int arith_index(int prec) { return prec == CTR_FP32_REFINE ? 0 : (prec == CTR_DF64 ? 1 : 2); }
+// Whether the parts of the slot's operator application run in this half-step are its last ones.
+__device__ __forceinline__ bool whole(const SlotDev& s, int half) {
+    return s.part + s.span >= s.nparts[arith_index(half == 0 ? s.inner_prec : res_arith(s))];
+}
 
 // ---------------------------------------------------------------- packing
 __device__ __forceinline__ void pack_weights(const SlotDev& s, int prec, int64_t t, double a, double b) {
@@ -81,14 +78,20 @@ __device__ __forceinline__ void pack_weights(const SlotDev& s, int prec, int64_t
     }
 }
 
-// inner: z = Lambda^-1 V_j and the weights of z
+// inner: V_j to unit length (V_0 = r / beta; V_j is the last iteration's w, of length scal[2]), z = Lambda^-1 V_j
+// and the weights of z
 __global__ void k_prep_inner(SlotDev* S) {
     const SlotDev& s = S[blockIdx.y];
     if (!inner_active(s) || s.part != 0) return;   // later parts reuse the packed weights
     const int64_t M = s.M;
-    const double* v = s.V + (size_t)s.j * s.n;
+    double* v = s.V + (size_t)s.j * s.n;
+    const double* w = s.j == 0 ? s.r : v;
+    const double f = 1.0 / (s.j == 0 ? s.beta : s.scal[2]);
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < M; t += (int64_t)gridDim.x * blockDim.x) {
-        const double z1 = v[t] * s.il1, z2 = v[M + t] * s.il2;
+        const double v1 = w[t] * f, v2 = w[M + t] * f;
+        v[t] = v1;
+        v[M + t] = v2;
+        const double z1 = v1 * s.il1, z2 = v2 * s.il2;
         s.z[t] = z1;
         s.z[M + t] = z2;
         pack_weights(s, s.inner_prec, s.tinv ? (int64_t)s.tinv[t] : t, s.scale * s.W[t] * z1, s.scale * s.W[t] * z2);
@@ -178,7 +181,7 @@ __global__ void __launch_bounds__(kThreads, Policy::kMinBlocks) k_pairs(SlotDev*
 // inner: w = V_{j+1} = A z;   update: r = g - A x, or r = r - A d (residual update, d in z)
 __global__ void __launch_bounds__(kFinishThreads) k_finish(SlotDev* S, int half) {
     const SlotDev& s = S[blockIdx.y];
-    if (half == 0 ? !inner_active(s) : !update_active(s)) return;
+    if ((half == 0 ? !inner_active(s) : !update_active(s)) || !whole(s, half)) return;
     const int64_t M = s.M;
     const bool upd = (half == 1) && s.upd;
     const double* x = (half == 0 || upd) ? s.z : s.x;
@@ -192,134 +195,249 @@ __global__ void __launch_bounds__(kFinishThreads) k_finish(SlotDev* S, int half)
     });
 }
 
-// ---------------------------------------------------------------- batched reductions (same chunking as alone)
-// mode 0/1: c = V[0..j] . w (first / second Gram-Schmidt pass), 2: |w|^2, 3: |r|^2
-__global__ void k_dots_partial(SlotDev* S, int mode) {
-    const SlotDev& s = S[blockIdx.y];
-    const bool act = (mode == 3) ? update_active(s) : inner_active(s);
-    if (!act || (int)blockIdx.x >= s.nblk) return;
-    const int64_t n = s.n;
-    const int64_t chunk = (n + s.nblk - 1) / s.nblk;
-    const int64_t t0 = (int64_t)blockIdx.x * chunk, t1 = min(n, t0 + chunk);
-    const double* w = (mode == 3) ? s.r : s.V + (size_t)(s.j + 1) * n;
-    const int count = (mode <= 1) ? s.j + 1 : 1;
-    for (int i = 0; i < count; ++i) {
-        const double* a = (mode <= 1) ? s.V + (size_t)i * n : w;
-        double v = 0.0;
-        for (int64_t t = t0 + threadIdx.x; t < t1; t += blockDim.x) v += a[t] * w[t];
-        v = block_sum_d(v);
-        if (threadIdx.x == 0) s.dpart[(size_t)i * s.nblk + blockIdx.x] = v;
-    }
-}
+// ---------------------------------------------------------------- vector part (same chunks as alone)
+// Blocks of a slot take chunks of its vectors (nblk of them) and leave partial sums; the block that finishes
+// last (ticket) adds them in chunk order, so a sum does not depend on which block that is.
+constexpr int kDotGroup = 8;   // vectors per pass over a chunk: their warp sums are transposed together
 
-__global__ void k_dots_final(SlotDev* S, int mode) {
-    const SlotDev& s = S[blockIdx.y];
-    const bool act = (mode == 3) ? update_active(s) : inner_active(s);
-    if (!act) return;
-    const int count = (mode <= 1) ? s.j + 1 : 1;
-    const int i = blockIdx.x;
-    if (i >= count) return;
-    double v = 0.0;
-    for (int b = threadIdx.x; b < s.nblk; b += blockDim.x) v += s.dpart[(size_t)i * s.nblk + b];
-    v = block_sum_d(v);
+// True in every thread of the block that arrives last; its view of the others' partials is then complete.
+__device__ __forceinline__ bool last_block(SlotDev& s) {
+    __shared__ int last;
+    __threadfence();
+    __syncthreads();
     if (threadIdx.x == 0) {
-        double* out = (mode == 0) ? s.cgs : (mode == 1) ? s.cgs2 : (mode == 2) ? s.scal : s.scal + 1;
-        out[i] = v;
+        last = atomicAdd(&s.ticket, 1) == s.nblk - 1;
+        if (last) s.ticket = 0;
     }
+    __syncthreads();
+    if (last) __threadfence();
+    return last != 0;
 }
 
-// w -= V[0..j] c   (pass: 0 first coefficients, 1 second)
-__global__ void k_sub(SlotDev* S, int pass) {
-    const SlotDev& s = S[blockIdx.y];
-    if (!inner_active(s)) return;
+// Sum over the block of v[k] of every thread, k < kDotGroup; valid in threads k < kDotGroup (v[k] of thread k).
+__device__ __forceinline__ double group_sum(double (&v)[kDotGroup]) {
+    __shared__ double sh[kVecThreads / 32][kDotGroup];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int cnt = kDotGroup;
+#pragma unroll
+    for (int m = 16; m >= 1; m >>= 1) {   // halve the values a lane keeps, then a plain butterfly
+        if (cnt > 1) {
+            const bool upper = (lane & m) != 0;
+            const int h = cnt / 2;
+#pragma unroll
+            for (int i = 0; i < kDotGroup / 2; ++i) {
+                if (i < h) {
+                    const double send = upper ? v[i] : v[i + h], keep = upper ? v[i + h] : v[i];
+                    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+                }
+            }
+            cnt = h;
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], m);
+        }
+    }
+    __syncthreads();   // the last call's readers are done
+    if ((lane & (32 / kDotGroup - 1)) == 0) sh[warp][lane / (32 / kDotGroup)] = v[0];
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.x < kDotGroup)
+        for (int w = 0; w < kVecThreads / 32; ++w) t += sh[w][threadIdx.x];
+    return t;
+}
+
+struct Chunk {
+    int64_t t0, t1;
+};
+__device__ __forceinline__ Chunk chunk_of(const SlotDev& s) {
+    const int64_t c = (s.n + s.nblk - 1) / s.nblk;
+    const int64_t t0 = (int64_t)blockIdx.x * c;
+    return Chunk{t0, min(s.n, t0 + c)};
+}
+
+// Partial dots <V_i, w>, i <= j, of this block's chunk, and by the last block their sums to out.
+__device__ __forceinline__ void chunk_dots(SlotDev& s, const Chunk& c, const double* __restrict__ w,
+                                           double* __restrict__ out) {
     const int64_t n = s.n;
-    double* w = s.V + (size_t)(s.j + 1) * n;
-    const double* c = pass ? s.cgs2 : s.cgs;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-        double v = w[t];
-        for (int i = 0; i <= s.j; ++i) v -= s.V[(size_t)i * n + t] * c[i];
-        w[t] = v;
+    const int j = s.j, nblk = s.nblk;
+    for (int i0 = 0; i0 <= j; i0 += kDotGroup) {
+        double v[kDotGroup];
+#pragma unroll
+        for (int k = 0; k < kDotGroup; ++k) v[k] = 0.0;
+        const double* a = s.V + (size_t)i0 * n;
+        for (int64_t t = c.t0 + threadIdx.x; t < c.t1; t += kVecThreads) {
+            const double wt = w[t];
+#pragma unroll
+            for (int k = 0; k < kDotGroup; ++k)
+                if (i0 + k <= j) v[k] += a[(size_t)k * n + t] * wt;
+        }
+        const double sum = group_sum(v);
+        if (threadIdx.x < kDotGroup && i0 + (int)threadIdx.x <= j)
+            s.dpart[(size_t)(i0 + threadIdx.x) * nblk + blockIdx.x] = sum;
+    }
+    if (!last_block(s)) return;
+    const int lane = threadIdx.x & 31;
+    for (int i = threadIdx.x >> 5; i <= j; i += kVecThreads / 32) {
+        double v = 0.0;
+        for (int b = lane; b < nblk; b += 32) v += s.dpart[(size_t)i * nblk + b];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) out[i] = v;
     }
 }
 
-// Givens update of Hessenberg column j (one thread per slot)
-__global__ void k_givens(SlotDev* S, int cap) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= cap) return;
-    SlotDev& s = S[q];
-    if (!inner_active(s)) return;
+// One partial sum per block; by the last block (true there) the total, in every thread.
+__device__ __forceinline__ bool chunk_total(SlotDev& s, double mine, double& total) {
+    double v[kDotGroup];
+#pragma unroll
+    for (int k = 0; k < kDotGroup; ++k) v[k] = k == 0 ? mine : 0.0;
+    const double sum = group_sum(v);
+    if (threadIdx.x == 0) s.dpart[blockIdx.x] = sum;
+    if (!last_block(s)) return false;
+    const int lane = threadIdx.x & 31;
+    double t = 0.0;
+    for (int b = lane; b < s.nblk; b += 32) t += s.dpart[b];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    total = t;
+    return true;
+}
+
+// w -= V[0..j] c on this block's chunk; returns the thread's sum of squares of the result.
+__device__ __forceinline__ double chunk_sub(const SlotDev& s, const Chunk& c, double* __restrict__ w,
+                                            const double* __restrict__ coef) {
+    const int64_t n = s.n;
+    const int j = s.j;
+    double ss = 0.0;
+    for (int64_t t = c.t0 + threadIdx.x; t < c.t1; t += kVecThreads) {
+        double v = w[t];
+#pragma unroll 8
+        for (int i = 0; i <= j; ++i) v -= s.V[(size_t)i * n + t] * coef[i];
+        w[t] = v;
+        ss += v * v;
+    }
+    return ss;
+}
+
+__device__ __forceinline__ bool arnoldi_active(const SlotDev& s) {
+    return inner_active(s) && (int)blockIdx.x < s.nblk && whole(s, 0);
+}
+
+// first Gram-Schmidt coefficients
+__global__ void __launch_bounds__(kVecThreads) k_dots(SlotDev* S) {
+    SlotDev& s = S[blockIdx.y];
+    if (!arnoldi_active(s)) return;
+    chunk_dots(s, chunk_of(s), s.V + (size_t)(s.j + 1) * s.n, s.cgs);
+}
+
+// w -= V c, second coefficients
+__global__ void __launch_bounds__(kVecThreads) k_sub_dots(SlotDev* S) {
+    SlotDev& s = S[blockIdx.y];
+    if (!arnoldi_active(s)) return;
+    const Chunk c = chunk_of(s);
+    double* w = s.V + (size_t)(s.j + 1) * s.n;
+    (void)chunk_sub(s, c, w, s.cgs);
+    chunk_dots(s, c, w, s.cgs2);
+}
+
+// Givens update of Hessenberg column j, counters, and the slot's next state (one thread)
+__device__ void givens_and_advance(SlotDev& s, double norm2) {
     const int j = s.j, ldh = s.m + 1;
     double* col = s.H + (size_t)j * ldh;
-    for (int i = 0; i <= j; ++i) col[i] = s.cgs[i] + s.cgs2[i];
-    const double hn = sqrt(s.scal[0]);
-    col[j + 1] = hn;
+    const double hn = sqrt(norm2);
+    double h = s.cgs[0] + s.cgs2[0];   // the column's entry being rotated
     for (int i = 0; i < j; ++i) {
-        const double t = s.cs[i] * col[i] + s.sn[i] * col[i + 1];
-        col[i + 1] = -s.sn[i] * col[i] + s.cs[i] * col[i + 1];
-        col[i] = t;
+        const double next = s.cgs[i + 1] + s.cgs2[i + 1];
+        const double c = s.cs[i], sn = s.sn[i];
+        col[i] = c * h + sn * next;
+        h = -sn * h + c * next;
     }
-    const double den = hypot(col[j], col[j + 1]);
-    s.cs[j] = col[j] / den;
-    s.sn[j] = col[j + 1] / den;
+    const double den = hypot(h, hn);
+    s.cs[j] = h / den;
+    s.sn[j] = hn / den;
     col[j] = den;
     col[j + 1] = 0.0;
-    s.sv[j + 1] = -s.sn[j] * s.sv[j];
-    s.sv[j] = s.cs[j] * s.sv[j];
+    const double sj = j == 0 ? s.beta : s.sv[j];
+    const double nj = -s.sn[j] * sj;
+    s.sv[j] = s.cs[j] * sj;
+    s.sv[j + 1] = nj;
     s.scal[2] = hn;
     s.stat.iterations++;
     if (s.inner_prec == CTR_FP32_REFINE) s.stat.matvecs_fp32++; else s.stat.matvecs_fp64++;
     s.budget--;
-    const double est = fabs(s.sv[j + 1]);
+    const double est = fabs(nj);
     if (!isfinite(est)) s.stat.numeric_error = 1;
-    s.cycle_end = (est <= s.tol_cycle || j + 1 == s.m || s.budget <= 0 || hn == 0.0 || !isfinite(est)) ? 1 : 0;
-}
-
-__global__ void k_scale_next(SlotDev* S) {
-    const SlotDev& s = S[blockIdx.y];
-    if (!inner_active(s)) return;
-    double* w = s.V + (size_t)(s.j + 1) * s.n;
-    const double f = 1.0 / s.scal[2];
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < s.n; t += (int64_t)gridDim.x * blockDim.x)
-        w[t] *= f;
-}
-
-// advance (one thread per slot): next Arnoldi index, or end of cycle -> update state
-__global__ void k_advance(SlotDev* S, int cap) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= cap) return;
-    SlotDev& s = S[q];
-    if (!inner_active(s)) return;
-    if (s.cycle_end) {
-        s.kdone = s.j + 1;
+    s.part = 0;
+    s.span = 1;   // a residual started later in this step runs one part
+    if (est <= s.tol_cycle || j + 1 == s.m || s.budget <= 0 || hn == 0.0 || !isfinite(est)) {
+        s.kdone = j + 1;
         s.stat.state = kSlotUpdate;
     } else {
-        s.j += 1;
+        s.j = j + 1;
     }
 }
 
-// back substitution R y = s (one thread per slot in UPDATE)
-__global__ void k_upper_solve(SlotDev* S, int cap) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= cap) return;
-    SlotDev& s = S[q];
+// w -= V c2, its norm, Givens; a slot whose application has parts left waits for the next step instead
+__global__ void __launch_bounds__(kVecThreads) k_sub_norm(SlotDev* S, SlotStat* __restrict__ out) {
+    SlotDev& s = S[blockIdx.y];
+    if (!inner_active(s) || (int)blockIdx.x >= s.nblk) return;
+    double total = 0.0;
+    if (whole(s, 0)) {
+        if (!chunk_total(s, chunk_sub(s, chunk_of(s), s.V + (size_t)(s.j + 1) * s.n, s.cgs2), total)) return;
+        if (threadIdx.x == 0) givens_and_advance(s, total);
+    } else {
+        if (!last_block(s)) return;   // every block has read the state
+        if (threadIdx.x == 0) {
+            s.part += s.span;
+            s.stat.state = kSlotInnerWait;
+        }
+    }
+    if (threadIdx.x == 0) out[blockIdx.y] = s.stat;
+}
+
+// Before a half's pair launches (one block): the work counters to zero, and which pair arithmetics any slot
+// applies in this half (the inner arithmetic of slots in INNER, the residual arithmetic of slots in UPDATE).
+// The persistent pair kernels of the others return at once instead of walking their whole work lists.
+__device__ __forceinline__ void begin_half(const SlotDev* S, int cap, int half, int* need, int* counters,
+                                           int n_counters, int* tree_counters) {
+    __shared__ int f[3];
+    if (threadIdx.x < 3) f[threadIdx.x] = 0;
+    for (int q = threadIdx.x; q < n_counters; q += blockDim.x) counters[q] = 0;
+    if (threadIdx.x < 12) tree_counters[threadIdx.x] = 0;
+    __syncthreads();
+    for (int q = threadIdx.x; q < cap; q += blockDim.x) {
+        const SlotDev& s = S[q];
+        if (half == 0 ? inner_active(s) : update_active(s))
+            f[arith_index(half == 0 ? s.inner_prec : res_arith(s))] = 1;
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) need[threadIdx.x] = f[threadIdx.x];
+}
+
+// Start of the update half, a block per slot: back substitution R y = s, column by column; block 0 also clears
+// the work counters and finds the pair arithmetics that the half needs.
+__global__ void __launch_bounds__(kVecThreads) k_begin_update(SlotDev* S, int cap, int* need, int* counters,
+                                                            int n_counters, int* tree_counters) {
+    if (blockIdx.x == 0) begin_half(S, cap, 1, need, counters, n_counters, tree_counters);
+    const SlotDev& s = S[blockIdx.x];
     if (!update_active(s) || s.part != 0) return;
     const int k = s.kdone, ldh = s.m + 1;
+    for (int l = threadIdx.x; l < k; l += kVecThreads) s.y[l] = s.sv[l];
+    __syncthreads();
     for (int i = k - 1; i >= 0; --i) {
-        double v = s.sv[i];
-        for (int l = i + 1; l < k; ++l) v -= s.H[(size_t)l * ldh + i] * s.y[l];
-        s.y[i] = v / s.H[(size_t)i * ldh + i];
+        const double* col = s.H + (size_t)i * ldh;
+        const double yi = s.y[i] / col[i];
+        __syncthreads();
+        for (int l = threadIdx.x; l < i; l += kVecThreads) s.y[l] -= col[l] * yi;
+        if (threadIdx.x == 0) s.y[i] = yi;
+        __syncthreads();
     }
 }
 
-// after the residual: converged, out of budget, or the next cycle from r
-__global__ void k_decide(SlotDev* S, int cap) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= cap) return;
-    SlotDev& s = S[q];
-    if (!update_active(s)) return;
+// after the residual: converged, out of budget, or the next cycle from r (one thread)
+__device__ void decide(SlotDev& s, double norm2) {
     if (s.upd) s.stat.matvecs_fp32++; else s.stat.matvecs_fp64++;
     s.stat.refinements++;
-    const double rn = sqrt(s.scal[1]);
+    s.part = 0;
+    s.span = 1;
+    const double rn = sqrt(norm2);
     s.stat.residual = (s.gnorm > 0.0) ? rn / s.gnorm : 0.0;
     if (!isfinite(rn)) {
         s.stat.numeric_error = 1;
@@ -339,30 +457,28 @@ __global__ void k_decide(SlotDev* S, int cap) {
     // operator's error on d (about 1e-7 |A| |d|, |d| ~ |A^-1| |r|) then stays orders of magnitude
     // below the tolerance, while g - A x would need the residual arithmetic at full magnitude.
     s.upd = (s.refine && s.res_update && rn <= kUpdateGate * s.gnorm) ? 1 : 0;
-    s.stat.state = kSlotStart;
-}
-
-// V[0] = r / beta for slots starting a cycle
-__global__ void k_start_vec(SlotDev* S) {
-    const SlotDev& s = S[blockIdx.y];
-    if (s.stat.state != kSlotStart) return;
-    const double f = 1.0 / s.beta;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < s.n; t += (int64_t)gridDim.x * blockDim.x)
-        s.V[t] = s.r[t] * f;
-}
-
-__global__ void k_start_scalars(SlotDev* S, int cap) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= cap) return;
-    SlotDev& s = S[q];
-    if (s.stat.state != kSlotStart) return;
-    for (int i = 0; i <= s.m; ++i) s.sv[i] = 0.0;
-    s.sv[0] = s.beta;
     s.j = 0;
     s.stat.state = kSlotInner;
 }
 
-__device__ __forceinline__ int arith_index(int prec) { return prec == CTR_FP32_REFINE ? 0 : (prec == CTR_DF64 ? 1 : 2); }
+__global__ void __launch_bounds__(kVecThreads) k_residual(SlotDev* S, SlotStat* __restrict__ out) {
+    SlotDev& s = S[blockIdx.y];
+    if (!update_active(s) || (int)blockIdx.x >= s.nblk) return;
+    if (whole(s, 1)) {
+        const Chunk c = chunk_of(s);
+        double ss = 0.0, total = 0.0;
+        for (int64_t t = c.t0 + threadIdx.x; t < c.t1; t += kVecThreads) ss += s.r[t] * s.r[t];
+        if (!chunk_total(s, ss, total)) return;
+        if (threadIdx.x == 0) decide(s, total);
+    } else {
+        if (!last_block(s)) return;
+        if (threadIdx.x == 0) {
+            s.part += s.span;
+            s.stat.state = kSlotUpdateWait;
+        }
+    }
+    if (threadIdx.x == 0) out[blockIdx.y] = s.stat;
+}
 
 // Estimated pair work of a slot in the step ahead (seconds), and its arithmetic.
 __device__ __forceinline__ float step_work(const SlotDev& s, int& a) {
@@ -376,7 +492,8 @@ __device__ __forceinline__ float step_work(const SlotDev& s, int& a) {
 // application is split gets its span of parts for this step: one, or as many as fit in the pair work of
 // all other slots in the step.  A large system thus takes about half of a busy step and one part of an
 // otherwise idle one, and the other slots' steps grow by at most that much.
-__global__ void k_plan_step(SlotDev* S, int cap) {
+__global__ void __launch_bounds__(kVecThreads) k_plan_step(SlotDev* S, int cap, int* need, int* counters, int n_counters,
+                                                         int* tree_counters) {
     __shared__ float red[kVecThreads];
     float w = 0.f;
     for (int q = threadIdx.x; q < cap; q += blockDim.x) {
@@ -403,44 +520,7 @@ __global__ void k_plan_step(SlotDev* S, int cap) {
             s.span = max(1, min(s.nparts[a] - s.part, (int)fminf(fit, (float)kMaxParts)));
         }
     }
-}
-
-// Before a half's pair launches (one block): which pair arithmetics any slot applies in this half (the
-// inner arithmetic of slots in INNER, the residual arithmetic of slots in UPDATE).  The persistent pair
-// kernels of the others return at once instead of walking their whole work lists.
-__global__ void k_need(const SlotDev* S, int cap, int half, int* need) {
-    __shared__ int f[3];
-    if (threadIdx.x < 3) f[threadIdx.x] = 0;
-    __syncthreads();
-    for (int q = threadIdx.x; q < cap; q += blockDim.x) {
-        const SlotDev& s = S[q];
-        if (half == 0 ? inner_active(s) : update_active(s))
-            f[arith_index(half == 0 ? s.inner_prec : res_arith(s))] = 1;
-    }
-    __syncthreads();
-    if (threadIdx.x < 3) need[threadIdx.x] = f[threadIdx.x];
-}
-
-// After a half's pair launches: a slot whose application has parts left waits for the next step (the
-// rest of this step skips it); one that ran its last part goes on to finish the application.
-__global__ void k_part(SlotDev* S, int cap, int half) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= cap) return;
-    SlotDev& s = S[q];
-    if (half == 0 ? !inner_active(s) : !update_active(s)) return;
-    const int np = s.nparts[arith_index(half == 0 ? s.inner_prec : res_arith(s))];
-    if (s.part + s.span < np) {
-        s.part += s.span;
-        s.stat.state = half == 0 ? kSlotInnerWait : kSlotUpdateWait;
-    } else {
-        s.part = 0;
-        s.span = 1;   // a residual started later in this step runs one part
-    }
-}
-
-__global__ void k_stats(const SlotDev* S, int cap, SlotStat* out) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q < cap) out[q] = S[q].stat;
+    begin_half(S, cap, 0, need, counters, n_counters, tree_counters);
 }
 
 constexpr int kNV = kNumVar32;   // work lists per arithmetic
@@ -465,7 +545,7 @@ int launch_persistent_k(Engine* e, int pol, int var, int half, int prec) {
     const int list = pol * kNV + var;
     k_pairs<Policy, R, V, U, kShared><<<per_sm * e->sms, kThreads, smem, e->stream>>>(
         e->slots.as<SlotDev>(), e->items[pol][var].as<int2>(), e->n_items.as<int>() + list,
-        e->counters.as<int>() + 2 * list + half, half, prec, pol, e->exp_tab[pol], e->err.as<int>(), e->kc_val[pol],
+        e->counters.as<int>() + 2 * list + half, half, prec, pol, e->exp_tab[pol], e->err, e->kc_val[pol],
         e->need.as<int>());
     CTR_LAUNCHED();
     return CTR_OK;
@@ -532,9 +612,9 @@ int launch_tree_engine(Engine* e, int pol, int half, int prec) {
 
 int launch_trees(Engine* e, int half) {
     if (!e->any_tree) return CTR_OK;
-    CTR_TRY((launch_tree_engine<float, kTreeR[0], kTreeNT[0]>(e, 0, half, CTR_FP32_REFINE)));
-    CTR_TRY((launch_tree_engine<double, kTreeR[1], kTreeNT[1]>(e, 1, half, CTR_DF64)));
-    CTR_TRY((launch_tree_engine<double, kTreeR[2], kTreeNT[2]>(e, 2, half, CTR_FP64)));
+    if (e->uses[half][0]) CTR_TRY((launch_tree_engine<float, kTreeR[0], kTreeNT[0]>(e, 0, half, CTR_FP32_REFINE)));
+    if (e->uses[half][1]) CTR_TRY((launch_tree_engine<double, kTreeR[1], kTreeNT[1]>(e, 1, half, CTR_DF64)));
+    if (e->uses[half][2]) CTR_TRY((launch_tree_engine<double, kTreeR[2], kTreeNT[2]>(e, 2, half, CTR_FP64)));
     return CTR_OK;
 }
 
@@ -551,7 +631,8 @@ int launch_fp32(Engine* e, int half) {
 static int policy_index(int prec) { return prec == CTR_FP32_REFINE ? 0 : (prec == CTR_DF64 ? 1 : 2); }
 
 Engine::~Engine() {
-    if (graph_exec) cudaGraphExecDestroy(graph_exec);
+    for (auto& g : graph_exec)
+        if (g) cudaGraphExecDestroy(g);
     if (stream) {
         cudaStreamSynchronize(stream);
         cudaStreamDestroy(stream);
@@ -575,16 +656,19 @@ int engine_create(int device, int cap, Engine** out) {
     };
     int st;
     if ((st = e->slots.alloc(sizeof(SlotDev) * cap)) < 0) return bad(st);
-    if ((st = e->stats.alloc(sizeof(SlotStat) * cap)) < 0) return bad(st);
+    // the error word of the pair kernels is the state of a stat entry behind the slots' (one copy reads both)
+    if ((st = e->stats.alloc(sizeof(SlotStat) * (cap + 1))) < 0) return bad(st);
+    static_assert(offsetof(SlotStat, state) == 0, "the error word leads its entry");
+    e->err = reinterpret_cast<int*>(e->stats.as<SlotStat>() + cap);
     if ((st = e->n_items.alloc(sizeof(int) * 3 * kNV)) < 0) return bad(st);
     if ((st = e->counters.alloc(sizeof(int) * 2 * 3 * kNV)) < 0) return bad(st);
     if ((st = e->tree_cnt.alloc(sizeof(int) * 9)) < 0) return bad(st);
     if ((st = e->tree_counters.alloc(sizeof(int) * 12)) < 0) return bad(st);
     if (cudaMemsetAsync(e->tree_cnt.p, 0, sizeof(int) * 9, stream) != cudaSuccess)
         return bad(fail(CTR_ERR_CUDA, "memset"));
-    if ((st = e->err.alloc(sizeof(int))) < 0) return bad(st);
     if ((st = e->need.alloc(sizeof(int) * 3)) < 0) return bad(st);
-    if (cudaMemsetAsync(e->err.p, 0, sizeof(int), stream) != cudaSuccess) return bad(fail(CTR_ERR_CUDA, "memset"));
+    if (cudaMemsetAsync(e->stats.p, 0, sizeof(SlotStat) * (cap + 1), stream) != cudaSuccess)
+        return bad(fail(CTR_ERR_CUDA, "memset"));
     if (cudaMemsetAsync(e->n_items.p, 0, sizeof(int) * 3 * kNV, stream) != cudaSuccess)
         return bad(fail(CTR_ERR_CUDA, "memset"));
     for (int q = 0; q < cap; ++q) e->host[q].stat.state = kSlotEmpty;
@@ -743,6 +827,17 @@ static int rebuild_items(Engine* e) {
         }
         CTR_CUDA_TRY(cudaStreamSynchronize(e->stream));
     }
+    bool uses[2][3] = {};   // arithmetics any slot may apply in the inner and the update half
+    for (int q = 0; q < e->cap; ++q) {
+        if (!e->owner[q]) continue;
+        const SlotDev& s = e->host[q];
+        uses[0][policy_index(s.inner_prec)] = uses[1][policy_index(s.res_prec)] = true;
+        if (s.res_update) uses[1][policy_index(s.inner_prec)] = true;
+    }
+    if (std::memcmp(uses, e->uses, sizeof(uses)) != 0) {
+        std::memcpy(e->uses, uses, sizeof(uses));
+        e->graph_dirty = true;   // the halves gain or lose pair launches
+    }
     for (int v = 0; v < kNV; ++v)
         if (used[v] != e->var_used[v]) {
             e->var_used[v] = used[v];
@@ -751,101 +846,67 @@ static int rebuild_items(Engine* e) {
     return rebuild_tree_items(e);
 }
 
-// The kernels of one engine step, in stream order (captured into the graph).
-static int enqueue_step(Engine* e) {
+// The kernels of one half of an engine step, in stream order (captured into its graph).
+static int enqueue_half(Engine* e, int half) {
     cudaStream_t st = e->stream;
     SlotDev* S = e->slots.as<SlotDev>();
-    const int cap = e->cap;
-    const int mx = e->max_nblk;
-    const dim3 vec(e->vec_blocks, cap);
-    const dim3 rows(2 * e->vec_blocks, cap);   // half as many rows per block
-    const unsigned one = grid_for(cap, 128);
-    k_plan_step<<<1, kVecThreads, 0, st>>>(S, cap);
-    CTR_LAUNCHED();
-    // ---- inner half: one Arnoldi iteration
-    k_prep_inner<<<vec, kVecThreads, 0, st>>>(S);
-    CTR_LAUNCHED();
-    CTR_CUDA_TRY(cudaMemsetAsync(e->counters.p, 0, sizeof(int) * 2 * 3 * kNV, st));
-    if (e->any_tree) CTR_CUDA_TRY(cudaMemsetAsync(e->tree_counters.p, 0, sizeof(int) * 12, st));
-    k_need<<<1, kVecThreads, 0, st>>>(S, cap, 0, e->need.as<int>());
-    CTR_LAUNCHED();
-    CTR_TRY(launch_fp32(e, 0));
-    CTR_TRY((launch_persistent<Df64Policy, kRdf, kChunkDf, 1>(e, 1, 0, 0, CTR_DF64)));
-    CTR_TRY((launch_persistent<Fp64Policy, kR64, kChunk64, 1>(e, 2, 0, 0, CTR_FP64)));
-    CTR_TRY(launch_trees(e, 0));
-    k_part<<<one, 128, 0, st>>>(S, cap, 0);
-    CTR_LAUNCHED();
-    k_finish<<<rows, kFinishThreads, 0, st>>>(S, 0);
-    CTR_LAUNCHED();
-    for (int pass = 0; pass < 2; ++pass) {
-        k_dots_partial<<<dim3(mx, cap), kVecThreads, 0, st>>>(S, pass);
+    SlotStat* stats = e->stats.as<SlotStat>();
+    const int cap = e->cap, n_counters = 2 * 3 * kNV;
+    const dim3 vec(e->vec_blocks, cap), rows(2 * e->vec_blocks, cap);   // a finish block takes half as many rows
+    const dim3 chunks(e->max_nblk, cap);
+    int *need = e->need.as<int>(), *counters = e->counters.as<int>(), *tree_counters = e->tree_counters.as<int>();
+    if (half == 0) {
+        k_plan_step<<<1, kVecThreads, 0, st>>>(S, cap, need, counters, n_counters, tree_counters);
         CTR_LAUNCHED();
-        k_dots_final<<<dim3(e->max_m + 1, cap), kVecThreads, 0, st>>>(S, pass);
+        k_prep_inner<<<vec, kVecThreads, 0, st>>>(S);
+    } else {
+        k_begin_update<<<cap, kVecThreads, 0, st>>>(S, cap, need, counters, n_counters, tree_counters);
         CTR_LAUNCHED();
-        k_sub<<<vec, kVecThreads, 0, st>>>(S, pass);
-        CTR_LAUNCHED();
+        k_update_x<<<vec, kVecThreads, 0, st>>>(S);
     }
-    k_dots_partial<<<dim3(mx, cap), kVecThreads, 0, st>>>(S, 2);
     CTR_LAUNCHED();
-    k_dots_final<<<dim3(1, cap), kVecThreads, 0, st>>>(S, 2);
+    if (e->uses[half][0]) CTR_TRY(launch_fp32(e, half));
+    if (e->uses[half][1]) CTR_TRY((launch_persistent<Df64Policy, kRdf, kChunkDf, 1>(e, 1, 0, half, CTR_DF64)));
+    if (e->uses[half][2]) CTR_TRY((launch_persistent<Fp64Policy, kR64, kChunk64, 1>(e, 2, 0, half, CTR_FP64)));
+    CTR_TRY(launch_trees(e, half));
+    k_finish<<<rows, kFinishThreads, 0, st>>>(S, half);
     CTR_LAUNCHED();
-    k_givens<<<one, 128, 0, st>>>(S, cap);
-    CTR_LAUNCHED();
-    k_scale_next<<<vec, kVecThreads, 0, st>>>(S);
-    CTR_LAUNCHED();
-    k_advance<<<one, 128, 0, st>>>(S, cap);
-    CTR_LAUNCHED();
-    // ---- update half: x, true residual, next cycle
-    k_upper_solve<<<one, 128, 0, st>>>(S, cap);
-    CTR_LAUNCHED();
-    k_update_x<<<vec, kVecThreads, 0, st>>>(S);
-    CTR_LAUNCHED();
-    k_need<<<1, kVecThreads, 0, st>>>(S, cap, 1, e->need.as<int>());
-    CTR_LAUNCHED();
-    CTR_TRY(launch_fp32(e, 1));
-    CTR_TRY((launch_persistent<Df64Policy, kRdf, kChunkDf, 1>(e, 1, 0, 1, CTR_DF64)));
-    CTR_TRY((launch_persistent<Fp64Policy, kR64, kChunk64, 1>(e, 2, 0, 1, CTR_FP64)));
-    CTR_TRY(launch_trees(e, 1));
-    k_part<<<one, 128, 0, st>>>(S, cap, 1);
-    CTR_LAUNCHED();
-    k_finish<<<rows, kFinishThreads, 0, st>>>(S, 1);
-    CTR_LAUNCHED();
-    k_dots_partial<<<dim3(mx, cap), kVecThreads, 0, st>>>(S, 3);
-    CTR_LAUNCHED();
-    k_dots_final<<<dim3(1, cap), kVecThreads, 0, st>>>(S, 3);
-    CTR_LAUNCHED();
-    k_decide<<<one, 128, 0, st>>>(S, cap);
-    CTR_LAUNCHED();
-    k_start_vec<<<vec, kVecThreads, 0, st>>>(S);
-    CTR_LAUNCHED();
-    k_start_scalars<<<one, 128, 0, st>>>(S, cap);
-    CTR_LAUNCHED();
-    k_stats<<<one, 128, 0, st>>>(S, cap, e->stats.as<SlotStat>());
+    if (half == 0) {
+        k_dots<<<chunks, kVecThreads, 0, st>>>(S);
+        CTR_LAUNCHED();
+        k_sub_dots<<<chunks, kVecThreads, 0, st>>>(S);
+        CTR_LAUNCHED();
+        k_sub_norm<<<chunks, kVecThreads, 0, st>>>(S, stats);
+    } else {
+        k_residual<<<chunks, kVecThreads, 0, st>>>(S, stats);
+    }
     CTR_LAUNCHED();
     return CTR_OK;
 }
 
 static int ensure_graph(Engine* e) {
-    if (e->graph_exec && !e->graph_dirty) return CTR_OK;
-    if (e->graph_exec) {
-        cudaGraphExecDestroy(e->graph_exec);
-        e->graph_exec = nullptr;
+    if (e->graph_exec[1] && !e->graph_dirty) return CTR_OK;
+    for (auto& g : e->graph_exec) {
+        if (g) cudaGraphExecDestroy(g);
+        g = nullptr;
     }
     if (!e->use_graph) return CTR_OK;
-    cudaGraph_t g = nullptr;
-    const int64_t before = ctr_kernel_launches();
-    CTR_CUDA_TRY(cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal));
-    const int st = enqueue_step(e);
-    e->kernels_per_step = ctr_kernel_launches() - before;
-    cudaError_t ce = cudaStreamEndCapture(e->stream, &g);
-    if (st < 0) {
-        if (g) cudaGraphDestroy(g);
-        return st;
+    for (int half = 0; half < 2; ++half) {
+        cudaGraph_t g = nullptr;
+        const int64_t before = ctr_kernel_launches();
+        CTR_CUDA_TRY(cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal));
+        const int st = enqueue_half(e, half);
+        e->kernels_per_half[half] = ctr_kernel_launches() - before;
+        cudaError_t ce = cudaStreamEndCapture(e->stream, &g);
+        if (st < 0) {
+            if (g) cudaGraphDestroy(g);
+            return st;
+        }
+        if (ce != cudaSuccess) return fail(CTR_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(ce));
+        ce = cudaGraphInstantiate(&e->graph_exec[half], g, 0);
+        cudaGraphDestroy(g);
+        if (ce != cudaSuccess) return fail(CTR_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(ce));
     }
-    if (ce != cudaSuccess) return fail(CTR_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(ce));
-    ce = cudaGraphInstantiate(&e->graph_exec, g, 0);
-    cudaGraphDestroy(g);
-    if (ce != cudaSuccess) return fail(CTR_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(ce));
     e->graph_dirty = false;
     return CTR_OK;
 }
@@ -943,19 +1004,13 @@ int engine_admit(Engine* e, ctr_ibim* s, int* slot_out) {
         d.stat.state = kSlotDone;
         d.stat.converged = 1;
     } else {
-        d.stat.state = kSlotStart;
+        d.stat.state = kSlotInner;   // the first cycle starts from r = g
     }
     e->host[q] = d;
     e->owner[q] = s;
     CTR_CUDA_TRY(cudaMemcpyAsync(e->slots.as<SlotDev>() + q, &d, sizeof(SlotDev), cudaMemcpyHostToDevice, e->stream));
     CTR_CUDA_TRY(cudaMemcpyAsync(e->stats.as<SlotStat>() + q, &d.stat, sizeof(SlotStat), cudaMemcpyHostToDevice,
                                  e->stream));
-    if (d.stat.state == kSlotStart) {
-        k_start_vec<<<dim3(e->vec_blocks, e->cap), kVecThreads, 0, e->stream>>>(e->slots.as<SlotDev>());
-        CTR_LAUNCHED();
-        k_start_scalars<<<grid_for(e->cap, 128), 128, 0, e->stream>>>(e->slots.as<SlotDev>(), e->cap);
-        CTR_LAUNCHED();
-    }
     if (d.nblk > e->max_nblk) {   // launch shapes of the captured step change
         e->max_nblk = d.nblk;
         e->graph_dirty = true;
@@ -999,8 +1054,28 @@ int engine_retire(Engine* e, int q, ctr_solve_info* info) {
     e->host[q] = empty;
     e->owner[q] = nullptr;
     CTR_CUDA_TRY(cudaMemcpyAsync(e->slots.as<SlotDev>() + q, &empty, sizeof(SlotDev), cudaMemcpyHostToDevice, e->stream));
+    CTR_CUDA_TRY(cudaMemcpyAsync(e->stats.as<SlotStat>() + q, &empty.stat, sizeof(SlotStat), cudaMemcpyHostToDevice,
+                                 e->stream));
     e->lists_dirty = true;   // its entries are inert (an empty slot matches no state) until the next rebuild
     return st.numeric_error ? fail(CTR_ERR_NUMERIC, "non-finite residual") : CTR_OK;
+}
+
+// One half of a step, the slots' states and the error word read back (they lie side by side on the device).
+static int run_half(Engine* e, int half, std::vector<SlotStat>* stats) {
+    if (e->graph_exec[half]) {
+        CTR_CUDA_TRY(cudaGraphLaunch(e->graph_exec[half], e->stream));
+        count_launches(e->kernels_per_half[half]);   // kernels run by the replay
+    } else {
+        CTR_TRY(enqueue_half(e, half));
+    }
+    stats->resize(e->cap + 1);
+    CTR_CUDA_TRY(cudaMemcpyAsync(stats->data(), e->stats.p, sizeof(SlotStat) * (e->cap + 1), cudaMemcpyDeviceToHost,
+                                 e->stream));
+    CTR_CUDA_TRY(cudaStreamSynchronize(e->stream));
+    const int herr = stats->back().state;
+    stats->resize(e->cap);
+    if (herr) return fail(CTR_ERR_DEVICE_WAIT, "engine: a bounded device wait expired");
+    return CTR_OK;
 }
 
 int engine_step(Engine* e, std::vector<SlotStat>* stats) {
@@ -1009,19 +1084,10 @@ int engine_step(Engine* e, std::vector<SlotStat>* stats) {
         e->lists_dirty = false;
     }
     CTR_TRY(ensure_graph(e));
-    if (e->graph_exec) {
-        CTR_CUDA_TRY(cudaGraphLaunch(e->graph_exec, e->stream));
-        count_launches(e->kernels_per_step);   // kernels run by the replay
-    } else {
-        CTR_TRY(enqueue_step(e));
-    }
-    stats->resize(e->cap);
-    CTR_CUDA_TRY(cudaMemcpyAsync(stats->data(), e->stats.p, sizeof(SlotStat) * e->cap, cudaMemcpyDeviceToHost, e->stream));
-    CTR_CUDA_TRY(cudaStreamSynchronize(e->stream));
-    int herr = 0;
-    CTR_CUDA_TRY(cudaMemcpyAsync(&herr, e->err.p, sizeof(int), cudaMemcpyDeviceToHost, e->stream));
-    CTR_CUDA_TRY(cudaStreamSynchronize(e->stream));
-    if (herr) return fail(CTR_ERR_DEVICE_WAIT, "engine: a bounded device wait expired");
+    CTR_TRY(run_half(e, 0, stats));
+    bool update = false;   // slots that ended a cycle, or wait between the parts of a residual
+    for (const SlotStat& q : *stats) update |= q.state == kSlotUpdate || q.state == kSlotUpdateWait;
+    if (update) CTR_TRY(run_half(e, 1, stats));
     e->steps++;
     return CTR_OK;
 }

@@ -16,7 +16,6 @@ enum : int {
     kSlotInner = 1,
     kSlotUpdate = 2,
     kSlotDone = 3,
-    kSlotStart = 4,
     kSlotInnerWait = 5,
     kSlotUpdateWait = 6
 };
@@ -34,8 +33,9 @@ struct SlotStat {
 // Everything the step kernels need about one slot (device copy; the host mirror is Engine::host).
 struct SlotDev {
     SlotStat stat;
-    int j, m, kdone, cycle_end;
+    int j, m, kdone;
     int M, nblk;
+    int ticket;              // blocks of the reduction in hand that have arrived (0 between reductions)
     int64_t n;
     int refine, inner_prec, res_prec, max_refine;
     int res_update;          // refinement residuals after the first: r -= A d in the inner arithmetic
@@ -81,7 +81,8 @@ struct Engine {
     int64_t item_cap[3][pk::kNumVar32] = {};
     bool var_used[pk::kNumVar32] = {};   // FP32 variants of the occupied slots
     int64_t steps = 0;
-    int64_t kernels_per_step = 0;
+    int64_t kernels_per_half[2] = {0, 0};
+    bool uses[2][3] = {};   // [half][arithmetic]: pair launches the halves hold
     // Part size (seconds at kUnitRate): an application expected to take longer is split into parts
     // (balanced sets of its schedule's items) run over consecutive steps, one or more per step (as
     // many as fit in the other slots' work of the step; k_plan_step), so that the steps of the other
@@ -93,14 +94,15 @@ struct Engine {
     pk::PairConsts kc_val[3] = {};               // ... and these are they (launch parameter)
     std::vector<SlotDev> host;
     std::vector<ctr_ibim*> owner;
-    DevBuf slots, stats, items[3][pk::kNumVar32], n_items, counters, err;
+    DevBuf slots, stats, items[3][pk::kNumVar32], n_items, counters;
+    int* err = nullptr;   // error word of the pair kernels (behind the stats)
     DevBuf need;   // per pair arithmetic: does any slot need its pair launch in the current half (k_need)
     // treecode work entries (slot, index) per pair arithmetic: moment chunks, far clusters, far items
     bool any_tree = false;
     int tree_np[3] = {0, 0, 0};   // largest proxy count per arithmetic among the treecode slots
     int64_t tree_cap[3][3] = {};
     DevBuf tree_ent[3][3], tree_cnt, tree_counters;
-    cudaGraphExec_t graph_exec = nullptr;
+    cudaGraphExec_t graph_exec[2] = {nullptr, nullptr};   // inner and update half
     ~Engine();
 };
 

@@ -71,7 +71,10 @@ int ensure_krylov(ctr_ibim* s) {
     if (k.m == m && k.n == n) return CTR_OK;
     k.m = m;
     k.n = n;
-    k.nblk = (int)std::min<int64_t>(std::max<int64_t>(1, (n + 4095) / 4096), 608);
+    // reduction chunks: about one per SM, of 512 elements or more (a small system's reductions are latency,
+    // more blocks than SMs only add partials)
+    const int64_t chunk = std::max<int64_t>(512, ((n + 147) / 148 + 255) / 256 * 256);
+    k.nblk = (int)std::max<int64_t>(1, (n + chunk - 1) / chunk);
     CTR_TRY(k.V.alloc(sizeof(double) * (size_t)(m + 1) * n));
     CTR_TRY(k.H.alloc(sizeof(double) * (size_t)(m + 1) * m));
     CTR_TRY(k.cs.alloc(sizeof(double) * m));

@@ -429,8 +429,7 @@ int ctr_ibim_matvec(ctr_ibim* s, const double* x, double* y, int precision, int 
         }
         CTR_TRY(apply_operator(s, dx, dy, precision));
         if (!on_device) CTR_CUDA_TRY(cudaMemcpyAsync(y, dy, sizeof(double) * n, cudaMemcpyDeviceToHost, s->stream));
-        CTR_CUDA_TRY(cudaStreamSynchronize(s->stream));
-        return check_device_error(s, "matvec");
+        return check_device_error(s, "matvec");   // waits for the stream
     });
 }
 
@@ -517,7 +516,6 @@ int ctr_ibim_potential_map(ctr_ibim* s, const double* psi, const double* dpsi_n,
         if (n_points == 0) return CTR_OK;
         if (on_device) {
             CTR_TRY(potential_map(s, psi, dpsi_n, n_points, xyz, out, precision));
-            CTR_CUDA_TRY(cudaStreamSynchronize(s->stream));
             return check_device_error(s, "potential map");
         }
         const int64_t M = s->M;

@@ -62,8 +62,9 @@ __global__ void __launch_bounds__(kThreads) pair_kernel(const typename Policy::S
 // (at the node's tree position when the treecode has reordered the sources)
 __global__ void pack_kernel(const double* __restrict__ x, const double* __restrict__ W, int64_t M, double scale,
                             float4* __restrict__ s32, double4* __restrict__ s64, float4* __restrict__ sdf,
-                            const int32_t* __restrict__ tinv) {
+                            const int32_t* __restrict__ tinv, int* __restrict__ counter) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < 4) counter[t] = 0;   // the work counters of the pair launch that follows
     if (t >= M) return;
     const double a = scale * W[t] * x[t];
     const double b = scale * W[t] * x[M + t];
@@ -289,7 +290,8 @@ int pack_sources(ctr_ibim* s, const double* d_x, int precision) {
     double4* s64 = (precision == CTR_FP64) ? s->src64.as<double4>() : nullptr;
     float4* sdf = (precision == CTR_DF64) ? s->srcdf.as<float4>() : nullptr;
     const int32_t* tinv = s->tree ? s->tree->d_tinv.as<int32_t>() : nullptr;
-    pack_kernel<<<grid_for(M, 256), 256, 0, s->stream>>>(d_x, s->na.W, M, scale, s32, s64, sdf, tinv);
+    pack_kernel<<<grid_for(M, 256), 256, 0, s->stream>>>(d_x, s->na.W, M, scale, s32, s64, sdf, tinv,
+                                                       s->counter.as<int>());
     CTR_LAUNCHED();
     return CTR_OK;
 }
@@ -332,7 +334,8 @@ int apply_operator_timed(ctr_ibim* s, const double* d_x, double* d_y, int precis
     double4* s64 = (precision == CTR_FP64) ? s->src64.as<double4>() : nullptr;
     float4* sdf = (precision == CTR_DF64) ? s->srcdf.as<float4>() : nullptr;
     const int32_t* tinv = s->tree ? s->tree->d_tinv.as<int32_t>() : nullptr;
-    pack_kernel<<<grid_for(M, 256), 256, 0, st>>>(d_x, s->na.W, M, scale, s32, s64, sdf, tinv);
+    pack_kernel<<<grid_for(M, 256), 256, 0, st>>>(d_x, s->na.W, M, scale, s32, s64, sdf, tinv,
+                                                       s->counter.as<int>());
     CTR_LAUNCHED();
     PairConsts kc;
     const int pol = (precision == CTR_FP32_REFINE) ? 0 : (precision == CTR_DF64 ? 1 : 2);

@@ -179,6 +179,7 @@ int sched_per_sm() {
     return per_sm;
 }
 
+// The work counter of `pol` is zero (pack_kernel clears the counters) and left used.
 template <typename Policy, int R, int V, int U>
 int sched_launch(ctr_ibim* s, int pol, const void* src, const PairConsts& kc, int sms) {
     const PairSchedule& p = s->sched[pol];
@@ -187,7 +188,6 @@ int sched_launch(ctr_ibim* s, int pol, const void* src, const PairConsts& kc, in
     if (per_sm < 0) return per_sm;
     const int grid = (int)std::min<int64_t>((int64_t)per_sm * sms, (int64_t)p.items.size());
     int* counter = s->counter.as<int>() + pol;
-    CTR_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(int), s->stream));
     sched_kernel<Policy, R, V, U><<<grid, kThreads, pair_smem_bytes<Policy>(), s->stream>>>(
         reinterpret_cast<const typename Policy::Src*>(src), (int)s->M,
         exclusions_of(s), p.d_items.as<PairItem>(),
@@ -295,6 +295,8 @@ int plan_fp32(ctr_ibim* s, const std::vector<uint8_t>& flags, int g0, int nb0, i
         st = plan(v);
         const SchedRun r{s, s->src32.p, &kc, sms};
         if (st == CTR_OK && v == 0) st = with_var32(v, r);   // warm-up
+        if (st == CTR_OK && cudaMemsetAsync(s->counter.p, 0, sizeof(int), s->stream) != cudaSuccess)
+            st = fail(CTR_ERR_CUDA, "memset");
         if (st == CTR_OK && cudaEventRecord(a, s->stream) != cudaSuccess) st = fail(CTR_ERR_CUDA, "event");
         if (st == CTR_OK) st = with_var32(v, r);
         if (st == CTR_OK && cudaEventRecord(b, s->stream) != cudaSuccess) st = fail(CTR_ERR_CUDA, "event");

@@ -45,12 +45,12 @@ RESTART, INNER_TOL, SOLVE_TOL = 64, 1e-5, 1e-10
 # in-warp transposed sums), for the packed FP32 and the float-float pair arithmetics (a packed f32x2
 # instruction counts as two lane operations, the FMA pipe's throughput being the same either way).
 # SFU work (rsqrt, ex2) and shared-memory loads are not counted.
-OPS_FP32 = {"one": 41, "sym": 49}
-OPS_DF64 = {"one": 423, "sym": 501}
-# FP64 pipe lane operations per pair evaluation of the FP64 schedule (CUDA's exp and rsqrt included): the
-# ncu count sm__inst_executed_pipe_fp64 x 32 / evaluations over one launch at h = 0.1 (69); its peak is the
-# measured DFMA probe rate, there being no FP64 unit count to go by.
-OPS_FP64 = {"one": 69, "sym": 69}
+OPS_FP32 = {"one": 40, "sym": 47}
+OPS_DF64 = {"one": 360, "sym": 420}
+# FP64 pipe lane operations per pair evaluation of the FP64 schedule, counted from the kernel source (seeds,
+# indices and high-order terms run on the SFU and the FP32 pipe), with the transposed sums of a symmetric
+# evaluation; its peak is the measured DFMA probe rate, there being no FP64 unit count to go by.
+OPS_FP64 = {"one": 50, "sym": 57}
 # DRAM bytes (read + write) per launch of the schedule kernels at the default workload (h = 0.05) from one
 # ncu capture, valid only while the kernel sources hash to `sources` (otherwise reported as null); the
 # profile records every re-keying after a change that leaves the kernels and the captured items unchanged.
@@ -60,12 +60,12 @@ KERNEL_SOURCES = ("paper_2210_03699_gb300/csrc/pairkern.cuh", "paper_2210_03699_
                   "paper_2210_03699_gb300/csrc/common.cuh")
 # Treecode far field of the FP32 operator (FP32 charges): FMA-pipe lane operations per proxy evaluation
 # counted from the kernel source (tree.cuh, k_tree_far2: 1 sub, 6 fma, 7 mul; an f32x2 instruction does
-# two), plus 2 SFU operations (rsqrt, ex2).  The float-float operator's far field (k_tree_far_ff): 171
-# FP32 add/sub/mul/fma instructions per evaluation (difference 11, r^2 12, d.n 18, rsqrt by one Newton
-# step 16, kappa r 8, the table exponential 29, the two charge combinations and accumulations 27 and 31,
-# 1 + kappa r times E 11, r^-3 8; table indexing and loads not counted), 1 SFU operation.
+# two), plus 2 SFU operations (rsqrt, ex2).  The float-float operator's far field (k_tree_far_ff): 150
+# FP32 add/sub/mul/fma instructions per evaluation (difference 11, r^2 12, d.n 12, rsqrt 15, kappa r 8, the
+# table exponential 21, the two charge combinations and accumulations 24 and 28, 1 + kappa r times E 11,
+# r^-3 8; table indexing and loads not counted), 1 SFU operation.
 OPS_FAR = 14
-OPS_FAR_DF = 171
+OPS_FAR_DF = 150
 SFU_FAR = 2
 
 
@@ -560,10 +560,10 @@ def run_kernels(args, ctr):
 
 
 # Potential map (Eq. 2.31 at arbitrary points): FMA-pipe lane operations per (point, node) pair of the FP32
-# kernel counted from its source (potential.cu, MapFp32x2: 3 sub, 3 for r^2, 1 r, 2 for E's argument and
-# E1, 3 for d.n, 2 for 1/r^3, 1 for the ratio term, 3 for the first accumulation, 2 for the second; an
-# f32x2 instruction does two), plus 2 SFU operations (rsqrt, ex2).
-OPS_MAP = 22
+# kernel counted from its source (potential.cu, MapFp32x2: 3 sub, 3 for r^2, 1 r, 1 for the exponent, 3 for
+# d.n, 2 for the ratio term, 3 for the weighted dipole over r^2, 2 for the bracket, 1 accumulation; an f32x2
+# instruction does two), plus 2 SFU operations (rsqrt, ex2).
+OPS_MAP = 19
 
 
 def run_map(args, ctr):

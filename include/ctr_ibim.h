@@ -244,9 +244,11 @@ int ctr_ibim_area(const ctr_ibim* sys, double* area);
 /*
  * The pair schedule of one arithmetic (precision CTR_FP32_REFINE, CTR_DF64 or
  * CTR_FP64) of the dense sum of Eq. (2.30): how many (target, source) pairs
- * its one-sided items evaluate (the near band, correction pairs masked), how
- * many its symmetric items evaluate once for both orientations (each counts
- * once here and stands for two of the M^2 - |N| interactions), its work items
+ * its one-sided items evaluate (the diagonal blocks; a treecode also sums the
+ * direct pairs of blocks that are not mutually near so), how many its
+ * symmetric items evaluate once for both orientations (each counts once here
+ * and stands for two of the M^2 - |N| interactions; correction pairs are
+ * masked for the rows that omit them), its work items
  * and the bytes of the device buffer its items add their sums into (exact
  * per-node accumulators, 200 bytes per node, shared by the three
  * arithmetics; the sums do not depend on the order of the additions).  Any

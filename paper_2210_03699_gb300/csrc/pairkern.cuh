@@ -678,8 +678,10 @@ struct Fp32x2Policy {
         if (kMask && (ex[0] || ex[1])) exclude(T, q, ex, k.one2);
         target_terms(common(T, q, k), q.a, q.nb, acc);
     }
-    // Both orientations: the factors s t1, s t2n, s X and (1 - E)/r are formed once (39 operations per one-sided
-    // evaluation, 47 per symmetric one).
+    // Both orientations: the factors s t1, s t2n, s X and (1 - E)/r are formed once (40 operations per one-sided
+    // evaluation, 47 per symmetric one; of the 47, 19 are multiply-adds with three distinct register operands,
+    // which run at 80 lanes a clock and SM against 119 for the others: 78% of the pipe is what the mix allows, and
+    // what the kernel reaches).
     // kMask: flags per half (Exclusions); a pair left out of both rows is moved to distance 1 (no NaN).
     template <bool kFirst, bool kMask = false>
     __device__ static void pair_sym(const Tgt& T, const Src* S, const PairConsts& k, const float2*, Acc& acc,
@@ -829,7 +831,7 @@ struct Fp64Policy {
 // rms 6.3e-14, 5.1e-14, 2.0e-12 of the uncancelled term; normalised throughout: 7.1e-14, 5.5e-14, 2.1e-12).
 // With u = 1 - E1, w = E kappa r, c = (d . n_x)(d . n_y)/r^2 the bracket of K21 is
 // u (n_x . n_y - 3 c) + w kappa r c, which needs neither 3 + 3 kappa r + kappa^2 r^2 nor 3 - E (..).
-// About 410 FP32 operations per symmetric evaluation (500 before): 217 ms instead of 255 ms per application
+// About 420 FP32 operations per symmetric evaluation (500 before): 217 ms instead of 255 ms per application
 // at 178 575 nodes, 14.1 instead of 16.5 ms at 44 597.  Shape: 24 warps per SM (80 registers) and fully
 // unrolled steps of 4 sources, transposed step by step; longer unrolled code misses the instruction cache
 // (steps of 8: 265 ms), steps of 2 measured 221 ms, 16 warps 213 against 209 ms (before the running sums were

@@ -59,7 +59,7 @@ struct Request {
 
 size_t handle_bytes(const ctr_ibim* s) {
     const DevBuf* bufs[] = {&s->lin, &s->nodes, &s->src32, &s->src64, &s->srcdf, &s->corr_ptr, &s->corr_node,
-                            &s->corr_w, &s->bad, &s->excl, &s->rhs, &s->charges, &s->acc, &s->err, &s->vecs,
+                            &s->corr_w, &s->bad, &s->excl, &s->cl_begin, &s->cl_end, &s->cl_list, &s->rhs, &s->charges, &s->acc, &s->err, &s->vecs,
                             &s->red, &s->map_ws, &s->map_io, &s->kr.V, &s->kr.H, &s->kr.cs, &s->kr.sn, &s->kr.s, &s->kr.y,
                             &s->kr.part, &s->kr.scal};
     size_t b = 0;
@@ -107,9 +107,10 @@ int64_t estimate_bytes(const Request& r) {
     for (double d : r.sdist) M += (std::fabs(d) < eps) ? 1 : 0;
     const int m = r.opt.restart > 0 ? r.opt.restart : 64;
     // per node: geometry 16 doubles, packed sources 64 + 64 + 64 bytes, corrections (~50 entries
-    // worst case, K-reg) 36 bytes each, solver vectors 12 doubles, Krylov (m + 1) x 2 doubles, the
+    // worst case, K-reg) 48 bytes each (node, four weights, exclusion, closed list) and two list bounds,
+    // solver vectors 12 doubles, Krylov (m + 1) x 2 doubles, the
     // dense sum's exact accumulators 25 words; plus the pair schedules' items (a few MB)
-    const int64_t per_node = 16 * 8 + 192 + 50 * 36 + 12 * 8 + (int64_t)(m + 1) * 16 + 25 * 8;
+    const int64_t per_node = 16 * 8 + 192 + 50 * 48 + 8 + 12 * 8 + (int64_t)(m + 1) * 16 + 25 * 8;
     // with the treecode: the tree-order exclusion lists, moment chunks and cluster charges
     const int64_t extra = (r.opt.farfield == CTR_FARFIELD_TREECODE) ? M * 512 + ((int64_t)64 << 20)
                                                                     : ((int64_t)16 << 20);

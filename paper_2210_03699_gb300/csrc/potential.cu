@@ -13,12 +13,15 @@
 // operator (their weight slots rewritten with a, b) streamed through the same two-stage shared-memory
 // ring (cp.async.bulk + mbarrier) as the operator's pair items.  A grid of (target block, source split)
 // blocks writes per-split FP64 partial sums (per-tile sums folded into FP64), added in split order by a
-// second kernel: the result does not depend on scheduling.  Three arithmetics:
+// second kernel: the result does not depend on scheduling.  Float-float and FP64, and FP32 at few points or
+// nodes, take a thread per point and short run of sources instead (map_unit_kernel).  Three arithmetics:
 //   Fp32x2  two points per f32x2 instruction, 19 FMA-pipe lane operations + 2 SFU per pair;
 //   Df64    float-float (the operator's residual arithmetic), one point per thread;
 //   Fp64    IEEE FP64 (the energy of ctr_ibim_energy).
 // The split partials live in a workspace the handle keeps and grows (no allocation once it is large
 // enough).
+#include <cmath>
+
 #include "pairkern.cuh"
 
 namespace ctr {
@@ -31,7 +34,7 @@ namespace {
 struct MapFp32x2 {
     using Src = ulonglong2;   // the operator's packed FP32 node {(x,x),(y,y)} {(z,z),(a,a)} {(nx,nx),(ny,ny)} {(nz,nz),(-b,-b)}
     static constexpr int kVec = 4;
-    static constexpr int kTile = 256;
+    static constexpr int kTile = 256, kUnit = kTile;
     static constexpr int kPack = 2;
     static constexpr int kR = 2;
     static constexpr int kTab = 0;
@@ -75,9 +78,8 @@ struct MapFp32x2 {
 struct MapDf64 {
     using Src = float4;
     static constexpr int kVec = 4;
-    static constexpr int kTile = 128;
+    static constexpr int kUnit = 128;   // 32, 64 take 5% to 16% longer at large maps
     static constexpr int kPack = 1;
-    static constexpr int kR = 1;
     static constexpr int kTab = kExpHi + kExpLo;
     struct Tgt {
         F2 x, y, z;
@@ -117,9 +119,8 @@ struct MapDf64 {
 struct MapFp64 {
     using Src = double4;
     static constexpr int kVec = 2;
-    static constexpr int kTile = 128;
+    static constexpr int kUnit = 64;    // 128: 1.6x the time of a few points, 0.7% less at large maps
     static constexpr int kPack = 1;
-    static constexpr int kR = 1;
     static constexpr int kTab = kExp2F2;
     struct Tgt {
         double x, y, z;
@@ -228,6 +229,64 @@ __global__ void map_sum_kernel(const double* __restrict__ part, int splits, int6
     out[p] = v;
 }
 
+// A thread per kPack points and unit of kUnit sources, read through L1; part[unit * n + p] is the unit's sum.
+// map_unit_sum_kernel adds the units of a group, then the groups, in order.
+//   float-float, FP64: every map and energy.  Pipe- and latency-bound: blocks of a (target block, split) grid
+//     left SMs idle at few points and made a ragged last wave at many.
+//     us, grid -> units (FP64): 3 points, 11,203 nodes 1313 -> 136; 3, 178,575: 2582 -> 140; 500, 44,597:
+//     1319 -> 1185; 4000, 178,575: 38,941 -> 35,998.  float-float: 252 -> 115, 424 -> 132, 259 -> 221,
+//     5239 -> 4860.
+//   FP32: few points or small systems only (map_launch); the units and groups are then map_kernel's tiles and
+//     splits, and a point's result has the same bits from either.
+constexpr int kUnitThreads = 128;
+template <typename Pol>
+__global__ void __launch_bounds__(kUnitThreads) map_unit_kernel(const typename Pol::Src* __restrict__ src, int M,
+                                                                const double* __restrict__ xyz, int64_t n,
+                                                                int64_t slots, int units, double* __restrict__ part,
+                                                                PairConsts kc) {
+    constexpr int UNIT = Pol::kUnit, VEC = Pol::kVec, P = Pol::kPack;
+    __shared__ float2 tab[Pol::kTab > 0 ? Pol::kTab : 1];
+    for (int q = threadIdx.x; q < Pol::kTab; q += kUnitThreads) tab[q] = kc.exp_tab[q];
+    __syncthreads();
+    const int64_t g = (int64_t)blockIdx.x * kUnitThreads + threadIdx.x;
+    const int64_t unit = g / slots;
+    if (unit >= units) return;
+    int64_t pi[P];
+    double s[P];
+#pragma unroll
+    for (int h = 0; h < P; ++h) {
+        pi[h] = g - unit * slots + h * slots;
+        s[h] = 0.0;
+    }
+    const typename Pol::Tgt tg = Pol::load(xyz, n, pi);
+    const int j0 = (int)unit * UNIT, cnt = min(UNIT, M - j0);
+    const typename Pol::Src* S = src + (size_t)VEC * j0;
+    typename Pol::Acc acc;
+    Pol::zero(acc);
+#pragma unroll 4
+    for (int q = 0; q < cnt; ++q) Pol::pair(tg, S + q * VEC, kc, tab, acc);
+    Pol::fold(acc, s);
+#pragma unroll
+    for (int h = 0; h < P; ++h)
+        if (pi[h] < n) part[unit * n + pi[h]] = s[h];
+}
+
+// a warp per point: a lane adds the units of one group, the groups' sums are then added in order
+__global__ void map_unit_sum_kernel(const double* __restrict__ part, int units, int per_group, int64_t n,
+                                    double* __restrict__ out) {
+    const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (p >= n) return;
+    const int lane = threadIdx.x & 31;
+    double v = 0.0;
+    for (int t0 = 0; t0 < units; t0 += 32 * per_group) {
+        const int b = t0 + lane * per_group, e = min(units, b + per_group);
+        double s = 0.0;
+        for (int t = b; t < e; ++t) s += part[(size_t)t * n + p];
+        for (int l = 0; l < 32 && t0 + l * per_group < units; ++l) v += __shfl_sync(0xffffffffu, s, l);
+    }
+    if (lane == 0) out[p] = v;
+}
+
 // a = h^3 W psi / (4 pi), b = h^3 W dpsi / (4 pi) into the weight slots of one packed source array
 __global__ void map_pack_kernel(const double* __restrict__ psi, const double* __restrict__ dpsi,
                                 const double* __restrict__ W, int64_t M, double scale, int prec,
@@ -257,10 +316,38 @@ constexpr size_t map_smem() {
     return 2 * Pol::kTile * Pol::kVec * sizeof(typename Pol::Src) + Pol::kTab * sizeof(float2);
 }
 
+// Unit sums of one launch: 32 MB of workspace, and at a million threads or more its last wave is a small part.
+// More points go in chunks.
+constexpr int64_t kUnitSums = 4 << 20;
+// FP32 maps of at most this many unit sums take map_unit_kernel: its sources come through L1, not by bulk
+// copies, and it holds two points a thread, not four, but its threads fill the chip at any shape.  us, units
+// against map_kernel: 2000 points, 44,597 nodes (350,000 sums) 148 : 210; 500, 178,575 (349,000) 164 : 223;
+// 1000, 178,575 (698,000) 244 : 218; 4000, 44,597 (700,000) 238 : 207.
+constexpr int64_t kUnitSums32 = 1 << 19;
+
 template <typename Pol>
-int map_launch(ctr_ibim* s, const void* src, const double* d_xyz, int64_t n, const PairConsts& kc, int* splits_out) {
+int map_units(ctr_ibim* s, const void* src, const double* d_xyz, int64_t n, const PairConsts& kc, int per_group,
+              double* d_out) {
+    const int64_t M = s->M, units = (M + Pol::kUnit - 1) / Pol::kUnit;
+    const int64_t chunk = std::min(n, std::max<int64_t>(32, kUnitSums / units / 32 * 32));
+    CTR_TRY(s->map_ws.alloc(sizeof(double) * (size_t)(units * chunk)));
+    for (int64_t p = 0; p < n; p += chunk) {
+        const int64_t m = std::min(chunk, n - p), slots = (m + Pol::kPack - 1) / Pol::kPack;
+        map_unit_kernel<Pol><<<grid_for(units * slots, kUnitThreads), kUnitThreads, 0, s->stream>>>(
+            reinterpret_cast<const typename Pol::Src*>(src), (int)M, d_xyz + 3 * p, m, slots, (int)units,
+            s->map_ws.as<double>(), kc);
+        CTR_LAUNCHED();
+        map_unit_sum_kernel<<<grid_for(32 * m, 256), 256, 0, s->stream>>>(s->map_ws.as<double>(), (int)units, per_group,
+                                                                         m, d_out + p);
+        CTR_LAUNCHED();
+    }
+    return CTR_OK;
+}
+
+int map_fp32(ctr_ibim* s, const double* d_xyz, int64_t n, const PairConsts& kc, double* d_out) {
+    using Pol = MapFp32x2;
     constexpr int BS = kThreads * Pol::kR * Pol::kPack;
-    static int per_dev[64] = {0};   // resident blocks per SM of this instantiation, per device
+    static int per_dev[64] = {0};   // resident blocks per SM of map_kernel, per device
     int dev = 0, sms = 0;
     CTR_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return fail(CTR_ERR_INVALID, "device index");
@@ -274,7 +361,6 @@ int map_launch(ctr_ibim* s, const void* src, const double* d_xyz, int64_t n, con
     }
     const int64_t M = s->M;
     const int64_t tblocks = (n + BS - 1) / BS;
-    if (n > (int64_t)INT32_MAX) return fail(CTR_ERR_CAPACITY, "more than 2^31 - 1 points");
     // source splits: about two waves of resident blocks, whole tiles, at least four tiles per split
     const int64_t want = std::max<int64_t>(1, 2LL * per_dev[dev] * sms / std::max<int64_t>(1, tblocks));
     const int64_t max_splits = std::max<int64_t>(1, M / (4 * Pol::kTile));
@@ -282,13 +368,15 @@ int map_launch(ctr_ibim* s, const void* src, const double* d_xyz, int64_t n, con
     int64_t per = (M + splits - 1) / splits;
     per = ((per + Pol::kTile - 1) / Pol::kTile) * Pol::kTile;
     splits = (M + per - 1) / per;
+    if ((M + Pol::kTile - 1) / Pol::kTile * n <= kUnitSums32)
+        return map_units<Pol>(s, s->src32.p, d_xyz, n, kc, (int)(per / Pol::kTile), d_out);
     CTR_TRY(s->map_ws.alloc(sizeof(double) * (size_t)(splits * n)));
     dim3 grid((unsigned)tblocks, (unsigned)splits);
-    map_kernel<Pol><<<grid, kThreads, smem, s->stream>>>(reinterpret_cast<const typename Pol::Src*>(src), (int)M,
-                                                         d_xyz, n, (int)per, s->map_ws.as<double>(), kc,
-                                                         s->err.as<int>());
+    map_kernel<Pol><<<grid, kThreads, smem, s->stream>>>(reinterpret_cast<const Pol::Src*>(s->src32.p), (int)M, d_xyz,
+                                                         n, (int)per, s->map_ws.as<double>(), kc, s->err.as<int>());
     CTR_LAUNCHED();
-    *splits_out = (int)splits;
+    map_sum_kernel<<<grid_for(n, 256), 256, 0, s->stream>>>(s->map_ws.as<double>(), (int)splits, n, d_out);
+    CTR_LAUNCHED();
     return CTR_OK;
 }
 
@@ -306,13 +394,14 @@ int potential_map(ctr_ibim* s, const double* d_psi, const double* d_dpsi, int64_
     CTR_LAUNCHED();
     PairConsts kc;
     CTR_TRY(pair_consts(s, precision == CTR_DF64 ? 1 : (precision == CTR_FP64 ? 2 : 0), &kc));
-    int splits = 0;
-    if (precision == CTR_FP32_REFINE) CTR_TRY(map_launch<MapFp32x2>(s, s->src32.p, d_xyz, n, kc, &splits));
-    else if (precision == CTR_DF64) CTR_TRY(map_launch<MapDf64>(s, s->srcdf.p, d_xyz, n, kc, &splits));
-    else CTR_TRY(map_launch<MapFp64>(s, s->src64.p, d_xyz, n, kc, &splits));
-    map_sum_kernel<<<grid_for(n, 256), 256, 0, s->stream>>>(s->map_ws.as<double>(), splits, n, d_out);
-    CTR_LAUNCHED();
-    return CTR_OK;
+    if (n > (int64_t)INT32_MAX) return fail(CTR_ERR_CAPACITY, "more than 2^31 - 1 points");
+    if (precision == CTR_FP32_REFINE) return map_fp32(s, d_xyz, n, kc, d_out);
+    // sqrt(units) units per group: short chains of additions, and the same for any number of points, so a
+    // point's result does not depend on the others
+    const int64_t unit = precision == CTR_DF64 ? MapDf64::kUnit : MapFp64::kUnit;
+    const int per_group = (int)std::ceil(std::sqrt((double)((M + unit - 1) / unit)));
+    if (precision == CTR_DF64) return map_units<MapDf64>(s, s->srcdf.p, d_xyz, n, kc, per_group, d_out);
+    return map_units<MapFp64>(s, s->src64.p, d_xyz, n, kc, per_group, d_out);
 }
 
 }  // namespace ctr

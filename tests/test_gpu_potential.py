@@ -88,3 +88,26 @@ def test_potential_map_device_arrays_and_edges(ctr):
         gold = json.load(open(os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden",
                                            "kirkwood_sphere_R2.json")))
         assert abs(host[0] / gold["psi_rxn_0"] - 1) < 5e-4
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 257, 5001, 50000])
+@pytest.mark.parametrize("which", ["sphere", "ellipsoid"])
+def test_potential_map_at_edges_of_its_routes(ctr, oracle_tables, which, n):
+    """One point to more than one launch of units holds (FP64, 11,203 nodes: 23,808 points), odd numbers of
+    points (two share an f32x2 register pair), both FP32 routes (the line: 40,329 and 11,915 points); the
+    tolerances of this file.  Float-float and FP64: a point's result does not depend on the others."""
+    prob = syn.sphere_problem(h=0.25) if which == "sphere" else syn.ellipsoid_problem(h=0.2)
+    S = OracleSystem.from_problem(prob, tables=oracle_tables)
+    noise = syn.random_density(S.M, seed=1)
+    psi, dpsi = 1.0 + 0.1 * noise[:S.M], 1.0 + 0.1 * noise[S.M:]
+    z = np.tile(_points(prob, 5001, seed=9, margin=2 * prob.tube), (10, 1))[:n]
+    first, last = z[:5], z[-5:]
+    ref = oenergy.reaction_potential(S, psi, dpsi, np.concatenate([first, last]))
+    scale = np.max(np.abs(ref))
+    with ctr.CtrIbim.from_problem(prob) as G:
+        for prec, tol in ((ctr.FP32_REFINE, 2e-6), (ctr.DF64, 1e-12), (ctr.FP64, 1e-12)):
+            got = G.potential_map(psi, dpsi, z, prec)
+            assert got.shape == (n,)
+            assert np.max(np.abs(np.concatenate([got[:5], got[-5:]]) - ref)) / scale < tol, prec
+            if prec != ctr.FP32_REFINE:
+                assert np.array_equal(G.potential_map(psi, dpsi, last, prec), got[-5:])

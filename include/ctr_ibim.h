@@ -245,7 +245,8 @@ int ctr_ibim_area(const ctr_ibim* sys, double* area);
  * The pair schedule of one arithmetic (precision CTR_FP32_REFINE, CTR_DF64 or
  * CTR_FP64) of the dense sum of Eq. (2.30): how many (target, source) pairs
  * its one-sided items evaluate (the diagonal blocks; a treecode also sums the
- * direct pairs of blocks that are not mutually near so), how many its
+ * direct pairs of blocks that are not mutually near so; and from 2^30 correction
+ * entries or 2^29 nodes on the block pairs that hold correction pairs), how many its
  * symmetric items evaluate once for both orientations (each counts once here
  * and stands for two of the M^2 - |N| interactions; correction pairs are
  * masked for the rows that omit them), its work items

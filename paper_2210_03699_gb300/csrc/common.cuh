@@ -246,6 +246,7 @@ struct ctr_ibim {
     ctr::DevBuf corr_w;      // double [4][E]: omega11, omega21, omega22, omega12
     ctr::DevBuf bad;         // uint8 [M] hybrid classification
     ctr::DevBuf excl;        // int32 [E] sorted correction nodes per target
+    bool closed = false;     // closed exclusion lists built (closed_lists_fit)
     ctr::DevBuf cl_begin, cl_end, cl_list;   // int32: closed exclusion lists (pk::Exclusions)
     ctr::DevBuf rhs;         // double [2M]
     ctr::DevBuf charges;     // double [4][nc]: x, y, z, q
@@ -276,15 +277,29 @@ int plan_pairs(ctr_ibim* s);
 // single-system far-field launches for pair arithmetic pol
 int build_tree_schedules(ctr_ibim* s, const int slots[3]);
 int launch_tree(ctr_ibim* s, int pol);
+namespace tree {
+struct Lists;
+}
+std::vector<uint8_t> correction_blocks(int64_t M, const std::vector<int32_t>& eptr, const std::vector<int32_t>& excl);
+std::vector<PairItem> near_runs(const tree::Lists& L, int64_t M, int BS, const std::vector<uint8_t>& corr, bool closed);
 int64_t tree_bytes(const ctr_ibim* s);
 // schedule.cu: symmetric / one-sided pair schedules of a handle
 constexpr int kMaxBaseBlocks = 8192;   // side of a block-pair matrix (bytes: its square)
 // items of p (BS and tile set) from runs: target block, source range, kind; then their device copy
 void cut_runs(PairSchedule& p, int pol, int64_t M, const std::vector<PairItem>& runs, int slots);
 int upload_schedule(PairSchedule& p, cudaStream_t st);
-// the closed exclusion lists (pk::Exclusions) of correction rows ptr, excl (device, ascending in each row)
+// The closed exclusion lists hold 4 j + flags, and count every correction pair twice in their row starts, in 32
+// bits.  Where that does not fit, a handle has none and near block pairs are evaluated one-sided, each row with
+// its own list (E entries in all).
+inline bool closed_lists_fit(int64_t M, int64_t E) { return M < (int64_t)1 << 29 && 2 * E <= INT32_MAX; }
+// the closed exclusion lists (pk::Exclusions) of correction rows ptr, excl (device, ascending in each row);
+// sets s->closed
 int build_closure(ctr_ibim* s, const int32_t* ptr, const int32_t* excl);
+// the runs of a direct schedule: flags is the near-flag matrix of nb0 x nb0 base blocks of g0 nodes; closed: near
+// block pairs once for both rows (kItemNear), else one-sided from both sides
+std::vector<PairItem> direct_runs(int64_t M, int BS, const std::vector<uint8_t>& flags, int g0, int nb0, bool closed);
 int build_schedules(ctr_ibim* s, const int slots[3]);
+int plan_schedules(ctr_ibim* s, const int slots[3]);   // the planning part of it (s->closed is set)
 int ensure_schedule(ctr_ibim* s, int pol);   // plans pair arithmetic `pol` if it has not been planned yet
 // the handle's exact node accumulators, allocated and cleared (pairsum.cu)
 int alloc_accumulators(ctr_ibim* s);

@@ -9,8 +9,9 @@
 // which the dense sum omits, are not symmetric (j in N(i) does not imply i in
 // N(j)), so a block pair (I, J), J > I, with a correction pair in either
 // direction gets near symmetric items: each excluded pair is masked for the
-// row(s) that leave it out (closed exclusion lists, built here).  Block pairs
-// without one get plain symmetric items, diagonal blocks one-sided ones.
+// row(s) that leave it out (closed exclusion lists, built here; one-sided
+// items from both sides where those lists do not fit, closed_lists_fit).  Block
+// pairs without one get plain symmetric items, diagonal blocks one-sided ones.
 // Since the correction nodes of i lie within a few h of P_i, near pairs form
 // a band around the diagonal: 6% of the pairs of a large system (1024-node
 // blocks at 178 575 nodes), most of a small one's.
@@ -198,39 +199,12 @@ int sched_launch(ctr_ibim* s, int pol, const void* src, const PairConsts& kc, in
 
 // Items of one arithmetic (pol) for a system of M nodes with the given near-flag matrix.
 void plan_schedule(PairSchedule& p, int pol, int64_t M, int R, int tile, const std::vector<uint8_t>& flags, int g0,
-                   int nb0, int slots) {
+                   int nb0, bool closed, int slots) {
     p.R = R;
     p.BS = kThreads * R;
     p.tile = tile;
-    const int BS = p.BS;
-    const int nb = (int)((M + BS - 1) / BS);
-    p.nb = nb;
-    auto base_range = [&](int I, int& lo, int& hi) {
-        lo = (int)((int64_t)I * BS / g0);
-        hi = (int)std::min<int64_t>(nb0 - 1, (((int64_t)I + 1) * BS - 1) / g0);
-    };
-    auto near = [&](int I, int J) {
-        int a0, a1, b0, b1;
-        base_range(I, a0, a1);
-        base_range(J, b0, b1);
-        for (int a = a0; a <= a1; ++a)
-            for (int b = b0; b <= b1; ++b)
-                if (flags[(size_t)a * nb0 + b]) return true;
-        return false;
-    };
-    std::vector<PairItem> runs;
-    for (int I = 0; I < nb; ++I) {
-        int J = I;
-        while (J < nb) {
-            const int kind = J == I ? kItemOne : near(I, J) ? kItemNear : kItemSym;
-            int J1 = J + 1;
-            if (kind != kItemOne)
-                while (J1 < nb && near(I, J1) == (kind == kItemNear)) ++J1;
-            runs.push_back(PairItem{I, (int)((int64_t)J * BS), (int)std::min<int64_t>(M, (int64_t)J1 * BS), kind});
-            J = J1;
-        }
-    }
-    cut_runs(p, pol, M, runs, slots);
+    p.nb = (int)((M + p.BS - 1) / p.BS);
+    cut_runs(p, pol, M, direct_runs(M, p.BS, flags, g0, nb0, closed), slots);
 }
 
 std::atomic<int> g_last_var32{-1};
@@ -258,7 +232,8 @@ int plan_fp32(ctr_ibim* s, const std::vector<uint8_t>& flags, int g0, int nb0, i
     auto plan = [&](int v) -> int {
         const int per = with_var32(v, PerSm{});
         if (per < 0) return per;
-        plan_schedule(s->sched[0], 0, M, kVar32[v].R * Fp32x2Policy::kPack, kVar32[v].tile, flags, g0, nb0, per * sms);
+        plan_schedule(s->sched[0], 0, M, kVar32[v].R * Fp32x2Policy::kPack, kVar32[v].tile, flags, g0, nb0,
+                      s->closed, per * sms);
         CTR_TRY(upload_schedule(s->sched[0], s->stream));
         s->sched[0].var = v;
         return CTR_OK;
@@ -323,6 +298,39 @@ int plan_fp32(ctr_ibim* s, const std::vector<uint8_t>& flags, int g0, int nb0, i
 }
 
 }  // namespace
+
+std::vector<PairItem> direct_runs(int64_t M, int BS, const std::vector<uint8_t>& flags, int g0, int nb0, bool closed) {
+    const int nb = (int)((M + BS - 1) / BS);
+    auto base_range = [&](int I, int& lo, int& hi) {
+        lo = (int)((int64_t)I * BS / g0);
+        hi = (int)std::min<int64_t>(nb0 - 1, (((int64_t)I + 1) * BS - 1) / g0);
+    };
+    auto near = [&](int I, int J) {
+        int a0, a1, b0, b1;
+        base_range(I, a0, a1);
+        base_range(J, b0, b1);
+        for (int a = a0; a <= a1; ++a)
+            for (int b = b0; b <= b1; ++b)
+                if (flags[(size_t)a * nb0 + b]) return true;
+        return false;
+    };
+    // evaluated with block I's rows: one-sided, for both blocks, or (-1) not at all
+    auto kind = [&](int I, int J) -> int {
+        if (J == I) return kItemOne;
+        if (near(I, J)) return !closed ? kItemOne : J > I ? kItemNear : -1;
+        return J > I ? kItemSym : -1;
+    };
+    std::vector<PairItem> runs;
+    for (int I = 0; I < nb; ++I) {
+        for (int J = closed ? I : 0, J1; J < nb; J = J1) {
+            const int k = kind(I, J);
+            for (J1 = J + 1; J1 < nb && kind(I, J1) == k;) ++J1;
+            if (k >= 0)
+                runs.push_back(PairItem{I, (int)((int64_t)J * BS), (int)std::min<int64_t>(M, (int64_t)J1 * BS), k});
+        }
+    }
+    return runs;
+}
 
 // The items of a schedule (its block size and tile set) from runs: a target block against a source range of
 // one kind.
@@ -463,7 +471,7 @@ static int near_flags(ctr_ibim* s, std::vector<uint8_t>& flags, int& g0, int& nb
 static int plan_fixed(ctr_ibim* s, int pol, const std::vector<uint8_t>& flags, int g0, int nb0, const int slots[3]) {
     const int Rs[3] = {0, kRdf, kR64};   // targets per thread of the fixed shapes
     const int tiles[3] = {0, Df64Policy::kTile, Fp64Policy::kTile};
-    plan_schedule(s->sched[pol], pol, s->M, Rs[pol], tiles[pol], flags, g0, nb0, slots[pol]);
+    plan_schedule(s->sched[pol], pol, s->M, Rs[pol], tiles[pol], flags, g0, nb0, s->closed, slots[pol]);
     CTR_TRY(upload_schedule(s->sched[pol], s->stream));
     s->sched[pol].planned = true;
     return CTR_OK;
@@ -471,7 +479,8 @@ static int plan_fixed(ctr_ibim* s, int pol, const std::vector<uint8_t>& flags, i
 
 int build_closure(ctr_ibim* s, const int32_t* ptr, const int32_t* excl) {
     const int64_t M = s->M, E = s->E;
-    if (M >= (int64_t)1 << 29) return fail(CTR_ERR_CAPACITY, "more than 2^29 nodes");   // 4 j + flags in an int32
+    s->closed = closed_lists_fit(M, E);
+    if (!s->closed) return CTR_OK;
     cudaStream_t st = s->stream;
     DevBuf scratch, work;
     CTR_TRY(s->cl_begin.alloc(sizeof(int32_t) * (M + 1)));
@@ -501,9 +510,13 @@ int build_closure(ctr_ibim* s, const int32_t* ptr, const int32_t* excl) {
 // Setup: the FP32 schedule (tuned), and the float-float and FP64 ones if the handle's options use them
 // (inner precision or refinement residual); an unused one is planned on first use (ensure_schedule).
 int build_schedules(ctr_ibim* s, const int slots[3]) {
+    CTR_TRY(build_closure(s, s->corr_ptr.as<int32_t>(), s->excl.as<int32_t>()));
+    return plan_schedules(s, slots);
+}
+
+int plan_schedules(ctr_ibim* s, const int slots[3]) {
     std::vector<uint8_t> flags;
     int g0 = 0, nb0 = 0;
-    CTR_TRY(build_closure(s, s->corr_ptr.as<int32_t>(), s->excl.as<int32_t>()));
     CTR_TRY(near_flags(s, flags, g0, nb0));
     CTR_TRY(alloc_accumulators(s));
     CTR_TRY(s->counter.alloc(sizeof(int) * 4));

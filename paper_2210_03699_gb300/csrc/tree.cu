@@ -111,6 +111,8 @@ int launch_tree_t(ctr_ibim* s, int pol) {
     return CTR_OK;
 }
 
+}  // namespace
+
 // Block pairs of kThreads-node blocks of tree positions with a correction pair between them (symmetric, nb x nb
 // bytes; empty beyond kMaxBaseBlocks).
 std::vector<uint8_t> correction_blocks(int64_t M, const std::vector<int32_t>& eptr, const std::vector<int32_t>& excl) {
@@ -129,8 +131,9 @@ std::vector<uint8_t> correction_blocks(int64_t M, const std::vector<int32_t>& ep
 // full are evaluated once for both, as in the direct schedules: a third (FP32) to half (float-float, FP64) of
 // the direct pairs at 178 575 nodes, the direct part of an application 7.9 -> 7.1 ms (FP32) and, with the
 // lighter float-float terms, 65.8 -> 47.0 ms.  The rest (one block's clusters at the edge of its near field
-// are not the other's) stays one-sided.  corr: correction_blocks().
-std::vector<PairItem> near_runs(const tree::Lists& L, int64_t M, int BS, const std::vector<uint8_t>& corr) {
+// are not the other's) stays one-sided, and so do near block pairs without closed exclusion lists (closed_lists_fit).
+// corr: correction_blocks().
+std::vector<PairItem> near_runs(const tree::Lists& L, int64_t M, int BS, const std::vector<uint8_t>& corr, bool closed) {
     const int nb = (int)((M + BS - 1) / BS);
     const bool pairs = !corr.empty();
     std::vector<uint8_t> full(pairs ? (size_t)nb * nb : 0, 0);   // J in full in I's direct ranges
@@ -152,12 +155,12 @@ std::vector<PairItem> near_runs(const tree::Lists& L, int64_t M, int BS, const s
         return false;
     };
     auto mutual = [&](int I, int J) {
-        return pairs && I != J && full[(size_t)I * nb + J] && full[(size_t)J * nb + I];
+        return pairs && I != J && full[(size_t)I * nb + J] && full[(size_t)J * nb + I] && (closed || !near(I, J));
     };
     std::vector<PairItem> runs;
     for (int I = 0; I < nb; ++I) {
         for (int J : fulls[(size_t)I]) {
-            if (J <= I || !full[(size_t)J * nb + I]) continue;
+            if (J <= I || !mutual(I, J)) continue;
             const int32_t kind = near(I, J) ? kItemNear : kItemSym;
             PairItem* run = runs.empty() ? nullptr : &runs.back();
             if (run && run->I == I && run->sym == kind && run->j_end == J * BS) run->j_end = last(J);
@@ -180,8 +183,6 @@ std::vector<PairItem> near_runs(const tree::Lists& L, int64_t M, int BS, const s
     }
     return runs;
 }
-
-}  // namespace
 
 int launch_tree(ctr_ibim* s, int pol) {
     if (!s->tree) return CTR_OK;
@@ -346,7 +347,7 @@ int build_tree_schedules(ctr_ibim* s, const int slots[3]) {
                 P.near_pairs += nt * (L.near_rng[2 * (size_t)r + 1] - L.near_rng[2 * (size_t)r]);
             far_total += (double)BS * P.np * kFarCost[p] * (double)(L.far_ptr[(size_t)I + 1] - L.far_ptr[(size_t)I]);
         }
-        cut_runs(sc, p, M, near_runs(L, M, BS, corr), slots[p]);
+        cut_runs(sc, p, M, near_runs(L, M, BS, corr, s->closed), slots[p]);
         CTR_TRY(upload_schedule(sc, st));
         const double far_cmax = std::max(1.0, far_total / ((double)kTreeItemsPerSlot * std::max(1, slots[p])));
         std::vector<int32_t> flist;

@@ -46,7 +46,7 @@ RESTART, INNER_TOL, SOLVE_TOL = 64, 1e-5, 1e-10
 # instruction counts as two lane operations, the FMA pipe's throughput being the same either way).
 # SFU work (rsqrt, ex2) and shared-memory loads are not counted.
 OPS_FP32 = {"one": 40, "sym": 47}
-OPS_DF64 = {"one": 360, "sym": 420}
+OPS_DF64 = {"one": 363, "sym": 423}
 # FP64 pipe lane operations per pair evaluation of the FP64 schedule, counted from the kernel source (seeds,
 # indices and high-order terms run on the SFU and the FP32 pipe), with the transposed sums of a symmetric
 # evaluation; its peak is the measured DFMA probe rate, there being no FP64 unit count to go by.
@@ -60,12 +60,12 @@ KERNEL_SOURCES = ("paper_2210_03699_gb300/csrc/pairkern.cuh", "paper_2210_03699_
                   "paper_2210_03699_gb300/csrc/common.cuh")
 # Treecode far field of the FP32 operator (FP32 charges): FMA-pipe lane operations per proxy evaluation
 # counted from the kernel source (tree.cuh, k_tree_far2: 1 sub, 6 fma, 7 mul; an f32x2 instruction does
-# two), plus 2 SFU operations (rsqrt, ex2).  The float-float operator's far field (k_tree_far_ff): 150
+# two), plus 2 SFU operations (rsqrt, ex2).  The float-float operator's far field (k_tree_far_ff): 153
 # FP32 add/sub/mul/fma instructions per evaluation (difference 11, r^2 12, d.n 12, rsqrt 15, kappa r 8, the
-# table exponential 21, the two charge combinations and accumulations 24 and 28, 1 + kappa r times E 11,
+# table exponential 24, the two charge combinations and accumulations 24 and 28, 1 + kappa r times E 11,
 # r^-3 8; table indexing and loads not counted), 1 SFU operation.
 OPS_FAR = 14
-OPS_FAR_DF = 150
+OPS_FAR_DF = 153
 SFU_FAR = 2
 
 

@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(NT, 2) k_tree_far2(Acc acc, const int2* __rest
 }
 
 // Float-float far items (the float-float operator): R targets per thread x NT threads = a 256-node block.
-// About 150 FP32 operations per evaluation; 128 registers (four blocks per SM) measured 54 -> 50 ms against the
+// About 153 FP32 operations per evaluation; 128 registers (four blocks per SM) measured 54 -> 50 ms against the
 // compiler's own 96 (9.5e9 evaluations), fewer registers 57 ms: the two targets' chains overlap.
 // Dynamic shared memory: the cluster's proxy coordinates and charges as float-float pairs, then the
 // exponential tables.

@@ -15,8 +15,10 @@ ONE, SYM, NEAR = 0, 1, 2
 
 @pytest.fixture(scope="module")
 def planner():
-    import planner as p
-    return p.load()
+    import native_lib
+    L = native_lib.load("planner.cpp")
+    L.plan_direct.restype = L.plan_tree.restype = ctypes.c_int64
+    return L
 
 
 def _p(a):

@@ -140,24 +140,30 @@ struct PlaneCtx {
     double tau;  // K-reg radius
 };
 
-// The K-reg cylinder of target i, by a whole warp: fn(m) for every cell of the search cube in ascending
-// node order, lane by lane of 32 consecutive cells (m: the tube node in the cylinder there, or -1); every lane
-// of the warp makes the same number of calls.  One thread per row would search the 11^3 cells alone (1.1 ms for
-// the K-reg rows of a 60-atom molecule; setup 3.9 -> 3.0 ms).
+// The K-reg cylinder of target i, by a whole warp: fn(m) for every cell of the search cube (clipped to the grid:
+// fewer than 2^31 cells however wide the tube) in ascending node order, lane by lane of 32 consecutive cells (m:
+// the tube node in the cylinder there, or -1); every lane of the warp makes the same number of calls.  One thread
+// per row would search the 11^3 cells alone (1.1 ms for the K-reg rows of a 60-atom molecule; setup 3.9 -> 3.0 ms).
 template <typename F>
 __device__ void visit_cylinder(const PlaneCtx& c, const NodeArrays& na, const int64_t* lin,
                                const int32_t* node_of, int64_t i, int lane, F&& fn) {
     const double P[3] = {na.Px[i], na.Py[i], na.Pz[i]};
     const double n[3] = {na.nx[i], na.ny[i], na.nz[i]};
-    const int64_t g = lin[i];
-    const int ci = (int)(g % c.nx), cj = (int)((g / c.nx) % c.ny), ck = (int)(g / (c.nx * c.ny));
+    const int64_t g = lin[i], at3[3] = {g % c.nx, (g / c.nx) % c.ny, g / (c.nx * c.ny)};
+    const int64_t dims[3] = {c.nx, c.ny, c.nz};
+    uint32_t lo[3], side[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        lo[a] = (uint32_t)max((int64_t)0, at3[a] - c.Kc);
+        side[a] = (uint32_t)(min(dims[a] - 1, at3[a] + c.Kc) + 1) - lo[a];
+    }
     const double tau2 = __dmul_rn(c.tau, c.tau);
-    const int side = 2 * c.Kc + 1, cells = side * side * side;
-    for (int at = lane; at - lane < cells; at += 32) {
+    const uint32_t cells = side[0] * side[1] * side[2];
+    for (uint32_t at = lane; at - lane < cells; at += 32) {
         int32_t m = -1;
-        const int q = ci - c.Kc + at % side, j = cj - c.Kc + (at / side) % side, k = ck - c.Kc + at / (side * side);
-        if (at < cells && q >= 0 && j >= 0 && k >= 0 && q < c.nx && j < c.ny && k < c.nz)
-            m = node_of[q + c.nx * (j + c.ny * (int64_t)k)];
+        const uint32_t row = at / side[0];
+        const uint32_t q = lo[0] + (at - row * side[0]), j = lo[1] + row % side[1], k = lo[2] + row / side[1];
+        if (at < cells) m = node_of[q + c.nx * (j + c.ny * (int64_t)k)];
         if (m >= 0) {
             const double y0 = __dadd_rn(c.origin[0], __dmul_rn(c.h, (double)q));
             const double y1 = __dadd_rn(c.origin[1], __dmul_rn(c.h, (double)j));

@@ -284,6 +284,8 @@ std::vector<uint8_t> correction_blocks(int64_t M, const std::vector<int32_t>& ep
 std::vector<PairItem> near_runs(const tree::Lists& L, int64_t M, int BS, const std::vector<uint8_t>& corr, bool closed);
 int64_t tree_bytes(const ctr_ibim* s);
 // schedule.cu: symmetric / one-sided pair schedules of a handle
+constexpr int kPartShift = 24;                            // engine work entries: item | part << kPartShift
+constexpr int64_t kMaxItems = (1 << kPartShift) - 1;      // items of a schedule the engine can run
 constexpr int kMaxBaseBlocks = 8192;   // side of a block-pair matrix (bytes: its square)
 // items of p (BS and tile set) from runs: target block, source range, kind; then their device copy
 void cut_runs(PairSchedule& p, int pol, int64_t M, const std::vector<PairItem>& runs, int slots);

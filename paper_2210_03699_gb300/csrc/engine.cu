@@ -43,9 +43,8 @@ namespace {
 
 constexpr int kVecThreads = 256;
 constexpr double kUpdateGate = 1e-4;   // |r| / |g| below which refinement residuals are updated
-// Work entries carry (slot, item | part << kPartShift): items of a schedule < 2^24, parts <= kMaxParts.
-constexpr int kPartShift = 24;
-constexpr int kItemMask = (1 << kPartShift) - 1;
+// Work entries carry (slot, item | part << kPartShift): items of a schedule <= kMaxItems, parts <= kMaxParts.
+constexpr int kItemMask = (int)kMaxItems;
 constexpr int kMaxParts = 127;
 constexpr int kMinItemsPerPart = 64;
 

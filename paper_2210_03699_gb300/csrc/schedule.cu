@@ -364,25 +364,48 @@ void cut_runs(PairSchedule& p, int pol, int64_t M, const std::vector<PairItem>& 
             }
         }
     }
+    // Pieces of a run: plen sources up to coarse_end, then fine ones.
+    struct Cut {
+        double unit;
+        int64_t plen, fine, coarse_end;
+    };
+    auto cut = [&](const PairItem& r, bool fine_end) {
+        const int64_t len = r.j_end - r.j_begin;
+        Cut c{(double)BS * costs[r.sym], piece, piece, r.j_end};
+        if (piece == 0) {
+            const int64_t pieces = std::max<int64_t>(1, (int64_t)std::ceil(c.unit * (double)len / cmax));
+            c.plen = (len + pieces - 1) / pieces;
+            c.plen = ((c.plen + tile - 1) / tile) * tile;
+            c.plen = std::max<int64_t>(c.plen, std::min<int64_t>(len, 2 * (int64_t)tile));
+            c.fine = std::max<int64_t>(kFineMin, c.plen / kFineDiv / kPieceStep * kPieceStep);
+            if (fine_end && len >= 2 * c.plen)   // runs of less than two pieces are cut evenly
+                c.coarse_end = r.j_begin + (int64_t)((double)len * kCoarse) / c.plen * c.plen;
+        }
+        return c;
+    };
+    auto count = [&](bool fine_end) {
+        int64_t n = 0;
+        for (const PairItem& r : runs) {
+            const Cut c = cut(r, fine_end);
+            n += (c.coarse_end - r.j_begin + c.plen - 1) / c.plen + (r.j_end - c.coarse_end + c.fine - 1) / c.fine;
+        }
+        return n;
+    };
+    // the fine pieces nearly double the number of items: where a schedule would pass what the engine's work entries
+    // can name (FP64 from 1.5 million nodes on, float-float from 3.1), it has none
+    int64_t n_items = count(true);
+    const bool fine_end = n_items <= kMaxItems;
+    if (!fine_end) n_items = count(false);
     p.total_cost = total;
     p.items.clear();
     p.cost.clear();
+    p.items.reserve((size_t)n_items);
+    p.cost.reserve((size_t)n_items);
     p.pairs_sym = p.pairs_one = 0;
     for (const PairItem& r : runs) {
-        const int64_t len = r.j_end - r.j_begin;
-        const double unit = (double)BS * costs[r.sym];
-        int64_t plen = piece;
-        if (piece == 0) {
-            const int64_t pieces = std::max<int64_t>(1, (int64_t)std::ceil(unit * (double)len / cmax));
-            plen = (len + pieces - 1) / pieces;
-            plen = ((plen + tile - 1) / tile) * tile;
-            plen = std::max<int64_t>(plen, std::min<int64_t>(len, 2 * (int64_t)tile));
-        }
-        const int64_t fine = piece != 0 ? plen : std::max<int64_t>(kFineMin, plen / kFineDiv / kPieceStep * kPieceStep);
-        const int64_t coarse_end =   // runs of less than two pieces are cut evenly
-            piece != 0 || len < 2 * plen ? r.j_end : r.j_begin + (int64_t)((double)len * kCoarse) / plen * plen;
+        const Cut c = cut(r, fine_end);
         for (int64_t a = r.j_begin, step; a < r.j_end; a += step) {
-            step = a < coarse_end ? plen : fine;
+            step = a < c.coarse_end ? c.plen : c.fine;
             PairItem it{};
             it.I = r.I;
             it.j_begin = (int32_t)a;
@@ -392,7 +415,7 @@ void cut_runs(PairSchedule& p, int pol, int64_t M, const std::vector<PairItem>& 
             if (r.sym) p.pairs_sym += tgt * (it.j_end - it.j_begin);
             else p.pairs_one += tgt * (it.j_end - it.j_begin);
             p.items.push_back(it);
-            p.cost.push_back(unit * (double)(it.j_end - it.j_begin));
+            p.cost.push_back(c.unit * (double)(it.j_end - it.j_begin));
         }
     }
 }

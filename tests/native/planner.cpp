@@ -25,6 +25,18 @@ int64_t plan_direct(int64_t M, int BS, const uint8_t* flags, int g0, int nb0, in
     return put(direct_runs(M, BS, std::vector<uint8_t>(flags, flags + (size_t)nb0 * nb0), g0, nb0, closed != 0), cap, out);
 }
 
+// A direct schedule of M nodes without correction pairs cut into items: their number; pairs: one-sided and symmetric
+int64_t cut_direct(int pol, int64_t M, int BS, int tile, int slots, int64_t* pairs, int64_t cap, int32_t* out) {
+    const int nb = (int)((M + BS - 1) / BS);
+    PairSchedule p;
+    p.BS = BS;
+    p.tile = tile;
+    cut_runs(p, pol, M, direct_runs(M, BS, std::vector<uint8_t>((size_t)nb * nb, 0), BS, nb, true), slots);
+    pairs[0] = p.pairs_one;
+    pairs[1] = p.pairs_sym;
+    return put(p.items, cap, out);
+}
+
 // ptr, excl: correction rows in tree positions; near ranges of every block as ctr_farfield_plan gives them
 int64_t plan_tree(int64_t M, int BS, const int32_t* ptr, const int32_t* excl, int64_t nb, const int64_t* near_ptr,
                   const int32_t* near_rng, int closed, int64_t cap, int32_t* out) {

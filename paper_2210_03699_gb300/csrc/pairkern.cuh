@@ -277,6 +277,10 @@ __device__ __forceinline__ double rsqrt_d(double x) {
     const double e = fma(-x, y * y, 1.0);
     return fma(y * e, fma(0.375, e, 0.5), y);
 }
+// 2^-990 <= x < 2^990: where rsqrt_d holds (its seed and the seed's square are normal)
+__device__ __forceinline__ bool rsqrt_d_range(double x) {
+    return (uint32_t)__double2hiint(x) - 0x02100000u < 0x7bc00000u;
+}
 // e^{-kappa r} = 2^-i T_j 2^-f with kappa r log2(e) = i + j/1024 + f: the index from FP32, f by one fused
 // operation, 2^-f - 1 = f (-ln2 + f (ln2^2/2 - f g)) with g in FP32 (f^3 g < 2^-37), corrected by the relative
 // rounding errors of T_j and of kappa log2(e) (q's constant term): within one rounding of the exact value

@@ -227,7 +227,7 @@ __global__ void rhs_kernel(NodeArrays na, int64_t M, const double* __restrict__ 
         const double dx = px - ch[c], dy = py - ch[nc + c], dz = pz - ch[2 * nc + c];
         const double q = ch[3 * nc + c] * inv_eps;
         const double r2 = dx * dx + dy * dy + dz * dz;
-        const double rinv = pk::rsqrt_d(r2);   // five FP64 operations (1 / sqrt takes about twenty)
+        const double rinv = pk::rsqrt_d_range(r2) ? pk::rsqrt_d(r2) : 1.0 / sqrt(r2);   // charges may lie anywhere
         const double t = q * inv4pi * rinv;
         g1 += t;
         g2 -= t * (dx * qx + dy * qy + dz * qz) * (rinv * rinv);

@@ -449,8 +449,9 @@ int ctr_ibim_reaction_potential(ctr_ibim* sys, const double* psi, const double* 
  *                CTR_FP64: IEEE FP64.
  *   on_device    0: every array is host memory; 1: every array is device
  *                memory of the handle's device.
- * The split partial sums (and, for host arrays, device copies of the
- * arguments) live in buffers the handle keeps: a call allocates only when it
+ * The partial sums (in CTR_DF64 and CTR_FP64 up to 32 MB; from 8.4 million nodes
+ * on up to 4 bytes per node) and, for host arrays, device copies of the
+ * arguments live in buffers the handle keeps: a call allocates only when it
  * needs more than an earlier call did.  The handle's packed source weights
  * are overwritten (as by ctr_ibim_matvec).  Errors: CTR_ERR_INVALID,
  * CTR_ERR_CAPACITY (n_points >= 2^31), CTR_ERR_NOMEM, CTR_ERR_CUDA,

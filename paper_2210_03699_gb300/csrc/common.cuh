@@ -315,6 +315,8 @@ int apply_operator_timed(ctr_ibim* s, const double* d_x, double* d_y, int precis
 // CTR_DF64 or CTR_FP64), all pointers device memory; enqueued on the handle's stream
 int potential_map(ctr_ibim* s, const double* d_psi, const double* d_dpsi, int64_t n, const double* d_xyz,
                   double* d_out, int precision);
+// the workspace of an energy of n charges (allocated at the first one; map_ws)
+int64_t energy_workspace_bytes(int64_t M, int64_t n);
 // reductions (krylov.cu)
 int device_dot(ctr_ibim* s, const double* a, const double* b, int64_t n, double* h_out);
 int check_device_error(ctr_ibim* s, const char* where);

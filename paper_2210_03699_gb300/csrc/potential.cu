@@ -316,7 +316,7 @@ constexpr size_t map_smem() {
     return 2 * Pol::kTile * Pol::kVec * sizeof(typename Pol::Src) + Pol::kTab * sizeof(float2);
 }
 
-// Unit sums of one launch: 32 MB of workspace, and at a million threads or more its last wave is a small part.
+// Unit sums of one launch: 32 MB of workspace (more only for 8.4 million nodes and up), and at a million threads or more its last wave is a small part.
 // More points go in chunks.
 constexpr int64_t kUnitSums = 4 << 20;
 // FP32 maps of at most this many unit sums take map_unit_kernel: its sources come through L1, not by bulk
@@ -325,11 +325,16 @@ constexpr int64_t kUnitSums = 4 << 20;
 // 1000, 178,575 (698,000) 244 : 218; 4000, 44,597 (700,000) 238 : 207.
 constexpr int64_t kUnitSums32 = 1 << 19;
 
+// points of one launch
+int64_t unit_chunk(int64_t units, int64_t n) {
+    return std::min(n, std::max<int64_t>(32, kUnitSums / units / 32 * 32));
+}
+
 template <typename Pol>
 int map_units(ctr_ibim* s, const void* src, const double* d_xyz, int64_t n, const PairConsts& kc, int per_group,
               double* d_out) {
     const int64_t M = s->M, units = (M + Pol::kUnit - 1) / Pol::kUnit;
-    const int64_t chunk = std::min(n, std::max<int64_t>(32, kUnitSums / units / 32 * 32));
+    const int64_t chunk = unit_chunk(units, n);
     CTR_TRY(s->map_ws.alloc(sizeof(double) * (size_t)(units * chunk)));
     for (int64_t p = 0; p < n; p += chunk) {
         const int64_t m = std::min(chunk, n - p), slots = (m + Pol::kPack - 1) / Pol::kPack;
@@ -381,6 +386,12 @@ int map_fp32(ctr_ibim* s, const double* d_xyz, int64_t n, const PairConsts& kc, 
 }
 
 }  // namespace
+
+int64_t energy_workspace_bytes(int64_t M, int64_t n) {
+    if (M <= 0 || n <= 0) return 0;
+    const int64_t units = (M + MapFp64::kUnit - 1) / MapFp64::kUnit;
+    return (int64_t)sizeof(double) * units * unit_chunk(units, n);
+}
 
 int potential_map(ctr_ibim* s, const double* d_psi, const double* d_dpsi, int64_t n, const double* d_xyz,
                   double* d_out, int precision) {

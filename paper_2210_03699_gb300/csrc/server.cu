@@ -18,7 +18,8 @@
 // footprint estimate counts the tube nodes on the host (|d| < eps) and charges
 // the per-node cost of geometry, packed sources, solver vectors and the
 // Krylov basis plus the dense sum's exact node accumulators (200 bytes);
-// after setup the handle's real allocation is charged instead.
+// after setup the handle's real allocation is charged instead, with the
+// workspace of its energy, which comes when it is solved.
 #include <chrono>
 #include <condition_variable>
 #include <cstring>
@@ -115,7 +116,7 @@ int64_t estimate_bytes(const Request& r) {
     const int64_t extra = (r.opt.farfield == CTR_FARFIELD_TREECODE) ? M * 512 + ((int64_t)64 << 20)
                                                                     : ((int64_t)16 << 20);
     const int64_t grid_bytes = (int64_t)r.sdist.size() * (8 + 4);   // staging copy + node map during setup
-    return M * per_node + extra + grid_bytes;
+    return M * per_node + extra + grid_bytes + energy_workspace_bytes(M, (int64_t)r.q.size());
 }
 
 void release_stream(Request* r) {
@@ -203,7 +204,9 @@ void setup_loop(ctr_server* sv) {
             sys = nullptr;
             release_stream(r);
         }
-        const int64_t real = sys ? (int64_t)handle_bytes(sys) : 0;
+        // the handle's allocation and what its energy will take when it is solved
+        const int64_t real =
+            sys ? (int64_t)handle_bytes(sys) + energy_workspace_bytes(sys->M, (int64_t)r->q.size()) : 0;
         std::unique_lock<std::mutex> lk(sv->mu);
         sv->preparing--;
         r->sdist.clear();

@@ -137,13 +137,14 @@ struct PairSchedule {
 
 // Throughput of each pair arithmetic ([0] FP32, [1] float-float, [2] FP64) on the whole GPU in the cost
 // units of a schedule (one-sided pair evaluations; a symmetric evaluation counts its relative cost),
-// as measured on a GB300 at M = 178,575 (1.23e12, 1.25e11 and 1.55e10 pair interactions/s).  Used only
-// to size work (item lengths, engine parts), never in the arithmetic.
-constexpr double kUnitRate[3] = {7.9e11, 7.5e10, 9.0e9};
-// Longest item per arithmetic: this many seconds of one resident block at the rates above.  Short
-// items keep the tail of a persistent launch short and let the engine split a large system's
-// application into parts (an FP32 application of 180k nodes takes 26 ms, a float-float one 256 ms).
-constexpr double kItemSeconds[3] = {8e-3, 4e-3, 4e-3};
+// as measured on a GB300 at M = 178,575 (1.28e12, 1.47e11 and 1.94e10 pair interactions/s: 25.0, 217 and
+// 1643 ms per application).  Used only to size work (engine parts), never in the arithmetic.
+constexpr double kUnitRate[3] = {8.0e11, 8.85e10, 1.12e10};
+// Longest item per arithmetic: this much work (in cost units) divided by the number of resident blocks, which one
+// block does in kItemCost / kUnitRate seconds (7.9, 3.4 and 3.2 ms).  Short items keep the tail of a persistent
+// launch short and let the engine split a large system's application into parts.
+constexpr double kItemCost[3] = {6.32e9, 3.0e8, 3.6e7};
+constexpr double item_seconds(int pol) { return kItemCost[pol] / kUnitRate[pol]; }
 
 // ---------------------------------------------------------------- far field (treecode)
 constexpr int kTreeMaxN1 = 13;                                        // degree <= 12

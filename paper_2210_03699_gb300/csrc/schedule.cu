@@ -17,7 +17,7 @@
 // blocks at 178 575 nodes), most of a small one's.
 //
 // Items are split to at most a quarter-wave of work each, and to at most
-// kItemSeconds of one resident block's time (small systems: to pieces of one
+// kItemCost (a few ms of one resident block; small systems: to pieces of one
 // length that fill whole waves), and sorted by cost for the
 // atomic-counter scheduler.  Every item adds its sums into the nodes'
 // exact accumulators (pairkern.cuh, fx_add: integer addition, so the order in
@@ -336,14 +336,12 @@ std::vector<PairItem> direct_runs(int64_t M, int BS, const std::vector<uint8_t>&
 // one kind.
 void cut_runs(PairSchedule& p, int pol, int64_t M, const std::vector<PairItem>& runs, int slots) {
     const double costs[3] = {1.0, kSymCost[pol], kNearCost[pol]};   // by item kind
-    const double item_cost = kUnitRate[pol] * kItemSeconds[pol];
     const int BS = p.BS, tile = p.tile;
     double total = 0.0;
     for (const PairItem& r : runs) total += (double)BS * (r.j_end - r.j_begin) * costs[r.sym];
-    // split runs into items of at most a quarter-wave of work and kItemSeconds of one block (item_cost:
-    // the arithmetic's rate x kItemSeconds; whole tiles, at least two when possible)
+    // split runs into items of at most a quarter-wave of work and kItemCost (whole tiles, at least two when possible)
     const double nslots = (double)std::max(1, slots);
-    const double cmax = std::max(1.0, std::min(total / ((double)kItemsPerSlot * nslots), item_cost / nslots));
+    const double cmax = std::max(1.0, std::min(total / ((double)kItemsPerSlot * nslots), kItemCost[pol] / nslots));
     // A system with less than eight tiles of work per resident block cannot be cut that way (few items, the
     // last wave nearly empty): its pieces have one common length, the one with the shortest estimated makespan
     // (waves of equal pieces, each with the cost of starting it).  The FP64 kernel is bound by one pipe per

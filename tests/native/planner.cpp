@@ -58,4 +58,7 @@ int replan_one_sided(ctr_ibim* s) {
     const int st = schedule_slots(sms, slots);
     return st < 0 ? st : plan_schedules(s, slots);
 }
+
+// What the engine takes one application of arithmetic pol (0 FP32, 1 float-float, 2 FP64) to last
+double estimated_seconds(const ctr_ibim* s, int pol) { return s->sched[pol].total_cost / kUnitRate[pol]; }
 }

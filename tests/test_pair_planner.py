@@ -18,6 +18,7 @@ def planner():
     import native_lib
     L = native_lib.load("planner.cpp")
     L.plan_direct.restype = L.plan_tree.restype = L.cut_direct.restype = ctypes.c_int64
+    L.estimated_seconds.restype = ctypes.c_double
     return L
 
 
@@ -144,3 +145,20 @@ def test_near_block_pairs_one_sided(planner, oracle_tables, name):
         assert G.pair_schedule(ctr.FP64)["symmetric_pairs"] < before
         for precision, tol in ((ctr.DF64, 1e-12), (ctr.FP64, 1e-12), (ctr.FP32_REFINE, 2e-5)):
             assert np.max(np.abs(G.matvec(x, precision) - ref)) / scale < tol
+
+
+@pytest.mark.gpu
+def test_estimated_application_times(planner):
+    """The engine's estimates, by which it splits applications, against the times: their ratios to the FP32 one
+    (clocks cancel) within 8%."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    with ctr.CtrIbim.from_problem(syn.ellipsoid_problem(h=0.05)) as G:
+        t, e = [], []
+        for pol, prec in enumerate((ctr.FP32_REFINE, ctr.DF64, ctr.FP64)):
+            G.time_operator(prec, reps=1)
+            t.append(min(G.time_operator(prec, reps=2)["pairs_ms"] for _ in range(2)))
+            e.append(planner.estimated_seconds(G._h, pol))
+    for pol in (1, 2):
+        assert abs((e[pol] / e[0]) / (t[pol] / t[0]) - 1) < 0.08, (t, e)

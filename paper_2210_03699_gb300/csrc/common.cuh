@@ -219,7 +219,7 @@ struct Krylov {
     DevBuf cs, sn, s;    // Givens and rhs of the least-squares problem
     DevBuf y;            // m
     DevBuf part;         // partial dot products: (m+1) x nblk
-    DevBuf scal;         // scalars: [0] beta, [1] hnorm, [2] residual estimate, [3] converged flag ...
+    DevBuf scal;         // scalars: [2] length of the next basis vector, [4] dot products read by the host
     int nblk = 0;
 };
 

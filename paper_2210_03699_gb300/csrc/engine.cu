@@ -1014,10 +1014,6 @@ int engine_admit(Engine* e, ctr_ibim* s, int* slot_out) {
         e->max_nblk = d.nblk;
         e->graph_dirty = true;
     }
-    if (d.m > e->max_m) {
-        e->max_m = d.m;
-        e->graph_dirty = true;
-    }
     const int vb = (int)std::min<int64_t>(grid_for(s->M, kVecThreads), 1024);
     if (vb > e->vec_blocks) {
         e->vec_blocks = vb;

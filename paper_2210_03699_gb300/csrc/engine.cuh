@@ -75,7 +75,6 @@ struct Engine {
     bool lists_dirty = false;   // slots admitted or retired since the work lists were built (engine_step rebuilds)
     int vec_blocks = 1;
     int max_nblk = 1;
-    int max_m = 1;
     int sms = 1;
     // work lists per pair arithmetic and kernel variant (FP32: the variant of each slot's schedule)
     int64_t item_cap[3][pk::kNumVar32] = {};
@@ -96,7 +95,7 @@ struct Engine {
     std::vector<ctr_ibim*> owner;
     DevBuf slots, stats, items[3][pk::kNumVar32], n_items, counters;
     int* err = nullptr;   // error word of the pair kernels (behind the stats)
-    DevBuf need;   // per pair arithmetic: does any slot need its pair launch in the current half (k_need)
+    DevBuf need;   // per pair arithmetic: does any slot need its pair launch in the current half (begin_half)
     // treecode work entries (slot, index) per pair arithmetic: moment chunks, far clusters, far items
     bool any_tree = false;
     int tree_np[3] = {0, 0, 0};   // largest proxy count per arithmetic among the treecode slots

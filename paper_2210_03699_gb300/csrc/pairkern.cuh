@@ -28,7 +28,7 @@ struct PairConsts {
     double c1kap;                    // (eps_E/eps_I) kappa
     const float2* exp_tab;           // exponential tables of the arithmetic (float-float or FP64), global
     // the FP32 values duplicated into both halves of a 64-bit word (f32x2 operands)
-    unsigned long long one2, mone2, three2, mthree2, c1x2, nc1x2, c2x2, nc2x2, kap2, kl2x2;
+    unsigned long long one2, mone2, three2, mthree2, c1x2, nc1x2, c2x2, kap2, kl2x2;
     unsigned long long c1kap2;       // (eps_E/eps_I) kappa
     uint32_t wait_limit;             // polls of a source-tile wait before the block gives up
     uint32_t pad_;
@@ -158,10 +158,6 @@ __device__ __forceinline__ F2 add(F2 a, F2 b) {
     return fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
 }
 __device__ __forceinline__ F2 sub(F2 a, F2 b) { return add(a, neg(b)); }
-__device__ __forceinline__ F2 add_f(F2 a, float b) {
-    const F2 s = two_sum(a.hi, b);
-    return fast_two_sum(s.hi, __fadd_rn(s.lo, a.lo));
-}
 __device__ __forceinline__ F2 mul(F2 a, F2 b) {
     const F2 p = two_prod(a.hi, b.hi);
     return fast_two_sum(p.hi, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, p.lo)));

@@ -233,7 +233,6 @@ void set_packed_consts(PairConsts& kc) {
     kc.c1x2 = dup(kc.c1f);
     kc.nc1x2 = dup(-kc.c1f);
     kc.c2x2 = dup(kc.c2f);
-    kc.nc2x2 = dup(-kc.c2f);
     kc.kap2 = dup(kc.kappaf);
     kc.kl2x2 = dup(kc.kl2f);
     kc.c1kap2 = dup((float)(kc.c1 * kc.kappa));

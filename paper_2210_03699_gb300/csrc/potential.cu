@@ -148,7 +148,7 @@ struct MapFp64 {
 };
 
 // One block: points [blockIdx.x * BS, +BS) against sources [j_begin, j_end) of its split; the sums go to
-// part[split * n + point].
+// part[split * n + point].  Pol: an arithmetic without exponential tables (FP32).
 template <typename Pol>
 __global__ void __launch_bounds__(kThreads) map_kernel(const typename Pol::Src* __restrict__ src, int M,
                                                        const double* __restrict__ xyz, int64_t n, int per_split,
@@ -159,9 +159,7 @@ __global__ void __launch_bounds__(kThreads) map_kernel(const typename Pol::Src* 
     constexpr int BS = kThreads * RP;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     Src* ring = reinterpret_cast<Src*>(smem_raw);
-    float2* tab = reinterpret_cast<float2*>(smem_raw + 2 * TILE * VEC * sizeof(Src));
     __shared__ __align__(8) uint64_t bar[2];
-    for (int q = threadIdx.x; q < Pol::kTab; q += kThreads) tab[q] = kc.exp_tab[q];
     if (threadIdx.x == 0) {
         mbar_init(&bar[0], 1);
         mbar_init(&bar[1], 1);
@@ -209,7 +207,7 @@ __global__ void __launch_bounds__(kThreads) map_kernel(const typename Pol::Src* 
 #pragma unroll 2
         for (int q = 0; q < cnt; ++q) {
 #pragma unroll
-            for (int r = 0; r < R; ++r) Pol::pair(tg[r], tile + q * VEC, kc, tab, acc[r]);
+            for (int r = 0; r < R; ++r) Pol::pair(tg[r], tile + q * VEC, kc, nullptr, acc[r]);
         }
 #pragma unroll
         for (int r = 0; r < R; ++r) Pol::fold(acc[r], &s[r * P]);
@@ -236,7 +234,7 @@ __global__ void map_sum_kernel(const double* __restrict__ part, int splits, int6
 //     us, grid -> units (FP64): 3 points, 11,203 nodes 1313 -> 136; 3, 178,575: 2582 -> 140; 500, 44,597:
 //     1319 -> 1185; 4000, 178,575: 38,941 -> 35,998.  float-float: 252 -> 115, 424 -> 132, 259 -> 221,
 //     5239 -> 4860.
-//   FP32: few points or small systems only (map_launch); the units and groups are then map_kernel's tiles and
+//   FP32: few points or small systems only (map_fp32); the units and groups are then map_kernel's tiles and
 //     splits, and a point's result has the same bits from either.
 constexpr int kUnitThreads = 128;
 template <typename Pol>
@@ -313,7 +311,8 @@ __global__ void map_pack_kernel(const double* __restrict__ psi, const double* __
 
 template <typename Pol>
 constexpr size_t map_smem() {
-    return 2 * Pol::kTile * Pol::kVec * sizeof(typename Pol::Src) + Pol::kTab * sizeof(float2);
+    static_assert(Pol::kTab == 0, "the tiled map kernel carries no exponential tables");
+    return 2 * Pol::kTile * Pol::kVec * sizeof(typename Pol::Src);
 }
 
 // Unit sums of one launch: 32 MB of workspace (more only for 8.4 million nodes and up), and at a million threads or more its last wave is a small part.

@@ -85,8 +85,8 @@ enum { CTR_METHOD_HYB = 0, CTR_METHOD_KREG = 1 };
  *       separated from it (theta |c_B - c_C| > r_B + r_C on the integer boxes
  *       widened by ceil(eps/h) grid units, decided exactly), that holds none of
  *       the block's correction nodes and that has more than (degree+1)^3 nodes
- *       (half of that for the float-float arithmetic, whose direct pairs cost
- *       about two of its float-float proxy evaluations each)
+ *       (half of that for the float-float arithmetic: a direct pair evaluated
+ *       for one row costs about two of its proxy evaluations)
  *       is replaced by (degree+1)^3 tensor Chebyshev points on the tight box of
  *       its points P carrying interpolated charges (barycentric Lagrange
  *       interpolation of the kernels' source variable, d/dn_y on the basis);

@@ -71,7 +71,7 @@ int ensure_krylov(ctr_ibim* s) {
     if (k.m == m && k.n == n) return CTR_OK;
     k.m = m;
     k.n = n;
-    // reduction chunks: about one per SM, of 512 elements or more (a small system's reductions are latency,
+    // reduction chunks: 148 at most (this chip has 152 SMs), of 512 elements or more (a small system's reductions are latency,
     // more blocks than SMs only add partials)
     const int64_t chunk = std::max<int64_t>(512, ((n + 147) / 148 + 255) / 256 * 256);
     k.nblk = (int)std::max<int64_t>(1, (n + chunk - 1) / chunk);

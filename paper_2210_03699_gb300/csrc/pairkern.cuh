@@ -266,7 +266,9 @@ __device__ __forceinline__ float narrow_pos(double v) {
     const int hi = min(max(__double2hiint(v), 0x38100000), 0x47e00000);
     return __uint_as_float(__funnelshift_l((uint32_t)__double2loint(v), (uint32_t)(hi - 0x38000000), 3));
 }
-// 1/sqrt(x): SFU seed of 20 bits (its square is exact in FP64), residual, third-order step; five operations
+// 1/sqrt(x): SFU seed y of 20 bits (its square is exact in FP64), residual e = 1 - x y^2, and the binomial series
+// of (1 - e)^(-1/2) to its second power: y (1 + e/2 + 3/8 e^2); five operations.  rms error 0.42 x 2^-53, largest
+// 1.0 x 2^-53.
 __device__ __forceinline__ double rsqrt_d(double x) {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -277,11 +279,12 @@ __device__ __forceinline__ double rsqrt_d(double x) {
 __device__ __forceinline__ bool rsqrt_d_range(double x) {
     return (uint32_t)__double2hiint(x) - 0x02100000u < 0x7bc00000u;
 }
-// e^{-kappa r} = 2^-i T_j 2^-f with kappa r log2(e) = i + j/1024 + f: the index from FP32, f by one fused
-// operation, 2^-f - 1 = f (-ln2 + f (ln2^2/2 - f g)) with g in FP32 (f^3 g < 2^-37), corrected by the relative
-// rounding errors of T_j and of kappa log2(e) (q's constant term): within one rounding of the exact value
-// times the rounding of the result, as CUDA's exp, in five FP64 operations instead of about sixteen (rms
-// error over r = 1e-3 to 1e3 0.36 x 2^-53, rsqrt_d 0.43 x 2^-53 as CUDA's).
+// e^{-kappa r} by table (Tang, "Table-driven implementation of the exponential function in IEEE floating-point
+// arithmetic", ACM TOMS 15(2), 1989): 2^-i T_j 2^-f with kappa r log2(e) = i + j/1024 + f, the index from FP32, f by
+// one fused operation, 2^-f - 1 = f (-ln2 + f (ln2^2/2 - f g)) by its Taylor series with g = ln2^3/6 - f ln2^4/24 in
+// FP32 (f^3 g < 2^-37), corrected by the relative rounding errors of T_j and of kappa log2(e) (q's constant term);
+// five FP64 operations.  Error in units of 2^-53: rms 0.42 and at most 1.03 up to kappa r = 30; the index comes from
+// 24 bits of r, so f grows with kappa r, and with it g's error: at most 1.9 up to 350, 3.8 up to 680 (rms 0.60).
 __device__ __forceinline__ double exp_neg_d(double r, const PairConsts& k, const float2* tab) {
     const double* T = reinterpret_cast<const double*>(tab);
     const float* tau = reinterpret_cast<const float*>(T + kExp2);
@@ -683,8 +686,8 @@ struct Fp32x2Policy {
     }
     // Both orientations: the factors s t1, s t2n, s X and (1 - E)/r are formed once (40 operations per one-sided
     // evaluation, 47 per symmetric one; of the 47, 19 are multiply-adds with three distinct register operands,
-    // which run at 80 lanes a clock and SM against 119 for the others: 78% of the pipe is what the mix allows, and
-    // what the kernel reaches).
+    // which run at 84 lanes a clock and SM against 127 for the others (probe/probe.cu; scalar ones at 85): the mix
+    // allows 82% of the pipe, the kernel keeps it busy for 78% of its active cycles).
     // kMask: flags per half (Exclusions); a pair left out of both rows is moved to distance 1 (no NaN).
     template <bool kFirst, bool kMask = false>
     __device__ static void pair_sym(const Tgt& T, const Src* S, const PairConsts& k, const float2*, Acc& acc,
@@ -754,8 +757,8 @@ struct Fp64Policy {
         return JAcc{__shfl_xor_sync(0xffffffffu, x.a1, m), __shfl_xor_sync(0xffffffffu, x.a2, m)};
     }
     // The factors the two orientations share: d . n_x, d . n_y, s t1, s t2, s X and (1 - E)/r (u, w, c as in
-    // Df64Policy): 55 FP64 operations per symmetric evaluation, 50 per one-sided one (69 per symmetric one with
-    // CUDA's rsqrt and exp).  Per application 9.7 -> 7.8 ms at 11 203 nodes, 133 -> 107 ms at 44 597, 90% of
+    // Df64Policy): 55 FP64 operations per symmetric evaluation, 50 per one-sided one (before rsqrt_d, exp_neg_d and
+    // the shared factors the profiler counted 69 per symmetric one).  Per application 9.7 -> 7.8 ms at 11 203 nodes, 133 -> 107 ms at 44 597, 90% of
     // the FP64 pipe's measured rate; every term's error as before.
     struct Common {
         double dnx, dny, st1, st2, sX, om;

@@ -15,18 +15,18 @@
 // block reads each source by broadcast.  The correction pairs N(i) (sorted
 // per target) are skipped exactly: a warp takes a masked path only for tiles
 // that contain one of its lanes' excluded nodes.  The work is a schedule of
-// one-sided and symmetric items (schedule.cu): block pairs without correction
-// pairs are evaluated once for both orientations, and each item adds its FP64
-// sums into the nodes' exact accumulators (integer addition: the result does
+// one-sided and symmetric items (schedule.cu): block pairs are evaluated once
+// for both orientations (those with correction pairs with masks), diagonal
+// blocks one-sided, and each item adds its FP64 sums into the nodes' exact accumulators (integer addition: the result does
 // not depend on the order in which blocks add), read and cleared by the
 // finishing kernel.
 //
 // Three pair arithmetics share this pipeline (policies below):
-//   Fp32  FP32 terms, rsqrt and exp2 on the SFU (44 FP32-pipe ops per pair);
-//   Fp64  IEEE FP64 (DFMA, 1/64 of the FP32 rate on this chip);
+//   Fp32  FP32 terms, rsqrt and exp2 on the SFU (47 FP32-pipe ops per symmetric pair);
+//   Fp64  IEEE FP64 (1/64 of the FP32 rate on this chip);
 //   Df64  double-FP32 "float-float" terms (error-free sums and products with
-//         FMA, rsqrt by one Newton step in df64, exp by two exact tables and
-//         a degree-4 polynomial), ~2^-44 relative, on the FP32 pipe.
+//         FMA, rsqrt by an SFU seed and a second-order step, exp by two tables
+//         and a degree-4 polynomial), ~2^-44 relative, on the FP32 pipe.
 #include <atomic>
 #include <cmath>
 #include <cstring>

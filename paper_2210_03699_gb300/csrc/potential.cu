@@ -132,7 +132,7 @@ struct MapFp64 {
     }
     __device__ static void zero(Acc& a) { a = 0.0; }
     __device__ static void fold(const Acc& a, double* s) { s[0] += a; }
-    // as MapFp32x2; 28 FP64 operations per pair (45 with CUDA's rsqrt and exp and the terms apart)
+    // as MapFp32x2; 28 FP64 operations per pair
     __device__ static void pair(const Tgt& T, const Src* S, const PairConsts& k, const float2* tab, Acc& acc) {
         const double4 pa = S[0], nb = S[1];
         const double dx = T.x - pa.x, dy = T.y - pa.y, dz = T.z - pa.z;

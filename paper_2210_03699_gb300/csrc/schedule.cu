@@ -345,7 +345,7 @@ void cut_runs(PairSchedule& p, int pol, int64_t M, const std::vector<PairItem>& 
     // A system with less than eight tiles of work per resident block cannot be cut that way (few items, the
     // last wave nearly empty): its pieces have one common length, the one with the shortest estimated makespan
     // (waves of equal pieces, each with the cost of starting it).  The FP64 kernel is bound by one pipe per
-    // SM whatever the blocks on it, so there the waves are counted in SMs.
+    // SM whatever the blocks on it (two, Fp64Policy::kMinBlocks), so there the waves are counted in SMs.
     int64_t piece = 0;
     const double servers = pol == 2 ? std::max(1.0, nslots / 2.0) : nslots;
     if (total < 8.0 * tile * BS * nslots) {

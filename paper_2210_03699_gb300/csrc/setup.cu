@@ -78,7 +78,7 @@ __global__ void tube_compact_kernel(const double* __restrict__ sd, int64_t total
 }
 
 // Single-block exclusive scan of n counts (any n), offsets[n] = total.  Four counts per thread and round, warp
-// scans by shuffles, two barriers a round: 275 -> 72 us for 178 575 counts (one count per thread and a scan
+// scans by shuffles, one barrier a round: 275 -> 72 us for 178 575 counts (one count per thread and a scan
 // over the block in shared memory before).
 __global__ void __launch_bounds__(1024) scan_kernel(const int32_t* __restrict__ in, int32_t* __restrict__ out, int64_t n) {
     __shared__ int32_t warp_sum[2][32];

@@ -2,8 +2,8 @@
 // handle.  Setup (once): the octree and interaction lists (tree_host.cpp),
 // the nodes' tree order (the packed source arrays are permuted to it, so that
 // every cluster and target block is a contiguous range), the exclusion lists
-// in tree positions, and per pair arithmetic the schedule: one-sided pair
-// items for the direct ("near") ranges, far items for the far clusters and the
+// in tree positions, and per pair arithmetic the schedule: pair items for the
+// direct ("near") ranges (symmetric where two blocks sum each other), far items for the far clusters and the
 // moment chunks of the clusters that carry charges; near and far items add
 // their sums into the nodes' exact accumulators (order-independent).  Per
 // operator application: the near items run in the
@@ -23,8 +23,10 @@ using namespace pk;
 namespace {
 
 constexpr int kTreeItemsPerSlot = 4;
-// A well-separated cluster is approximated when it has more than (degree+1)^3 / kMinFarDiv nodes: a
-// float-float pair costs about two float-float proxy evaluations, an FP32 or FP64 pair about one.
+// A well-separated cluster is approximated when it has more than (degree+1)^3 / kMinFarDiv nodes.  The divisor is
+// the cost of a float-float pair in proxy evaluations as it was when both were evaluated one-sided (about two); with
+// near pairs shared a float-float interaction costs 1.1 evaluations (1.47e11 interactions against 1.67e11 evaluations
+// a second), an FP32 or FP64 one about one.  The divisor decides which clusters are approximated, hence the result.
 constexpr int kMinFarDiv[3] = {1, 2, 1};
 // Cost of one proxy evaluation relative to one one-sided pair of the arithmetic (item splitting only).
 constexpr double kFarCost[3] = {0.4, 0.45, 0.5};

@@ -22,7 +22,9 @@ enum {
     CTR_PROBE_FFMA2 = 1,    /* fma.rn.f32x2 (two FP32 lanes per instruction) */
     CTR_PROBE_EX2 = 2,      /* ex2.approx.ftz.f32 (SFU) */
     CTR_PROBE_RSQRT = 3,    /* rsqrt.approx.ftz.f32 (SFU) */
-    CTR_PROBE_DFMA = 4      /* fma.rn.f64 */
+    CTR_PROBE_DFMA = 4,     /* fma.rn.f64 */
+    CTR_PROBE_FFMA_3R = 5,  /* fma.rn.f32 whose three operands are registers of its own */
+    CTR_PROBE_FFMA2_3R = 6  /* fma.rn.f32x2 likewise */
 };
 
 /*

@@ -48,6 +48,49 @@ __global__ void ffma2_kernel(float* out, int64_t iters, float a, float b) {
     if (s == 1234.5f) out[threadIdx.x] = s;
 }
 
+// x = a b + x with a, b and x of every chain in registers of their own (above, a and b are shared by the chains)
+__global__ void ffma_3r_kernel(float* out, int64_t iters, float a0, float b0) {
+    float x[kChains], a[kChains], b[kChains];
+#pragma unroll
+    for (int c = 0; c < kChains; ++c) {
+        x[c] = threadIdx.x * 1e-3f + c;
+        a[c] = a0 + 1e-3f * c * threadIdx.x;
+        b[c] = b0 + 1e-6f * (c + 1) * threadIdx.x;
+    }
+    for (int64_t i = 0; i < iters; ++i) {
+#pragma unroll
+        for (int c = 0; c < kChains; ++c) asm volatile("fma.rn.f32 %0, %1, %2, %0;" : "+f"(x[c]) : "f"(a[c]), "f"(b[c]));
+    }
+    float s = 0.f;
+#pragma unroll
+    for (int c = 0; c < kChains; ++c) s += x[c];
+    if (s == 1234.5f) out[threadIdx.x] = s;
+}
+
+__global__ void ffma2_3r_kernel(float* out, int64_t iters, float a0, float b0) {
+    unsigned long long x[kChains], a[kChains], b[kChains];
+#pragma unroll
+    for (int c = 0; c < kChains; ++c) {
+        const float v = threadIdx.x * 1e-3f + c, p = a0 + 1e-3f * c * threadIdx.x, q = b0 + 1e-6f * (c + 1) * threadIdx.x;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(x[c]) : "f"(v), "f"(v + 0.5f));
+        asm("mov.b64 %0, {%1, %2};" : "=l"(a[c]) : "f"(p), "f"(p + 0.25f));
+        asm("mov.b64 %0, {%1, %2};" : "=l"(b[c]) : "f"(q), "f"(q + 1e-7f));
+    }
+    for (int64_t i = 0; i < iters; ++i) {
+#pragma unroll
+        for (int c = 0; c < kChains; ++c)
+            asm volatile("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(x[c]) : "l"(a[c]), "l"(b[c]));
+    }
+    float s = 0.f;
+#pragma unroll
+    for (int c = 0; c < kChains; ++c) {
+        float lo, hi;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x[c]));
+        s += lo + hi;
+    }
+    if (s == 1234.5f) out[threadIdx.x] = s;
+}
+
 __global__ void ex2_kernel(float* out, int64_t iters) {
     float x[kChains];
 #pragma unroll
@@ -93,7 +136,7 @@ __global__ void dfma_kernel(double* out, int64_t iters, double a, double b) {
 }  // namespace
 
 extern "C" int ctr_probe_rate(int kind, int64_t iters, double* ops_per_s, double* seconds) {
-    if (!ops_per_s || iters <= 0 || kind < CTR_PROBE_FFMA || kind > CTR_PROBE_DFMA) return -1;
+    if (!ops_per_s || iters <= 0 || kind < CTR_PROBE_FFMA || kind > CTR_PROBE_FFMA2_3R) return -1;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return -4;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -4;
@@ -107,10 +150,12 @@ extern "C" int ctr_probe_rate(int kind, int64_t iters, double* ops_per_s, double
             case CTR_PROBE_FFMA2: ffma2_kernel<<<blocks, kThreads>>>((float*)out, it, 0.9999f, 1e-4f); break;
             case CTR_PROBE_EX2: ex2_kernel<<<blocks, kThreads>>>((float*)out, it); break;
             case CTR_PROBE_RSQRT: rsqrt_kernel<<<blocks, kThreads>>>((float*)out, it); break;
+            case CTR_PROBE_FFMA_3R: ffma_3r_kernel<<<blocks, kThreads>>>((float*)out, it, 0.9999f, 1e-4f); break;
+            case CTR_PROBE_FFMA2_3R: ffma2_3r_kernel<<<blocks, kThreads>>>((float*)out, it, 0.9999f, 1e-4f); break;
             default: dfma_kernel<<<blocks, kThreads>>>((double*)out, it, 0.9999, 1e-4); break;
         }
     };
-    const double per_thread_iter = (kind == CTR_PROBE_FFMA2) ? 2.0 * kChains : (double)kChains;
+    const double per_thread_iter = (kind == CTR_PROBE_FFMA2 || kind == CTR_PROBE_FFMA2_3R) ? 2.0 * kChains : (double)kChains;
     float ms = 0.f;
     bool ok = cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess;
     if (ok) {

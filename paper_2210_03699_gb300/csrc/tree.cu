@@ -25,7 +25,7 @@ namespace {
 constexpr int kTreeItemsPerSlot = 4;
 // A well-separated cluster is approximated when it has more than (degree+1)^3 / kMinFarDiv nodes.  The divisor is
 // the cost of a float-float pair in proxy evaluations as it was when both were evaluated one-sided (about two); with
-// near pairs shared a float-float interaction costs 1.1 evaluations (1.47e11 interactions against 1.67e11 evaluations
+// near pairs shared a float-float interaction costs 1.1 evaluations (1.47e11 interactions against 1.65e11 evaluations
 // a second), an FP32 or FP64 one about one.  The divisor decides which clusters are approximated, hence the result.
 constexpr int kMinFarDiv[3] = {1, 2, 1};
 // Cost of one proxy evaluation relative to one one-sided pair of the arithmetic (item splitting only).
